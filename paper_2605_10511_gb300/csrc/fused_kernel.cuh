@@ -24,6 +24,11 @@
 namespace dpf {
 namespace {
 
+// The CTA's dynamic shared memory: accumulators, join tables, the warps'
+// survivor lists (and staging rings).
+extern __shared__ __align__(16) uint8_t dyn[];
+__device__ __forceinline__ uint32_t* shared_acc() { return reinterpret_cast<uint32_t*>(dyn); }
+
 struct alignas(16) CtaState {
   DevQuery q;
   int wq[32];          // query of the ticket each warp holds (INT_MAX: none left)
@@ -49,6 +54,14 @@ __device__ __forceinline__ uint32_t block_rank(bool flag, CtaState& cs, uint32_t
   return before + __popc(b & ((1u << lane) - 1u));
 }
 
+// Aggregate a of group g (count rows): a COUNT is the group's row count and
+// has no accumulator of its own.
+__device__ __forceinline__ long long agg_value(const DevQuery& Q, uint32_t g, int a, long long count) {
+  if (a >= int(Q.naggs)) return 0;
+  if (Q.agg_op[a] == DPF_AGG_COUNT) return count;
+  return (long long)__ldcg(Q.acc + uint64_t(g) * (1 + Q.naggs) + 1 + a);
+}
+
 // Converts a query's global accumulators into records and clears them.
 __device__ void assemble(const DevQuery& Q, CtaState& cs) {
   const uint32_t S1 = 1 + Q.naggs;
@@ -58,7 +71,7 @@ __device__ void assemble(const DevQuery& Q, CtaState& cs) {
       dpf_record r;
       r.key[0] = r.key[1] = 0;
       r.count = (long long)__ldcg(Q.acc);
-      for (int a = 0; a < 4; ++a) r.val[a] = a < int(Q.naggs) ? (long long)__ldcg(Q.acc + 1 + a) : 0;
+      for (int a = 0; a < 4; ++a) r.val[a] = agg_value(Q, 0, a, r.count);
       out[0] = r;
       *Q.out_n = 1;
     }
@@ -80,8 +93,7 @@ __device__ void assemble(const DevQuery& Q, CtaState& cs) {
           }
         }
         r.count = (long long)cnt;
-        for (int a = 0; a < 4; ++a)
-          r.val[a] = a < int(Q.naggs) ? (long long)__ldcg(Q.acc + uint64_t(g) * S1 + 1 + a) : 0;
+        for (int a = 0; a < 4; ++a) r.val[a] = agg_value(Q, g, a, r.count);
         out[base + rank] = r;
       }
       base += total;
@@ -96,15 +108,19 @@ __device__ void assemble(const DevQuery& Q, CtaState& cs) {
 }
 
 // Adds the CTA's accumulators for Q to global memory, counts the chunks it
-// processed and, if they were the query's last, assembles the result.
-__device__ void finish_query(const DevQuery& Q, unsigned long long* sacc, uint32_t mine,
-                             CtaState& cs) {
+// processed and, if they were the query's last, assembles the result.  Each
+// CTA starts at its own group, so that the CTAs leaving a query together add
+// to different addresses.
+__device__ void finish_query(const DevQuery& Q, uint32_t mine, CtaState& cs) {
+  const uint32_t* sacc = shared_acc();
   const uint32_t S1 = 1 + Q.naggs;
   if (Q.use_smem_acc) {
-    const uint32_t n = Q.domain * S1;
+    const uint32_t n = Q.domain * S1, rot = uint32_t((uint64_t(blockIdx.x) * n) / gridDim.x);
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-      const unsigned long long x = sacc[i];
-      if (x) atomicAdd(Q.acc + i, x);
+      const uint32_t j = i + rot < n ? i + rot : i + rot - n, g = j / S1;  // global accumulators: [group][slot]
+      const uint32_t at = (j - g * S1) * Q.domain + g;
+      const unsigned long long x = sacc[at] | ((unsigned long long)sacc[n + at] << 32);
+      if (x) atomicAdd(Q.acc + j, x);
     }
   }
   __threadfence();
@@ -121,6 +137,27 @@ __device__ void finish_query(const DevQuery& Q, unsigned long long* sacc, uint32
   __syncthreads();
 }
 
+// The accumulators a warp adds to: the CTA's shared ones, or the query's
+// global int64 ones when the domain does not fit.  A shared
+// int64 accumulator is kept as two 32-bit halves, all low halves first
+// (slot-major: slot * domain + group, so that neighbouring groups lie in
+// different banks), then all high halves.  32-bit shared atomics are done by
+// the memory pipe, also when lanes of one instruction hit the same address;
+// a 64-bit one is a compare-and-swap loop that repeats for each of them.  An
+// add needs the high half only when it carries (or the value itself has high
+// bits), so most adds are one 32-bit atomic; the sum is exact modulo 2^64.
+__device__ __forceinline__ void acc_add(const DevQuery& Q, uint32_t gid, uint32_t slot, unsigned long long x) {
+  if (!Q.use_smem_acc) {
+    atomicAdd(Q.acc + uint64_t(gid) * (1 + Q.naggs) + slot, x);
+    return;
+  }
+  uint32_t* p = shared_acc() + slot * Q.domain + gid;
+  const uint32_t lo = uint32_t(x);
+  const uint32_t old = atomicAdd(p, lo);
+  const uint32_t hi = uint32_t(x >> 32) + uint32_t(old + lo < lo);
+  if (hi) atomicAdd(p + Q.domain * (1 + Q.naggs), hi);
+}
+
 // Warp-aggregated group-by update (hash aggregation of Kernel #3, Sec. 3.1),
 // by the round's leading group: the lanes holding the group id of the
 // round's first valid lane combine their values with warp reductions and
@@ -132,8 +169,8 @@ __device__ void finish_query(const DevQuery& Q, unsigned long long* sacc, uint32
 // the 64-bit value; otherwise the value is an int32, whose low 16 bits and
 // signed high 16 bits are summed).  Warp-uniform call.
 template <bool kWide>
-__device__ __forceinline__ void lead_group_add(unsigned long long* acc, uint32_t gid, uint32_t S1, uint32_t slot,
-                                               unsigned long long x, bool valid, int lane) {
+__device__ __forceinline__ void lead_group_add(const DevQuery& Q, uint32_t gid, uint32_t slot, unsigned long long x,
+                                               bool valid, int lane) {
   const uint32_t vm = __ballot_sync(kFull, valid);
   if (vm == 0) return;
   const int lead = __ffs(vm) - 1;
@@ -154,19 +191,19 @@ __device__ __forceinline__ void lead_group_add(unsigned long long* acc, uint32_t
       const int32_t s_hi = int32_t(__reduce_add_sync(m, uint32_t(v >> 16)));  // |sum| < 2^20
       t = (unsigned long long)((long long)s_lo + (long long)s_hi * 65536ll);
     }
-    if (lane == lead) atomicAdd(acc + uint64_t(g0) * S1 + slot, t);
+    if (lane == lead) acc_add(Q, g0, slot, t);
   } else if (valid) {
-    atomicAdd(acc + uint64_t(gid) * S1 + slot, x);
+    acc_add(Q, gid, slot, x);
   }
 }
 
 // A grouped update: warp-aggregated by the leading group (Q.warp_agg) or one
 // atomic per row.
 template <bool kWide>
-__device__ __forceinline__ void group_add(const DevQuery& Q, unsigned long long* acc, uint32_t gid, uint32_t S1,
-                                          uint32_t slot, unsigned long long x, bool valid, int lane) {
-  if (Q.warp_agg) lead_group_add<kWide>(acc, gid, S1, slot, x, valid, lane);
-  else if (valid) atomicAdd(acc + uint64_t(gid) * S1 + slot, x);
+__device__ __forceinline__ void group_add(const DevQuery& Q, uint32_t gid, uint32_t slot,
+                                          unsigned long long x, bool valid, int lane) {
+  if (Q.warp_agg) lead_group_add<kWide>(Q, gid, slot, x, valid, lane);
+  else if (valid) acc_add(Q, gid, slot, x);
 }
 
 // One aggregate over a warp's list, specialised on its operation (dpf_agg_op)
@@ -174,10 +211,9 @@ __device__ __forceinline__ void group_add(const DevQuery& Q, unsigned long long*
 // per row; otherwise any codec through row_value (DELTA decodes densely).
 template <bool kHost, int kOp, bool kPoint>
 __device__ __forceinline__ void agg_pass(const DevQuery& Q, const PageState& P, uint32_t seg_mb,
-                                         const uint32_t* list, uint32_t n, int lane, unsigned long long* acc,
+                                         const uint32_t* list, uint32_t n, int lane,
                                          uint32_t slot, int ca, int cb, bool single, unsigned int* status) {
   constexpr int U = kPoint ? kListUnroll : 1;  // rounds whose loads are issued together
-  const uint32_t S1 = 1 + Q.naggs;
   long long sum = 0;
   for (uint32_t i0 = 0; i0 < n; i0 += 32 * U) {
     uint32_t r[U], gid[U];
@@ -194,30 +230,28 @@ __device__ __forceinline__ void agg_pass(const DevQuery& Q, const PageState& P, 
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       va[u] = vb[u] = 0;
-      if (kOp != DPF_AGG_COUNT)
-        va[u] = int32_t(kPoint ? point_value<kHost>(Q, ca, P, seg_mb, r[u], valid[u])
-                               : row_value<kHost>(Q, ca, P, seg_mb, r[u], valid[u], lane, status));
+      va[u] = int32_t(kPoint ? point_value<kHost>(Q, ca, P, seg_mb, r[u], valid[u])
+                             : row_value<kHost>(Q, ca, P, seg_mb, r[u], valid[u], lane, status));
       if (kOp == DPF_AGG_SUM_MUL || kOp == DPF_AGG_SUM_SUB)
         vb[u] = int32_t(kPoint ? point_value<kHost>(Q, cb, P, seg_mb, r[u], valid[u])
                                : row_value<kHost>(Q, cb, P, seg_mb, r[u], valid[u], lane, status));
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      long long x = 1;
-      if (kOp == DPF_AGG_SUM) x = va[u];
-      else if (kOp == DPF_AGG_SUM_MUL)
+      long long x = va[u];
+      if (kOp == DPF_AGG_SUM_MUL)
         x = (long long)((unsigned long long)(long long)va[u] * (unsigned long long)(long long)vb[u]);
       else if (kOp == DPF_AGG_SUM_SUB)
         x = (long long)va[u] - (long long)vb[u];
       if (single) sum += valid[u] ? x : 0;
-      else group_add<kOp == DPF_AGG_SUM_MUL || kOp == DPF_AGG_SUM_SUB>(Q, acc, gid[u], S1, slot,
+      else group_add<kOp == DPF_AGG_SUM_MUL || kOp == DPF_AGG_SUM_SUB>(Q, gid[u], slot,
                                                                       (unsigned long long)x, valid[u], lane);
     }
   }
   if (single) {
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) sum += __shfl_down_sync(kFull, sum, d);
-    if (lane == 0 && sum != 0) atomicAdd(acc + slot, (unsigned long long)sum);
+    if (lane == 0 && sum != 0) acc_add(Q, 0, slot, (unsigned long long)sum);
   }
 }
 
@@ -227,9 +261,8 @@ __device__ __forceinline__ void agg_pass(const DevQuery& Q, const PageState& P, 
 // allocation as it was.
 template <bool kHost, int kOp>
 __device__ __forceinline__ void agg_pass_wide(const DevQuery& Q, const PageState& P, uint32_t seg_mb,
-                                           const uint32_t* list, uint32_t n, int lane, unsigned long long* acc,
+                                           const uint32_t* list, uint32_t n, int lane,
                                            uint32_t slot, int ca, int cb, bool single, unsigned int* status) {
-  const uint32_t S1 = 1 + Q.naggs;
   unsigned long long sum = 0;
   for (uint32_t i0 = 0; i0 < n; i0 += 32) {
     bool valid = i0 + lane < n;
@@ -242,30 +275,31 @@ __device__ __forceinline__ void agg_pass_wide(const DevQuery& Q, const PageState
       b = (unsigned long long)value64<kHost>(Q, cb, P, seg_mb, r, valid, lane, status);
     const unsigned long long x = kOp == DPF_AGG_SUM ? a : (kOp == DPF_AGG_SUM_MUL ? a * b : a - b);
     if (single) sum += valid ? x : 0ull;
-    else group_add<true>(Q, acc, gid, S1, slot, x, valid, lane);
+    else group_add<true>(Q, gid, slot, x, valid, lane);
   }
   if (single) {
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) sum += __shfl_down_sync(kFull, sum, d);
-    if (lane == 0 && sum != 0) atomicAdd(acc + slot, sum);
+    if (lane == 0 && sum != 0) acc_add(Q, 0, slot, sum);
   }
 }
 
 template <bool kHost, int kOp>
 __device__ __forceinline__ void agg_dispatch(const DevQuery& Q, const PageState& P, uint32_t seg_mb,
-                                             const uint32_t* list, uint32_t n, int lane, unsigned long long* acc,
+                                             const uint32_t* list, uint32_t n, int lane,
                                              uint32_t slot, int ca, int cb, bool single, unsigned int* status) {
   if (Q.cols[ca].codec == C_FOR64 || (kOp != DPF_AGG_SUM && Q.cols[cb].codec == C_FOR64)) {
-    agg_pass_wide<kHost, kOp>(Q, P, seg_mb, list, n, lane, acc, slot, ca, cb, single, status);
+    agg_pass_wide<kHost, kOp>(Q, P, seg_mb, list, n, lane, slot, ca, cb, single, status);
     return;
   }
   const bool point = Q.cols[ca].codec != C_DELTA && (kOp == DPF_AGG_SUM || Q.cols[cb].codec != C_DELTA);
-  if (point) agg_pass<kHost, kOp, true>(Q, P, seg_mb, list, n, lane, acc, slot, ca, cb, single, status);
-  else agg_pass<kHost, kOp, false>(Q, P, seg_mb, list, n, lane, acc, slot, ca, cb, single, status);
+  if (point) agg_pass<kHost, kOp, true>(Q, P, seg_mb, list, n, lane, slot, ca, cb, single, status);
+  else agg_pass<kHost, kOp, false>(Q, P, seg_mb, list, n, lane, slot, ca, cb, single, status);
 }
 
 // Aggregation over a warp's survivor list (Kernel #3 hash aggregation;
-// int64 as in Sec. 4.3): slot 0 counts rows, slot 1 + a holds aggregate a.
+// int64 as in Sec. 4.3): slot 0 counts rows, slot 1 + a holds aggregate a
+// (unused when that is a COUNT).
 // domain == 1: per-lane int64 sums reduced across the warp; otherwise
 // int64 atomics (one per row, or warp-aggregated by the round's leading
 // group: group_add) into the CTA's shared accumulators (or the query's
@@ -273,12 +307,13 @@ __device__ __forceinline__ void agg_dispatch(const DevQuery& Q, const PageState&
 template <bool kHost>
 __device__ __forceinline__ void list_aggregate(const DevQuery& Q, const PageState& P, uint32_t seg_mb,
                                                const uint32_t* list, uint32_t n, int lane,
-                                               unsigned long long* acc, unsigned int* status) {
-  const uint32_t S1 = 1 + Q.naggs;
+                                               unsigned int* status) {
   const bool single = Q.domain == 1;
   if (single) {
-    if (lane == 0) atomicAdd(acc, (unsigned long long)n);
+    if (lane == 0) acc_add(Q, 0, 0, (unsigned long long)n);
   } else {
+    // a shared count needs no high half while the table has fewer than 2^32 rows
+    const bool narrow = Q.use_smem_acc && (Q.nrows >> 32) == 0 && !Q.warp_agg;
     for (uint32_t i0 = 0; i0 < n; i0 += 32) {
       bool valid = i0 + lane < n;
       const uint32_t gid = valid ? list[i0 + lane] >> kRowBits : 0u;
@@ -286,27 +321,22 @@ __device__ __forceinline__ void list_aggregate(const DevQuery& Q, const PageStat
         atomicOr(status, S_CORRUPT);  // a corrupt dictionary code
         valid = false;
       }
-      group_add<false>(Q, acc, gid, S1, 0, 1ull, valid, lane);
+      if (!narrow) group_add<false>(Q, gid, 0, 1ull, valid, lane);
+      else if (valid) atomicAdd(shared_acc() + gid, 1u);
     }
   }
   for (uint32_t a = 0; a < Q.naggs; ++a) {
     const int ca = Q.agg_a[a], cb = Q.agg_b[a];
     switch (Q.agg_op[a]) {
-      case DPF_AGG_COUNT:
-        if (single) {
-          if (lane == 0) atomicAdd(acc + 1 + a, (unsigned long long)n);
-        } else {
-          agg_pass<kHost, DPF_AGG_COUNT, true>(Q, P, seg_mb, list, n, lane, acc, 1 + a, ca, cb, single, status);
-        }
-        break;
+      case DPF_AGG_COUNT: break;  // the row count (slot 0)
       case DPF_AGG_SUM:
-        agg_dispatch<kHost, DPF_AGG_SUM>(Q, P, seg_mb, list, n, lane, acc, 1 + a, ca, cb, single, status);
+        agg_dispatch<kHost, DPF_AGG_SUM>(Q, P, seg_mb, list, n, lane, 1 + a, ca, cb, single, status);
         break;
       case DPF_AGG_SUM_MUL:
-        agg_dispatch<kHost, DPF_AGG_SUM_MUL>(Q, P, seg_mb, list, n, lane, acc, 1 + a, ca, cb, single, status);
+        agg_dispatch<kHost, DPF_AGG_SUM_MUL>(Q, P, seg_mb, list, n, lane, 1 + a, ca, cb, single, status);
         break;
       default:
-        agg_dispatch<kHost, DPF_AGG_SUM_SUB>(Q, P, seg_mb, list, n, lane, acc, 1 + a, ca, cb, single, status);
+        agg_dispatch<kHost, DPF_AGG_SUM_SUB>(Q, P, seg_mb, list, n, lane, 1 + a, ca, cb, single, status);
         break;
     }
   }
@@ -352,7 +382,7 @@ __device__ __forceinline__ FirstCol first_col(const DevQuery& Q, const PageState
 // segment of at most 2^kRowBits rows of one page) before the later steps and
 // the aggregation run on them.
 template <bool kHost, bool kText, bool kStage>
-__device__ void process_ticket(const DevQuery& Q, uint64_t chunk, unsigned long long* acc, const uint8_t* stab,
+__device__ void process_ticket(const DevQuery& Q, uint64_t chunk, const uint8_t* stab,
                                uint32_t* list, int lane, unsigned int* status,
                                uint8_t* ring) {
   const uint64_t PR = Q.page_rows;
@@ -424,7 +454,7 @@ __device__ void process_ticket(const DevQuery& Q, uint64_t chunk, unsigned long 
       const uint32_t next = i0 + TB;
       if (j + 1 == ntiles || n + kTileRows > kListCap || next + TB - seg_mb > kSegMbs) {
         n = list_steps<kHost, kText>(Q, P, seg_mb, list, n, stab, lane, status, 1);
-        if (n) list_aggregate<kHost>(Q, P, seg_mb, list, n, lane, acc, status);
+        if (n) list_aggregate<kHost>(Q, P, seg_mb, list, n, lane, status);
         n = 0;
         seg_mb = next;
       }
@@ -473,9 +503,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
                                                        const uint64_t* __restrict__ qbegin, int nq,
                                                        uint64_t total, Sched* sched, uint32_t acc_slots,
                                                      uint32_t tables_bytes, uint32_t stage_bw) {
-  extern __shared__ __align__(16) uint8_t dyn[];
   __shared__ CtaState cs;
-  unsigned long long* sacc = reinterpret_cast<unsigned long long*>(dyn);
+  uint32_t* sacc = shared_acc();
   uint8_t* stab = dyn + ((acc_slots * sizeof(unsigned long long) + 15) & ~size_t(15));
   uint32_t* lists = reinterpret_cast<uint32_t*>(stab + tables_bytes);
   // Warps draw tickets on their own (one ticket = chunk_rows rows of one
@@ -507,7 +536,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
     __syncthreads();
     int next = INT_MAX;
     for (int w = 0; w < nw; ++w) next = min(next, cs.wq[w]);
-    if (cur >= 0) finish_query(cs.q, sacc, cs.mine, cs);
+    if (cur >= 0) finish_query(cs.q, cs.mine, cs);
     if (next == INT_MAX) break;
     {  // bring the query's plan into shared memory
       const uint4* src = reinterpret_cast<const uint4*>(queries + next);
@@ -518,16 +547,15 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
     __syncthreads();
     const DevQuery& Q = cs.q;
     if (Q.use_smem_acc) {
-      const uint32_t n = Q.domain * (1 + Q.naggs);
-      for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) sacc[i] = 0ull;
+      const uint32_t n = 2 * Q.domain * (1 + Q.naggs);
+      for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) sacc[i] = 0u;
     }
     load_smem_tables(Q, stab);
     __syncthreads();
     cur = next;
-    unsigned long long* acc = Q.use_smem_acc ? sacc : Q.acc;
     uint32_t done_here = 0;
     while (hq == cur) {
-      process_ticket<kHost, kText, kStage>(Q, held - Q.chunk_begin, acc, stab, list, lane, &sched->status,
+      process_ticket<kHost, kText, kStage>(Q, held - Q.chunk_begin, stab, list, lane, &sched->status,
                                            ring);
       ++done_here;
       hq = draw(held);
