@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(256) build_kernel(const DevQuery* __restrict__
     TileState T;
     tile_init(P, i0, nmb, lane, T);
     tile_dense_step<kHost>(Q, 0, P, H, T, nullptr, lane, status);
-    uint32_t n = tile_compact(T, list, 0, 0, lane);
+    uint32_t n = tile_compact<kHost>(T, list, 0, 0, lane);
     n = list_steps<kHost>(Q, P, i0, list, n, nullptr, lane, status);
     // rank builds: one staging slot per kept row of the tile, reserved at once
     unsigned long long sbase = 0;

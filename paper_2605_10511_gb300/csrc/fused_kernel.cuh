@@ -353,7 +353,7 @@ __device__ __forceinline__ uint32_t tile_first_step(const DevQuery& Q, const Pag
   TileState T;
   tile_init<kGid>(P, i0, nmb, lane, T);
   tile_dense_step<kHost, kText, kGid, kStaged>(Q, 0, P, H, T, stab, lane, status, sp);
-  return tile_compact<kGid>(T, list, n, row_base, lane);
+  return tile_compact<kHost, kGid>(T, list, n, row_base, lane);
 }
 
 // The first step's column of Q in page P: its page address and packed words.

@@ -973,11 +973,17 @@ __device__ __forceinline__ bool step_adds_gid(const DevStep& S) {
 
 // Appends the tile's live rows to the warp's list after its first n0
 // entries; row_base = the tile's first row within the list's segment.
-// Returns the list length.  Each lane counts its live rows, a warp exclusive
-// scan of the counts gives the lane's first slot, and the lane writes its
-// rows there in (t, k) order (the list's order is free: later steps and the
-// aggregation visit every entry once, whatever its position).
-template <bool kGid = true>
+// Returns the list length.  The list's order is free: later steps and the
+// aggregation visit every entry once, whatever its position.
+//  - Few rows: a warp scan of the lanes' counts gives each lane its first
+//    slot, and it writes its rows there one after the other.
+//  - From kOrderedRows rows on (and always when the pages come over the host
+//    link, where a sector read twice costs most): in row order, one ballot per
+//    32 rows.  A later round's 32 entries are then neighbours, whose packed
+//    fields share sectors, and the writes fall into distinct banks.
+//  - A tile that lost no row is copied without ballots.
+constexpr uint32_t kOrderedRows = kMB * TB / 4;
+template <bool kHost, bool kGid = true>
 __device__ __forceinline__ uint32_t tile_compact(const TileState& T, uint32_t* list, uint32_t n0, uint32_t row_base,
                                                  int lane) {
   const uint32_t cnt = __popc(T.alive);
@@ -988,15 +994,38 @@ __device__ __forceinline__ uint32_t tile_compact(const TileState& T, uint32_t* l
     if (lane >= d) incl += y;
   }
   const uint32_t total = __shfl_sync(kFull, incl, 31);
-  uint32_t pos = n0 + incl - cnt;
+  if (total == kTileRows) {
 #pragma unroll
-  for (int t = 0; t < TB; ++t)
+    for (int t = 0; t < TB; ++t)
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if ((T.alive >> (4 * t + k)) & 1u) {
-        list[pos] = (row_base + uint32_t(t * kMB + k * 32 + lane)) | (kGid ? T.gid[t][k] << kRowBits : 0u);
-        ++pos;
+      for (int k = 0; k < 4; ++k)
+        list[n0 + uint32_t(t * kMB + k * 32 + lane)] =
+            (row_base + uint32_t(t * kMB + k * 32 + lane)) | (kGid ? T.gid[t][k] << kRowBits : 0u);
+  } else if (kHost || total >= kOrderedRows) {
+    const uint32_t lt = (1u << lane) - 1u;
+    uint32_t n = n0;
+#pragma unroll
+    for (int t = 0; t < TB; ++t)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const bool live = (T.alive >> (4 * t + k)) & 1u;
+        const uint32_t m = __ballot_sync(kFull, live);
+        if (live)
+          list[n + __popc(m & lt)] =
+              (row_base + uint32_t(t * kMB + k * 32 + lane)) | (kGid ? T.gid[t][k] << kRowBits : 0u);
+        n += __popc(m);
       }
+  } else {
+    uint32_t pos = n0 + incl - cnt;
+#pragma unroll
+    for (int t = 0; t < TB; ++t)
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if ((T.alive >> (4 * t + k)) & 1u) {
+          list[pos] = (row_base + uint32_t(t * kMB + k * 32 + lane)) | (kGid ? T.gid[t][k] << kRowBits : 0u);
+          ++pos;
+        }
+  }
   __syncwarp();
   return n0 + total;
 }
