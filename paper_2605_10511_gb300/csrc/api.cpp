@@ -502,6 +502,18 @@ dpf_status compile_pred_body(const Column& c, const dpf_pred& p, DevStep& S, int
     S.kind = op == DPF_OP_PREFIX ? ST_PREFIX : op == DPF_OP_CONTAINS ? ST_CONTAINS : ST_LIKE;
     S.plen = uint8_t(plen);
     std::memcpy(S.pfx, pat, size_t(plen));
+    if (S.kind == ST_LIKE) {
+      // the longest run of literal bytes: a row without it cannot match
+      for (int32_t i = 0; i < plen;) {
+        int32_t j = i;
+        while (j < plen && pat[j] != '%' && pat[j] != '_') ++j;
+        if (j - i > S.in[1]) {
+          S.in[0] = i;
+          S.in[1] = j - i;
+        }
+        i = j + 1;
+      }
+    }
     if (S.kind == ST_CONTAINS) {
       // a pattern of <= 8 bytes packed for the sliding-window compare: byte k
       // of the pattern at bits 8 * (plen - 1 - k) (the newest byte lowest)
@@ -1327,11 +1339,11 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   int min_blocks = kFusedMinBlocksLo;
   int per_sm = 0;
   if (t.ctas_per_sm >= uint32_t(kFusedMinBlocksHi)) {
-    per_sm = fused_blocks_per_sm(int(t.threads), acc_slots, max_tables, host, kFusedMinBlocksHi, stage_bw);
+    per_sm = fused_blocks_per_sm(int(t.threads), acc_slots, max_tables, host, kFusedMinBlocksHi, stage_bw, text);
     if (per_sm >= kFusedMinBlocksHi * 256 / int(t.threads)) min_blocks = kFusedMinBlocksHi;
   }
   if (min_blocks == kFusedMinBlocksLo)
-    per_sm = fused_blocks_per_sm(int(t.threads), acc_slots, max_tables, host, kFusedMinBlocksLo, stage_bw);
+    per_sm = fused_blocks_per_sm(int(t.threads), acc_slots, max_tables, host, kFusedMinBlocksLo, stage_bw, text);
   if (per_sm < 1) {
     release_prep(c, p.get());
     return fail(DPF_EINVAL, "fused kernel does not fit on an SM with %u threads and %zu table bytes", t.threads, max_tables);
@@ -1399,8 +1411,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   p->L.stage_bw = stage_bw;
   p->tuning.staging = stage_bw ? DPF_STAGE_ON : DPF_STAGE_OFF;  // what the launch does
   p->tuning.group_agg = any_warp_agg ? DPF_GROUP_AGG_WARP : DPF_GROUP_AGG_ATOMIC;
-  p->L.text = false;
-  for (const DevQuery& q : p->hq) p->L.text = p->L.text || needs_string_matcher(q);
+  p->L.text = text;
   p->fetched.assign(size_t(n), 0);
   p->id = c->next_prep++;
   *out = p.get();
@@ -1594,7 +1605,7 @@ dpf_status dpf_load_encoded(dpf_ctx* c, const dpf_column_desc* d, const uint8_t*
     col.raw_bytes = (codec == C_FOR64 ? 8 : 4) * nrows;
   }
   if (col.placement == DPF_PLACE_HOST_PINNED) {
-    cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&col.host_blob), size, cudaHostAllocMapped | cudaHostAllocPortable);
+    cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&col.host_blob), (size + 255) & ~uint64_t(255), cudaHostAllocMapped | cudaHostAllocPortable);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return fail(DPF_ENOMEM, "cudaHostAlloc(%llu): %s", (unsigned long long)size, cudaGetErrorString(e));
@@ -2324,7 +2335,7 @@ dpf_status dpf_capture_graph(dpf_ctx* c, dpf_prep_id id, void* stream) {
   if (p->graph) { cudaGraphDestroy(p->graph); p->graph = nullptr; }
   // set the smem attribute before capture (not a stream operation)
   fused_blocks_per_sm(p->L.threads, p->L.acc_slots, p->L.smem_tables, p->L.host_data, p->L.min_blocks,
-                      p->L.stage_bw);
+                      p->L.stage_bw, p->L.text);
   CUDA_TRY(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = launch_prep(p, s);
   cudaGraph_t graph = nullptr;

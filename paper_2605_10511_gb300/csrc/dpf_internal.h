@@ -104,7 +104,8 @@ struct DevStep {
   uint8_t kind, col, nin, plen;
   int32_t lo, hi;
   int32_t in[kMaxIn];     // IN operands; ST_CONTAINS: in[0..1] = a pattern of <= 8 bytes
-                          // packed for the sliding-window compare
+                          // packed for the sliding-window compare; ST_LIKE: in[0..1] =
+                          // start and length of the pattern's longest literal run
   // ST_PROBE
   const void* ht;         // OPEN: uint2 slots; DIRECT: uint32 entries; RANK: directory + payloads (global)
   uint32_t ht_mask;       // OPEN: capacity - 1 (power of two)

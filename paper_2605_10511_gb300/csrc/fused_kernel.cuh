@@ -349,10 +349,11 @@ template <bool kHost, bool kText, bool kGid, bool kStaged = false>
 __device__ __forceinline__ uint32_t tile_first_step(const DevQuery& Q, const PageState& P, const TileHdr& H,
                                                     uint32_t i0, uint32_t nmb, uint32_t row_base, const uint8_t* stab,
                                                     uint32_t* list, uint32_t n, int lane, unsigned int* status,
-                                                    StagedPay sp = StagedPay{nullptr, 0, 0}) {
+                                                    StagedPay sp = StagedPay{nullptr, 0, 0},
+                                                    uint32_t* search = nullptr) {
   TileState T;
   tile_init<kGid>(P, i0, nmb, lane, T);
-  tile_dense_step<kHost, kText, kGid, kStaged>(Q, 0, P, H, T, stab, lane, status, sp);
+  tile_dense_step<kHost, kText, kGid, kStaged>(Q, 0, P, H, T, stab, lane, status, sp, search);
   return tile_compact<kHost, kGid>(T, list, n, row_base, lane);
 }
 
@@ -448,8 +449,11 @@ __device__ void process_ticket(const DevQuery& Q, uint64_t chunk, const uint8_t*
       } else {
         const TileHdr H = load_headers<kHost>(Q, P, i0, nmb, lane);
         if (!kHost && Q.pf_step) prefetch_words(Q, P, H, Q.steps[1].col, nmb, lane);
-        if (gid0) n = tile_first_step<kHost, kText, true>(Q, P, H, i0, nmb, row_base, stab, list, n, lane, status);
-        else n = tile_first_step<kHost, kText, false>(Q, P, H, i0, nmb, row_base, stab, list, n, lane, status);
+        // without a staging ring its place holds the string search's scratch
+        uint32_t* search = kText ? reinterpret_cast<uint32_t*>(ring) : nullptr;
+        const StagedPay none{nullptr, 0, 0};
+        if (gid0) n = tile_first_step<kHost, kText, true>(Q, P, H, i0, nmb, row_base, stab, list, n, lane, status, none, search);
+        else n = tile_first_step<kHost, kText, false>(Q, P, H, i0, nmb, row_base, stab, list, n, lane, status, none, search);
       }
       const uint32_t next = i0 + TB;
       if (j + 1 == ntiles || n + kTileRows > kListCap || next + TB - seg_mb > kSegMbs) {
@@ -515,7 +519,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
   // finished query's accumulators first.
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   uint32_t* list = lists + uint32_t(warp) * kListCap;
-  uint8_t* ring = reinterpret_cast<uint8_t*>(lists + nw * kListCap) + size_t(warp) * stage_warp_bytes(stage_bw);
+  uint8_t* ring = reinterpret_cast<uint8_t*>(lists + nw * kListCap) +
+                  size_t(warp) * (kText ? kSearchWords * sizeof(uint32_t) : stage_warp_bytes(stage_bw));
   auto draw = [&](unsigned long long& t) -> int {
     unsigned long long x = 0;
     if (lane == 0) x = atomicAdd(&sched->next, 1ull);

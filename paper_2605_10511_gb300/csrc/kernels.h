@@ -21,6 +21,9 @@ constexpr int kFusedMinBlocksHi = 4;
 constexpr uint32_t kDefaultChunkRows = 4096;
 // Shared memory of one warp's survivor list (1,024 entries).
 constexpr uint32_t kListBytesPerWarp = 1024 * 4;
+// Words of one warp's scratch of the cooperative string search (search_mb),
+// in launches that have a string-matcher step.
+constexpr uint32_t kSearchWords = 336;
 // Estimated selectivity of the first step from which step 1's mini blocks
 // are prefetched into L2 during the dense tiles (DevQuery::pf_step).
 constexpr double kPrefetchMinSel = 0.03;
@@ -64,8 +67,8 @@ cudaError_t launch_fused(const FusedLaunch& L, cudaStream_t s);
 // Occupancy of the fused kernel for (threads, dynamic smem); also sets the
 // kernel's dynamic shared-memory limit.
 int fused_blocks_per_sm(int threads, uint32_t acc_slots, size_t smem_tables, bool host_data, int min_blocks,
-                        uint32_t stage_bw = 0);
-size_t fused_dynamic_smem(uint32_t acc_slots, size_t smem_tables, int threads, uint32_t stage_bw = 0);
+                        uint32_t stage_bw, bool text);
+size_t fused_dynamic_smem(uint32_t acc_slots, size_t smem_tables, int threads, uint32_t stage_bw, bool text);
 
 // Hash build (Kernel #1 of Sec. 3.1).  `q` describes the dimension scan:
 // cols/steps as for the fused kernel, build_key/build_pay name columns.

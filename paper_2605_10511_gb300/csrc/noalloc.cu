@@ -144,7 +144,7 @@ extern "C" dpf_status dpf_execute_noalloc(dpf_ctx* ctx, const dpf_plan* plan, vo
   L.host_data = host;
   L.text = needs_string_matcher(Q);
   L.min_blocks = kFusedMinBlocksLo;
-  const int per_sm = fused_blocks_per_sm(L.threads, L.acc_slots, smem_tables, host, L.min_blocks);
+  const int per_sm = fused_blocks_per_sm(L.threads, L.acc_slots, smem_tables, host, L.min_blocks, 0, L.text);
   if (per_sm < 1) return fail(DPF_EINVAL, "dpf_execute_noalloc: fused kernel does not fit on an SM");
   L.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(uint64_t(num_sms) * per_sm, Q.nchunks)));
   e = launch_fused(L, s);

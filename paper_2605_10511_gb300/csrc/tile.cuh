@@ -489,16 +489,267 @@ __device__ __forceinline__ bool string_match(const DevStep& S, const uint8_t* s,
   return string_scan<kHost, ST_CONTAINS>(S, s, len, sym);
 }
 
+// ------------------------------------------------- cooperative search
+// CONTAINS (and the filter of a general LIKE) over a whole mini block: its
+// strings' bytes lie one after the other, so the warp reads them as
+// consecutive 16-byte chunks, a lane per chunk, and tests every position of
+// the pattern's occurrences at once, instead of each lane walking its own
+// string byte by byte (32 different cache lines a load, each load waiting on
+// the last, and a warp as slow as its longest string).  The positions found
+// are a bitmap in the warp's scratch; a row matches when a bit lies in its
+// own range.  Bytes are taken kSearchWin at a time, so strings of any length
+// fit the scratch.
+constexpr uint32_t kSearchWin = 4096;
+constexpr uint32_t kSearchAhead = 2 * kMaxPrefix;           // bytes an FSST match may run past its first code
+constexpr uint32_t kSearchHits = kSearchWin / 32;            // words of the hit bitmap
+constexpr uint32_t kSearchStarts = (kSearchWin + kSearchAhead) / 32;  // FSST: words of the row-start bitmap
+constexpr uint32_t kLikeQueue = 64;                          // LIKE: candidate rows {offset, length, row}, then
+constexpr uint32_t kLikeWords = 3 * kLikeQueue + kMB * TB / 32;  // one result bit per row of the tile
+static_assert(kSearchHits + kLikeWords == kSearchWords && kSearchStarts <= kLikeWords,
+              "the host's per-warp shared-memory figure");
+
+// Whether bitmap bits [lo, hi) hold a set bit.
+__device__ __forceinline__ bool any_bit(const uint32_t* bits, uint32_t lo, uint32_t hi) {
+  if (lo >= hi) return false;
+  const uint32_t last = (hi - 1) >> 5;
+  uint32_t w = lo >> 5, x = bits[w] & (0xffffffffu << (lo & 31u));
+  while (w < last) {
+    if (x) return true;
+    x = bits[++w];
+  }
+  return (x & (0xffffffffu >> (31u - ((hi - 1) & 31u)))) != 0;
+}
+
+// Occurrences of pat[0..plen), plen >= 1, starting in the 16 bytes at p (bit
+// o: at p[o]); avail = bytes of the mini block from p on.  The first four
+// bytes are compared at every offset; a longer pattern's rest byte by byte.
+template <bool kHost>
+__device__ __forceinline__ uint32_t find_raw(const uint8_t* p, uint64_t avail, const uint8_t* pat, uint32_t plen,
+                                             uint32_t pat4, uint32_t mask4) {
+  const uint4 v = ld_u4<kHost>(reinterpret_cast<const uint4*>(p));
+  const uint32_t w[5] = {v.x, v.y, v.z, v.w, avail > 16 ? ld_u32<kHost>(reinterpret_cast<const uint32_t*>(p + 16)) : 0u};
+  uint32_t m = 0;
+#pragma unroll
+  for (int o = 0; o < 16; ++o) {
+    const uint32_t x = __funnelshift_r(w[o >> 2], w[(o >> 2) + 1], 8 * (o & 3));
+    m |= uint32_t(((x ^ pat4) & mask4) == 0) << o;
+  }
+  if (plen > 4) {
+    uint32_t cand = m;
+    while (cand) {
+      const uint32_t o = uint32_t(__ffs(cand) - 1);
+      cand &= cand - 1;
+      bool ok = o + plen <= avail;
+      for (uint32_t i = 4; ok && i < plen; ++i) ok = ld_u8<kHost>(p + o + i) == pat[i];
+      if (!ok) m &= ~(1u << o);
+    }
+  }
+  return m;
+}
+
+// Bytes of a 16-byte chunk that are literals (the byte after an escape),
+// given esc = its bytes equal to the escape code and whether its first byte
+// is one; *out = whether the next chunk's first byte is.
+__device__ __forceinline__ uint32_t literals(uint32_t esc, bool first, bool* out) {
+  uint32_t lit = first ? 1u : 0u;
+  esc &= ~lit;
+  while (esc) {
+    const uint32_t b = esc & (0u - esc);
+    lit |= b << 1;
+    esc &= ~(b | (b << 1));
+  }
+  *out = (lit >> 16) & 1u;
+  return lit & 0xffffu;
+}
+
+// Code positions among the 16 bytes at p where a match of the pattern starts
+// (bit o), for a warp's 32 consecutive chunks; *carry = whether the first
+// chunk starts with a literal, then whether the next 32 do.  skip = leading
+// bytes of the chunk before the mini block, avail = its bytes from p on
+// (0: the lane has no chunk).  A match is found from the code its first byte
+// lies in: the matcher run from its empty state at every code whose table
+// entry leaves that state (a bit row of few codes), for at most plen codes (an
+// occurrence starting inside the first code ends within them), up to the
+// row's end (starts: a bit per row start, from this chunk's window on).
+template <bool kHost>
+__device__ __forceinline__ uint32_t find_fsst(const uint8_t* p, uint32_t at, uint32_t skip, uint64_t avail, bool* carry,
+                                              const uint8_t* tab, uint32_t plen, const uint32_t* starts, int lane) {
+  uint4 v = make_uint4(0, 0, 0, 0);
+  if (avail) v = ld_u4<kHost>(reinterpret_cast<const uint4*>(p));
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  uint32_t m = 0, seen = 0;
+#pragma unroll
+  for (int o = 0; o < 16; ++o) {
+    const uint32_t e = tab[(w[o >> 2] >> (8 * (o & 3))) & 0xffu];
+    seen |= e;
+    m |= uint32_t(e != 0) << o;
+  }
+  const uint32_t keep = avail == 0 ? 0u : (0xffffu << skip) & (avail >= 16 ? 0xffffu : (1u << uint32_t(avail)) - 1u);
+  m &= keep;
+  // kFsstDead (bit 6) is the escape code's entry; matcher states stay below 32
+  if (__any_sync(kFull, (seen & 0x40u) != 0) || *carry) {
+    uint32_t esc = 0;
+#pragma unroll
+    for (int o = 0; o < 16; ++o) esc |= uint32_t(((w[o >> 2] >> (8 * (o & 3))) & 0xffu) == kFsstEscape) << o;
+    esc &= keep;
+    bool o0, o1;
+    const uint32_t lit0 = literals(esc, false, &o0), lit1 = literals(esc, true, &o1);
+    // the chunk maps "starts with a literal" (0 / 1) to the next chunk's;
+    // a warp scan composes the maps
+    uint32_t f = uint32_t(o0) | (uint32_t(o1) << 1);
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t g = __shfl_up_sync(kFull, f, d);  // the map of the chunks before
+      if (lane >= d) f = ((f >> (g & 1u)) & 1u) | (((f >> ((g >> 1) & 1u)) & 1u) << 1);
+    }
+    const uint32_t before = __shfl_up_sync(kFull, f, 1);
+    const bool in = lane == 0 ? *carry : ((before >> uint32_t(*carry)) & 1u) != 0;
+    *carry = (__shfl_sync(kFull, f, 31) >> uint32_t(*carry)) & 1u;
+    m &= ~(in ? lit1 : lit0);
+  }
+  const uint8_t* btab = tab + (plen + 1) * 256;
+  uint32_t hits = 0;
+  while (m) {
+    const uint32_t o = uint32_t(__ffs(m) - 1);
+    m &= m - 1;
+    uint32_t q = 0;
+    uint64_t i = o;
+    for (uint32_t n = 0; n < plen; ++n) {
+      const uint32_t c = ld_u8<kHost>(p + i++);
+      const uint32_t e = c == kFsstEscape ? btab[q * 256 + ld_u8<kHost>(p + i++)] : tab[q * 256 + c];
+      if (e & kFsstHit) {
+        hits |= 1u << o;
+        break;
+      }
+      q = e;
+      if (q == 0 || i >= avail) break;
+      const uint32_t b = at + uint32_t(i);
+      if ((starts[b >> 5] >> (b & 31u)) & 1u) break;
+    }
+  }
+  return hits;
+}
+
+// Rows of one mini block (bit k: row 32k + lane, string bytes at mb + st[k],
+// len[k] of them) that hold the pattern pat[0..plen), plen >= 1: kFsst with
+// the code-level matcher tables tab, else compared with the raw bytes.  Out of
+// line: inlined it would be compiled once per mini block of the tile.
+template <bool kHost, bool kFsst>
+__device__ __noinline__ uint32_t search_mb(const uint8_t* mb, uint4 st4, uint4 len4, const uint8_t* pat, uint32_t plen,
+                                           const uint8_t* tab, uint32_t* scratch, int lane) {
+  const uint32_t st[4] = {st4.x, st4.y, st4.z, st4.w}, len[4] = {len4.x, len4.y, len4.z, len4.w};
+  uint32_t* hits = scratch;
+  uint32_t* starts = scratch + kSearchHits;
+  const uint32_t total = __shfl_sync(kFull, st[3] + len[3], 31), skew = uint32_t(reinterpret_cast<uintptr_t>(mb)) & 15u;
+  const uint64_t end = uint64_t(skew) + total;
+  uint32_t pat4 = 0, mask4 = 0, match = 0;
+  if (!kFsst) {
+    for (uint32_t i = 0; i < tmin<uint32_t>(plen, 4u); ++i) {
+      pat4 |= uint32_t(pat[i]) << (8 * i);
+      mask4 |= 0xffu << (8 * i);
+    }
+  }
+  bool carry = false;
+  for (uint64_t w0 = 0; w0 < end; w0 += kSearchWin) {
+    const uint8_t* wp = mb - skew + w0;
+    const uint64_t left = end - w0;
+    const uint32_t wend = uint32_t(tmin<uint64_t>(left, kSearchWin));
+    if (kFsst) {
+      for (uint32_t i = lane; i < kSearchStarts; i += 32) starts[i] = 0;
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint64_t s = uint64_t(skew) + st[k] - w0;  // wraps below the window
+        if (s < kSearchWin + kSearchAhead) atomicOr(starts + (s >> 5), 1u << (s & 31u));
+      }
+      __syncwarp();
+    }
+    for (uint32_t c0 = 0; c0 * 16 < wend; c0 += 32) {
+      const uint32_t c = c0 + lane, at = c * 16;
+      uint32_t m = 0;
+      if (kFsst) {
+        const uint32_t skip = w0 == 0 && c == 0 ? skew : 0u;
+        m = find_fsst<kHost>(wp + at, at, skip, at < wend ? left - at : 0u, &carry, tab, plen, starts, lane);
+      } else if (at < wend) {
+        m = find_raw<kHost>(wp + at, left - at, pat, plen, pat4, mask4);
+      }
+      if (at < wend) reinterpret_cast<uint16_t*>(hits)[c] = uint16_t(m);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      // an occurrence in the raw bytes starts at most len - plen into the row
+      const uint32_t span = kFsst ? len[k] : (len[k] >= plen ? len[k] - plen + 1 : 0u);
+      const int64_t s = int64_t(skew) + int64_t(st[k]) - int64_t(w0), e = s + int64_t(span);
+      const uint32_t lo = uint32_t(tmax<int64_t>(s, 0)), hi = uint32_t(tmax<int64_t>(tmin<int64_t>(e, wend), 0));
+      if (s < int64_t(wend) && !((match >> k) & 1u) && any_bit(hits, lo, hi)) match |= 1u << k;
+    }
+    __syncwarp();
+  }
+  return match;
+}
+
+// A general LIKE over a tile: rows that hold the pattern's longest run of
+// literal bytes (S.in[0..1]: where it starts and its length, from the plan)
+// are candidates, queued over the tile's mini blocks and matched in full 32
+// at a time, so the byte-by-byte matcher runs on few rows and full warps.
+// like_push queues the rows of one mini block, matching a round when 32 are
+// waiting; like_round matches the queue's first up to 32; a matching row sets
+// its result bit.
+template <bool kHost>
+__device__ __forceinline__ void like_round(const DevStep& S, const uint8_t* bytes, uint32_t* queue, uint32_t* result,
+                                           uint32_t n, int lane) {
+  if (lane < int(n)) {
+    const uint32_t row = queue[3 * lane + 2];
+    if (like_match<kHost>(S, bytes + queue[3 * lane], queue[3 * lane + 1]))
+      atomicOr(result + (row >> 5), 1u << (row & 31u));
+  }
+  __syncwarp();
+}
+template <bool kHost>
+__device__ __forceinline__ uint32_t like_push(const DevStep& S, const uint8_t* bytes, uint32_t mb_start,
+                                              const uint32_t (&st)[4], const uint32_t (&len)[4], uint32_t cand, int t,
+                                              uint32_t* queue, uint32_t* result, uint32_t n, int lane) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const bool c = (cand >> k) & 1u;
+    const uint32_t m = __ballot_sync(kFull, c);
+    if (c) {
+      uint32_t* q = queue + 3 * (n + __popc(m & ((1u << lane) - 1u)));
+      q[0] = mb_start + st[k];
+      q[1] = len[k];
+      q[2] = uint32_t(t * kMB + k * 32 + lane);
+    }
+    __syncwarp();
+    n += __popc(m);
+    if (n < 32) continue;
+    like_round<kHost>(S, bytes, queue, result, 32, lane);
+    n -= 32;  // the rows left over move to the front
+    uint32_t e[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) e[i] = queue[3 * (32 + lane) + i];
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 3; ++i) queue[3 * lane + i] = e[i];
+    __syncwarp();
+  }
+  return n;
+}
+
 // PREFIX / CONTAINS step over a string column, dense: lengths decoded, their
 // exclusive scan gives each string's start, then each live row's string is
 // matched.  kText = false compiles the raw-PREFIX path only (the general
 // matcher of CONTAINS and FSST is left out of the kernel's code); the host
 // launches that build only for batches without such steps, and a step it
-// cannot run drops its rows and reports S_INTERNAL.
+// cannot run drops its rows and reports S_INTERNAL.  With the warp's scratch
+// (search), a CONTAINS (on FSST: with its matcher tables) and a general LIKE
+// search the mini blocks' bytes cooperatively; without it (the build kernels)
+// and for PREFIX on FSST, which reads a code or two, each lane matches its
+// own strings.
 template <bool kHost, bool kText = true>
 __device__ __forceinline__ void tile_prefix(const DevQuery& Q, const DevStep& S, const PageState& P,
                                             const TileHdr& Hd, TileState& T, int lane, unsigned int* status,
-                                            const uint8_t* stab) {
+                                            const uint8_t* stab, uint32_t* search) {
   uint32_t len[TB][4];
   uint32_t anym;
   tile_decode<kHost>(Q, S.col, P, Hd, T.alive, lane, len, anym, status);
@@ -507,12 +758,27 @@ __device__ __forceinline__ void tile_prefix(const DevQuery& Q, const DevStep& S,
   const int4* sym = Q.cols[S.col].codec == C_FSST ? Q.cols[S.col].sym : nullptr;
   const uint8_t* tab = sym != nullptr && S.smem_width ? stab + S.smem_off : nullptr;
   const bool lockstep = S.kind == ST_PREFIX && sym == nullptr;
+  uint32_t* queue = search + kSearchHits;
+  uint32_t* result = queue + 3 * kLikeQueue;
+  uint32_t waiting = 0;
+  const bool coop = kText && search != nullptr && S.plen != 0 &&
+                    ((S.kind == ST_CONTAINS && (sym == nullptr || tab != nullptr)) || (S.kind == ST_LIKE && sym == nullptr));
+  if (kText && coop && S.kind == ST_LIKE) {
+    if (lane < int(kMB * TB / 32)) result[lane] = 0;
+    __syncwarp();
+  }
 #pragma unroll
   for (int t = 0; t < TB; ++t) {
     if (!((anym >> t) & 1u)) continue;
+    if (coop) {  // rows past the page's last have no bytes (their field decodes to the mini block's base)
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (!((T.alive >> (4 * t + k)) & 1u)) len[t][k] = 0;
+    }
     uint32_t st[4];
     excl_scan128(len[t], lane, st);
-    const uint8_t* mb = bytes + __shfl_sync(kFull, Hd.sstart, S.col * TB + t);
+    const uint32_t mb_start = __shfl_sync(kFull, Hd.sstart, S.col * TB + t);
+    const uint8_t* mb = bytes + mb_start;
     uint32_t match = 0;
     if (lockstep) {
       // raw PREFIX: the warp compares byte i of all its rows' strings at once
@@ -532,15 +798,41 @@ __device__ __forceinline__ void tile_prefix(const DevQuery& Q, const DevStep& S,
       }
     } else {
       if constexpr (kText) {
+        if (coop) {
+          const uint32_t live = (T.alive >> (4 * t)) & 15u;
+          const uint4 st4 = make_uint4(st[0], st[1], st[2], st[3]);
+          const uint4 len4 = make_uint4(len[t][0], len[t][1], len[t][2], len[t][3]);
+          if (S.kind == ST_CONTAINS) {
+            match = sym != nullptr ? search_mb<kHost, true>(mb, st4, len4, S.pfx, S.plen, tab, search, lane)
+                                   : search_mb<kHost, false>(mb, st4, len4, S.pfx, S.plen, nullptr, search, lane);
+          } else {
+            const uint32_t run = uint32_t(S.in[1]);
+            match = run == 0 ? live
+                             : search_mb<kHost, false>(mb, st4, len4, S.pfx + S.in[0], run, nullptr, search, lane);
+            waiting = like_push<kHost>(S, bytes, mb_start, st, len[t], match & live, t, queue, result, waiting, lane);
+          }
+        } else {
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (((T.alive >> (4 * t + k)) & 1u) && string_match<kHost>(S, mb + st[k], len[t][k], sym, tab))
-            match |= 1u << k;
+          for (int k = 0; k < 4; ++k)
+            if (((T.alive >> (4 * t + k)) & 1u) && string_match<kHost>(S, mb + st[k], len[t][k], sym, tab))
+              match |= 1u << k;
+        }
       } else {
         if (lane == 0) atomicOr(status, S_INTERNAL);
       }
     }
     T.alive &= ~((~match & 15u) << (4 * t));
+  }
+  if constexpr (kText) {
+    if (coop && S.kind == ST_LIKE) {
+      like_round<kHost>(S, bytes, queue, result, waiting, lane);
+#pragma unroll
+      for (int t = 0; t < TB; ++t)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (!((result[4 * t + k] >> lane) & 1u)) T.alive &= ~(1u << (4 * t + k));
+      __syncwarp();
+    }
   }
 }
 
@@ -952,12 +1244,12 @@ static_assert(kSegMbs <= 32, "segment mini blocks must fit a 32-bit mask");
 template <bool kHost, bool kText = true, bool kGid = true, bool kStaged = false>
 __device__ __forceinline__ void tile_dense_step(const DevQuery& Q, uint32_t s, const PageState& P, const TileHdr& Hd,
                                                 TileState& T, const uint8_t* stab, int lane, unsigned int* status,
-                                                StagedPay sp = StagedPay{nullptr, 0, 0}) {
+                                                StagedPay sp = StagedPay{nullptr, 0, 0}, uint32_t* search = nullptr) {
   if (s >= Q.nsteps) return;
   const DevStep& S = Q.steps[s];
   if (S.kind == ST_ALL) return;  // every row passes; its column is never read
   if (S.kind == ST_PREFIX || S.kind == ST_CONTAINS || S.kind == ST_LIKE) {
-    if (!kStaged) tile_prefix<kHost, kText>(Q, S, P, Hd, T, lane, status, stab);
+    if (!kStaged) tile_prefix<kHost, kText>(Q, S, P, Hd, T, lane, status, stab, search);
     else if (lane == 0) atomicOr(status, S_INTERNAL);
   } else if (Q.cols[S.col].codec == C_DELTA) {
     dense_step_t<kHost, true, kGid, kStaged>(Q, S, P, Hd, T, stab, lane, status, sp);
