@@ -1078,7 +1078,9 @@ uint64_t plans_signature(dpf_ctx* c, const dpf_plan* plans, int32_t n) {
 
 // Fields left 0 take the tuning dpf_autotune stored for these plans, else the
 // defaults.
-void fill_tuning_defaults(dpf_ctx* c, dpf_tuning& t, const dpf_plan* plans, int32_t n) {
+// Returns whether something named the ticket size (else kDefaultChunkRows is
+// the largest one and layout_tickets chooses).
+bool fill_tuning_defaults(dpf_ctx* c, dpf_tuning& t, const dpf_plan* plans, int32_t n) {
   if (t.chunk_rows == 0 || t.threads == 0 || t.ht_placement == 0 || t.ctas_per_sm == 0 || t.staging == 0 ||
       t.group_agg == 0) {
     auto it = c->tune_cache.find(plans_signature(c, plans, n));
@@ -1098,11 +1100,13 @@ void fill_tuning_defaults(dpf_ctx* c, dpf_tuning& t, const dpf_plan* plans, int3
   if (t.ctas_per_sm == 0) t.ctas_per_sm = d.ctas_per_sm;
   if (t.staging == 0) t.staging = d.staging;
   if (t.group_agg == 0) t.group_agg = d.group_agg;
+  const bool fixed_chunk = t.chunk_rows != 0;
   if (t.chunk_rows == 0) t.chunk_rows = kDefaultChunkRows;
   if (t.threads == 0) t.threads = 256;
   if (t.ht_placement == 0) t.ht_placement = DPF_HT_AUTO;
   if (t.staging == 0) t.staging = kDefaultStaging;
   if (t.group_agg == 0) t.group_agg = kDefaultGroupAgg;
+  return fixed_chunk;
 }
 
 // A flat JSON object of launch-configuration fields (dpf_set_tuning): the
@@ -1237,7 +1241,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   p->hq.resize(size_t(n));
   dpf_tuning t{};
   if (tuning) t = *tuning;
-  fill_tuning_defaults(c, t, plans, n);
+  const bool fixed_chunk = fill_tuning_defaults(c, t, plans, n);
   if (t.chunk_rows % (kMbPerWarpTile * kMB) != 0 || t.chunk_rows > (1u << 24))
     return fail(DPF_EINVAL, "chunk_rows %u must be a multiple of %u and at most 2^24", t.chunk_rows, kMbPerWarpTile * kMB);
   if (t.threads != 128 && t.threads != 256 && t.threads != 512 && t.threads != 1024)
@@ -1247,8 +1251,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     return fail(DPF_EINVAL, "group_agg must be 0, 1 or 2");
   bool any_warp_agg = false;
   bool host = false;
-  uint64_t tickets = 0;
-  std::vector<uint64_t> qbegin(size_t(n) + 1);
+  std::vector<uint64_t> qbegin(2 * size_t(n) + 2);
   // scratch layout per query: acc | done | out_n | out
   std::vector<uint64_t> off_acc(n), off_done(n), off_outn(n), off_out(n);
   uint64_t scratch = 0;
@@ -1270,11 +1273,6 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     host |= h;
     const size_t used = place_tables(Q, table_budget, t.ht_placement == DPF_HT_AUTO);
     max_tables = std::max(max_tables, used);
-    Q.chunk_rows = t.chunk_rows;
-    Q.nchunks = (Q.nrows + t.chunk_rows - 1) / t.chunk_rows;
-    Q.chunk_begin = tickets;
-    qbegin[i] = tickets;
-    tickets += Q.nchunks;
     const uint32_t S1 = 1 + Q.naggs;
     Q.use_smem_acc = uint64_t(Q.domain) * S1 <= kSmemAccSlots ? 1u : 0u;
     Q.warp_agg = t.group_agg == DPF_GROUP_AGG_WARP && Q.domain > 1 ? 1u : 0u;
@@ -1285,7 +1283,6 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     off_outn[i] = scratch; scratch += 16;
     off_out[i] = scratch; scratch += align16(uint64_t(std::max<uint32_t>(Q.domain, 1)) * sizeof(dpf_record));
   }
-  qbegin[n] = tickets;
   // Staging ring: a launch stages all of its queries or none; a query can be
   // staged when its first step is an integer step over device-resident
   // pages.  The ring's slots are as wide as the widest mini block of those
@@ -1312,7 +1309,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
                 t.threads);
   dpf_status st;
   if ((st = dev_alloc(c, scratch, reinterpret_cast<void**>(&p->scratch)))) return st;
-  if ((st = dev_alloc_t(c, uint64_t(n), &p->dq)) || (st = dev_alloc_t(c, uint64_t(n) + 1, &p->dqbegin)) ||
+  if ((st = dev_alloc_t(c, uint64_t(n), &p->dq)) || (st = dev_alloc_t(c, qbegin.size(), &p->dqbegin)) ||
       (st = dev_alloc_t(c, 1, &p->sched))) {
     release_prep(c, p.get());
     return st;
@@ -1326,9 +1323,6 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   }
   cudaError_t e = cudaMemsetAsync(p->scratch, 0, scratch, c->io);
   if (e == cudaSuccess) e = cudaMemsetAsync(p->sched, 0, sizeof(Sched), c->io);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(p->dq, p->hq.data(), sizeof(DevQuery) * n, cudaMemcpyHostToDevice, c->io);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(p->dqbegin, qbegin.data(), 8 * (n + 1), cudaMemcpyHostToDevice, c->io);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->io);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     release_prep(c, p.get());
@@ -1349,62 +1343,25 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     return fail(DPF_EINVAL, "fused kernel does not fit on an SM with %u threads and %zu table bytes", t.threads, max_tables);
   }
   if (t.ctas_per_sm == 0 || int(t.ctas_per_sm) > per_sm || min_blocks == kFusedMinBlocksHi) t.ctas_per_sm = uint32_t(per_sm);
-  // Tickets are handed out in order, so the launch ends on the last query's
-  // last tickets.  Whole-size tickets there leave most warps idle while the
-  // last few finish; the final rows (about two tickets of tail_rows per warp
-  // of the grid, taken from the last queries backwards) are cut into tickets
-  // of chunk_rows / 8 rows instead.  In a batch the same holds at every query
-  // switch: a CTA's warps meet when their tickets leave a query (its plan,
-  // tables and accumulators sit in shared memory), so each query's last rows
-  // (one small ticket per warp of the grid) are cut small as well.
-  {
-    const uint64_t warps = uint64_t(c->num_sms) * t.ctas_per_sm * (t.threads / 32);
-    const uint32_t tile_rows = kMbPerWarpTile * kMB;
-    const uint32_t tail_rows = std::max<uint32_t>(tile_rows, t.chunk_rows / 8 / tile_rows * tile_rows);
-    std::vector<uint64_t> tail_len(size_t(n), 0);
-    if (tail_rows < t.chunk_rows) {
-      if (n > 1)
-        for (int i = 0; i < n; ++i) tail_len[size_t(i)] = std::min<uint64_t>(p->hq[i].nrows, warps * tail_rows);
-      uint64_t want = 2 * warps * tail_rows;
-      for (int i = n - 1; i >= 0 && want > 0; --i) {
-        const uint64_t rows = std::min<uint64_t>(p->hq[i].nrows, want);
-        tail_len[size_t(i)] = std::max(tail_len[size_t(i)], rows);
-        want -= rows;
-      }
-    }
-    for (int i = 0; i < n; ++i) {
-      DevQuery& Q = p->hq[i];
-      if (tail_len[size_t(i)] == 0) continue;
-      const uint64_t keep_big = (Q.nrows - tail_len[size_t(i)]) / t.chunk_rows;
-      Q.tail_first = keep_big;
-      Q.tail_rows = tail_rows;
-      const uint64_t tail = Q.nrows - keep_big * t.chunk_rows;
-      Q.nchunks = keep_big + (tail + tail_rows - 1) / tail_rows;
-    }
-    tickets = 0;
-    for (int i = 0; i < n; ++i) {
-      p->hq[i].chunk_begin = tickets;
-      qbegin[i] = tickets;
-      tickets += p->hq[i].nchunks;
-    }
-    qbegin[n] = tickets;
-    e = cudaMemcpyAsync(p->dq, p->hq.data(), sizeof(DevQuery) * n, cudaMemcpyHostToDevice, c->io);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(p->dqbegin, qbegin.data(), 8 * (n + 1), cudaMemcpyHostToDevice, c->io);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->io);
-    if (e != cudaSuccess) {
-      release_prep(c, p.get());
-      return fail(DPF_ECUDA, "prepare: %s", cudaGetErrorString(e));
-    }
+  layout_tickets(p->hq.data(), n, uint64_t(c->num_sms) * t.ctas_per_sm * (t.threads / 32), t.chunk_rows, fixed_chunk,
+                 qbegin.data());
+  e = cudaMemcpyAsync(p->dq, p->hq.data(), sizeof(DevQuery) * n, cudaMemcpyHostToDevice, c->io);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(p->dqbegin, qbegin.data(), 8 * qbegin.size(), cudaMemcpyHostToDevice, c->io);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->io);
+  if (e != cudaSuccess) {
+    release_prep(c, p.get());
+    return fail(DPF_ECUDA, "prepare: %s", cudaGetErrorString(e));
   }
   p->L.min_blocks = min_blocks;
   p->tuning = t;
   p->L.queries = p->dq;
   p->L.qbegin = p->dqbegin;
   p->L.nq = n;
-  p->L.total_chunks = tickets;
+  p->L.owned = qbegin[size_t(n)];
+  p->L.pool = qbegin[2 * size_t(n) + 1];
   p->L.sched = p->sched;
   p->L.threads = int(t.threads);
-  p->L.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(uint64_t(c->num_sms) * t.ctas_per_sm, tickets)));
+  p->L.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(uint64_t(c->num_sms) * t.ctas_per_sm, p->L.owned + p->L.pool)));
   p->L.smem_tables = max_tables;
   p->L.acc_slots = acc_slots;
   p->L.host_data = host;

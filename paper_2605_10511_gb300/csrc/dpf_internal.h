@@ -141,11 +141,11 @@ struct alignas(16) DevQuery {
   uint64_t nrows;
   uint32_t page_rows;
   uint32_t chunk_rows;
-  uint64_t chunk_begin;        // first global ticket of this query
+  // Tickets of the query (layout_tickets): the first tail_first are owned by
+  // CTAs and cover chunk_rows rows each; the others are in the pool and cover
+  // tail_rows rows each, from row tail_first * chunk_rows on (tail_rows == 0:
+  // every ticket is owned).
   uint64_t nchunks;
-  // The launch's last tickets are cut smaller so that warps finish together:
-  // tickets from tail_first on cover tail_rows rows each, starting at row
-  // tail_first * chunk_rows (tail_rows == 0: every ticket covers chunk_rows).
   uint64_t tail_first;
   uint32_t tail_rows;
   uint32_t stage;              // > 0: the first step's mini blocks are staged in the warp's

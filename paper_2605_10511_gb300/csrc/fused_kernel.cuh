@@ -4,10 +4,9 @@
 // general string matcher, host-resident pages; 3 and 4 resident CTAs per
 // SM each), so the builds compile in parallel.
 //
-// One launch executes every query of a batch.  Each CTA repeatedly takes a
+// One launch executes every query of a batch.  Each warp repeatedly takes a
 // ticket (one chunk of one query's fact table: the outer loop of Sec. 3.2
-// without host intervention), splits the chunk into warp tiles of
-// TB mini blocks and runs decode -> predicates -> probes -> aggregation on
+// without host intervention), splits the chunk into tiles of TB mini blocks and runs decode -> predicates -> probes -> aggregation on
 // them with all row state in registers.  Per-CTA int64 accumulators live in
 // shared memory while the CTA stays on one query; they are added to the
 // query's global accumulators when the CTA moves to another query or exits.
@@ -32,6 +31,7 @@ __device__ __forceinline__ uint32_t* shared_acc() { return reinterpret_cast<uint
 struct alignas(16) CtaState {
   DevQuery q;
   int wq[32];          // query of the ticket each warp holds (INT_MAX: none left)
+  unsigned int drawn;  // tickets drawn from the CTA's own range
   unsigned int mine;   // tickets of the current query this CTA processed
   int last;
   unsigned int warp_sum[32];
@@ -374,8 +374,8 @@ __device__ __forceinline__ FirstCol first_col(const DevQuery& Q, const PageState
 }
 
 // One ticket: the rows [chunk*chunk_rows, +chunk_rows) of Q's fact table
-// (a smaller range for the launch's last tickets: tail_first / tail_rows),
-// processed by one warp, cut at page boundaries into tiles.  A page whose
+// (a smaller range for the pool's tickets: tail_first / tail_rows), processed
+// by one warp, cut at page boundaries into tiles.  A page whose
 // zone map misses the first step's value range is skipped whole; inside a
 // page, mini blocks whose headers miss it are skipped by the first step.
 // Each tile loads its headers as it starts (the other resident warps hide
@@ -388,7 +388,7 @@ __device__ void process_ticket(const DevQuery& Q, uint64_t chunk, const uint8_t*
                                uint8_t* ring) {
   const uint64_t PR = Q.page_rows;
   uint64_t r0 = chunk * Q.chunk_rows, r1 = r0 + Q.chunk_rows;
-  if (Q.tail_rows != 0 && chunk >= Q.tail_first) {  // one of the launch's small last tickets
+  if (Q.tail_rows != 0 && chunk >= Q.tail_first) {  // one of the pool's
     r0 = Q.tail_first * Q.chunk_rows + (chunk - Q.tail_first) * Q.tail_rows;
     r1 = r0 + Q.tail_rows;
   }
@@ -505,32 +505,52 @@ __device__ void load_smem_tables(const DevQuery& Q, uint8_t* stab) {
 template <bool kHost, int kMinBlocks, bool kText, bool kStage = false, int kThreads = 256>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQuery* __restrict__ queries,
                                                        const uint64_t* __restrict__ qbegin, int nq,
-                                                       uint64_t total, Sched* sched, uint32_t acc_slots,
-                                                     uint32_t tables_bytes, uint32_t stage_bw) {
+                                                       uint64_t owned, uint64_t pool, Sched* sched,
+                                                       uint32_t acc_slots, uint32_t tables_bytes,
+                                                       uint32_t stage_bw) {
   __shared__ CtaState cs;
   uint32_t* sacc = shared_acc();
   uint8_t* stab = dyn + ((acc_slots * sizeof(unsigned long long) + 15) & ~size_t(15));
   uint32_t* lists = reinterpret_cast<uint32_t*>(stab + tables_bytes);
-  // Warps draw tickets on their own (one ticket = chunk_rows rows of one
-  // query, processed by one warp), so no CTA barrier separates tickets.  The
-  // CTA meets only when its warps' tickets leave the current query: it then
-  // moves to the smallest query any warp holds (tickets are handed out in
-  // query order, so every warp reaches that meeting point), flushing the
-  // finished query's accumulators first.
+  // Warps draw tickets on their own (one ticket = a range of rows of one
+  // query, processed by one warp), so no CTA barrier separates tickets.  Each
+  // CTA owns an equal run of the launch's `owned` tickets, which its warps
+  // draw with a shared-memory counter: it stays on one query, or few, of a
+  // batch, and a small launch's warps need no global atomic.  Then its warps
+  // draw from the `pool` of small tickets all CTAs share (sched->next), so
+  // that they finish together.  The CTA meets only when its warps' tickets
+  // leave the current query: it flushes that query's accumulators and moves to
+  // the smallest query any warp holds.
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   uint32_t* list = lists + uint32_t(warp) * kListCap;
   uint8_t* ring = reinterpret_cast<uint8_t*>(lists + nw * kListCap) +
                   size_t(warp) * (kText ? kSearchWords * sizeof(uint32_t) : stage_warp_bytes(stage_bw));
+  const uint64_t own0 = owned * blockIdx.x / gridDim.x, own1 = owned * (blockIdx.x + 1) / gridDim.x;
+  if (threadIdx.x == 0) cs.drawn = 0;
+  __syncthreads();
+  // Draws the warp's next ticket: its query (INT_MAX: none left), and in t its
+  // index among the query's tickets (owned ones first).  qbegin[0..nq] = each
+  // query's first owned ticket, qbegin[nq + 1 ..] = its first pool ticket.
   auto draw = [&](unsigned long long& t) -> int {
-    unsigned long long x = 0;
-    if (lane == 0) x = atomicAdd(&sched->next, 1ull);
-    t = __shfl_sync(kFull, x, 0);
-    if (t >= total) return INT_MAX;
-    int lo = 0, hi = nq - 1;  // last query with qbegin <= t
+    unsigned int x = 0;
+    if (lane == 0) x = atomicAdd(&cs.drawn, 1u);
+    t = own0 + __shfl_sync(kFull, x, 0);
+    const uint64_t* begin = qbegin;
+    const bool mine = t < own1;
+    if (!mine) {
+      if (pool == 0) return INT_MAX;
+      if (lane == 0) t = atomicAdd(&sched->next, 1ull);
+      t = __shfl_sync(kFull, t, 0);
+      if (t >= pool) return INT_MAX;
+      begin += nq + 1;
+    }
+    int lo = 0, hi = nq - 1;  // last query with begin <= t
     while (lo < hi) {
       const int mid = (lo + hi + 1) / 2;
-      if (__ldg(qbegin + mid) <= t) lo = mid; else hi = mid - 1;
+      if (__ldg(begin + mid) <= t) lo = mid; else hi = mid - 1;
     }
+    if (nq > 1) t -= __ldg(begin + lo);
+    if (!mine) t += nq > 1 ? __ldg(qbegin + lo + 1) - __ldg(qbegin + lo) : owned;
     return lo;
   };
   unsigned long long held;
@@ -560,7 +580,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
     cur = next;
     uint32_t done_here = 0;
     while (hq == cur) {
-      process_ticket<kHost, kText, kStage>(Q, held - Q.chunk_begin, stab, list, lane, &sched->status,
+      process_ticket<kHost, kText, kStage>(Q, held, stab, list, lane, &sched->status,
                                            ring);
       ++done_here;
       hq = draw(held);
@@ -594,7 +614,7 @@ cudaError_t launch_as(const FusedLaunch& L, size_t smem, uint32_t tb, cudaStream
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   k<<<L.grid, L.threads, smem, s>>>(
-      L.queries, L.qbegin, L.nq, L.total_chunks, L.sched, L.acc_slots, tb, L.stage_bw);
+      L.queries, L.qbegin, L.nq, L.owned, L.pool, L.sched, L.acc_slots, tb, L.stage_bw);
   return cudaGetLastError();
 }
 

@@ -46,13 +46,20 @@ constexpr uint64_t kRankMaxRange = uint64_t(1) << 28;
 // after one literal byte (256 entries).
 inline uint32_t fsst_match_bytes(uint32_t plen) { return (plen + 1) * 512u; }
 
+// Cuts the n queries of a launch into tickets for `warps` resident warps: sets
+// each query's chunk_rows, tail_first, tail_rows and nchunks and fills begin
+// (2 n + 2 entries, FusedLaunch::qbegin).  chunk_rows = the largest ticket;
+// fixed: every owned ticket has that size (a tuning that names it).
+void layout_tickets(DevQuery* Q, int n, uint64_t warps, uint32_t chunk_rows, bool fixed, uint64_t* begin);
+
 // Fused persistent kernel over a batch of compiled queries (Sec. 3.2).
-// qbegin[0..nq] = first ticket of each query (qbegin[nq] = total tickets).
+// qbegin[0..nq] = first owned ticket of each query (qbegin[nq] = owned),
+// qbegin[nq + 1 .. 2 nq + 1] = its first pool ticket (the last one = pool).
 struct FusedLaunch {
   const DevQuery* queries;
   const uint64_t* qbegin;
   int nq;
-  uint64_t total_chunks;
+  uint64_t owned, pool;
   Sched* sched;
   int grid, threads;
   uint32_t acc_slots;   // int64 shared accumulators per CTA (max over the batch)

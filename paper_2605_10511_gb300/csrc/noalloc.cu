@@ -113,30 +113,15 @@ extern "C" dpf_status dpf_execute_noalloc(dpf_ctx* ctx, const dpf_plan* plan, vo
   uint8_t* base = nullptr;
   if ((st = scratch_address(device, &base))) return st;
 
-  const uint32_t chunk_rows = kDefaultChunkRows;
-  Q.chunk_rows = chunk_rows;
-  Q.nchunks = (Q.nrows + chunk_rows - 1) / chunk_rows;
-  Q.chunk_begin = 0;
   Q.use_smem_acc = slots <= kSmemAccSlots ? 1u : 0u;
   Q.acc = reinterpret_cast<unsigned long long*>(base + kOffAcc);
   Q.done = reinterpret_cast<unsigned int*>(base + kOffDone);
   Q.out = out;
   Q.out_n = out_count;
-  const uint64_t qbegin[2] = {0, Q.nchunks};
-
-  // the region keeps the previous call's contents: clear the counters and
-  // accumulators, then write this call's plan
-  cudaError_t e = cudaMemsetAsync(base + kOffSched, 0, sizeof(Sched), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(base + kOffDone, 0, 256 + slots * 8, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(base + kOffBegin, qbegin, sizeof qbegin, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(base + kOffQuery, &Q, sizeof Q, cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) return fail(DPF_ECUDA, "dpf_execute_noalloc: %s", cudaGetErrorString(e));
-
   FusedLaunch L{};
   L.queries = reinterpret_cast<const DevQuery*>(base + kOffQuery);
   L.qbegin = reinterpret_cast<const uint64_t*>(base + kOffBegin);
   L.nq = 1;
-  L.total_chunks = Q.nchunks;
   L.sched = reinterpret_cast<Sched*>(base + kOffSched);
   L.threads = 256;
   L.smem_tables = smem_tables;
@@ -146,7 +131,19 @@ extern "C" dpf_status dpf_execute_noalloc(dpf_ctx* ctx, const dpf_plan* plan, vo
   L.min_blocks = kFusedMinBlocksLo;
   const int per_sm = fused_blocks_per_sm(L.threads, L.acc_slots, smem_tables, host, L.min_blocks, 0, L.text);
   if (per_sm < 1) return fail(DPF_EINVAL, "dpf_execute_noalloc: fused kernel does not fit on an SM");
+  uint64_t qbegin[4];
+  layout_tickets(&Q, 1, uint64_t(num_sms) * per_sm * (L.threads / 32), kDefaultChunkRows, false, qbegin);
+  L.owned = qbegin[1];
+  L.pool = qbegin[3];
   L.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(uint64_t(num_sms) * per_sm, Q.nchunks)));
+
+  // the region keeps the previous call's contents: clear the counters and
+  // accumulators, then write this call's plan
+  cudaError_t e = cudaMemsetAsync(base + kOffSched, 0, sizeof(Sched), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(base + kOffDone, 0, 256 + slots * 8, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(base + kOffBegin, qbegin, sizeof qbegin, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(base + kOffQuery, &Q, sizeof Q, cudaMemcpyHostToDevice, s);
+  if (e != cudaSuccess) return fail(DPF_ECUDA, "dpf_execute_noalloc: %s", cudaGetErrorString(e));
   e = launch_fused(L, s);
   if (e != cudaSuccess) return fail(DPF_ECUDA, "dpf_execute_noalloc launch: %s", cudaGetErrorString(e));
   return DPF_OK;
