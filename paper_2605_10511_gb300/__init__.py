@@ -438,7 +438,7 @@ class Context:
         n = C.c_uint64()
         cap = 1024
         while True:
-            buf = np.zeros(cap, RECORD_DTYPE)
+            buf = np.empty(cap, RECORD_DTYPE)
             st = lib().dpf_read_result(self.h, prep, i, _ptr(buf), cap, C.byref(n), timeout_ms)
             if st == -7:
                 cap = int(n.value)
@@ -517,7 +517,7 @@ class Context:
         n = C.c_uint64()
         cap = 1024
         while True:
-            buf = np.zeros(cap, RECORD_DTYPE)
+            buf = np.empty(cap, RECORD_DTYPE)
             st = lib().dpf_fetch_result(self.h, qid, _ptr(buf), cap, C.byref(n), timeout_ms)
             if st == -7:
                 cap = int(n.value)
@@ -548,7 +548,7 @@ class Server:
         times = QueryTimes()
         cap = 1024
         while True:
-            buf = np.zeros(cap, RECORD_DTYPE)
+            buf = np.empty(cap, RECORD_DTYPE)
             st = lib().dpf_server_wait(self.h, ticket, _ptr(buf), cap, C.byref(n), timeout_ms, C.byref(times))
             if st == -7:
                 cap = int(n.value)

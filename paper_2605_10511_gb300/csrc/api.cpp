@@ -73,6 +73,7 @@ struct HashTable {
   uint2* slots = nullptr;         // HT_OPEN
   uint32_t capacity = 0;          // HT_OPEN slots, HT_DIRECT entries, HT_RANK keys covered
   uint32_t* direct = nullptr;     // HT_DIRECT
+  uint32_t* block = nullptr;      // HT_DIRECT: its allocation, where that starts before direct
   uint8_t* rank = nullptr;        // HT_RANK: directory words, then payloads
   uint8_t* stage = nullptr;       // HT_RANK while building: pair count, then the staged pairs
   int32_t kmin = 0;
@@ -103,7 +104,12 @@ struct Prep {
   DevQuery* dq = nullptr;
   uint64_t* dqbegin = nullptr;
   Sched* sched = nullptr;
-  uint8_t* scratch = nullptr;     // accumulators, counters, outputs of all queries
+  uint8_t* scratch = nullptr;     // accumulators and counters of all queries
+  // Results, in mapped pinned host memory that the kernels write directly, so
+  // a read waits for the launch's event and copies nothing from the device:
+  // the launch's status word, then each query's record count and records.
+  uint8_t* results = nullptr;
+  std::vector<uint64_t> off_n, off_rec;  // byte offsets of the queries' counts and records
   FusedLaunch L{};
   dpf_tuning tuning{};
   cudaEvent_t ev = nullptr;
@@ -135,9 +141,8 @@ struct dpf_ctx {
   std::map<int32_t, std::unique_ptr<Prep>> preps;
   int32_t next_col = 1, next_ht = 1, next_prep = 1;
   cudaStream_t io = nullptr;      // private non-blocking stream for copies
-  Sched* bsched = nullptr;        // status word of hash builds
-  unsigned long long* bcount = nullptr;
-  int32_t* bkminmax = nullptr;
+  BuildStat* bstat = nullptr;     // outcome of the exactly sized hash builds: status, rows and key range
+  BuildStat* bout = nullptr;      // its pinned host copy
   int num_sms = 0;
   int smem_optin = 0;
   std::map<uint64_t, dpf_tuning> tune_cache;  // plan-set signature -> tuning chosen by dpf_autotune
@@ -148,6 +153,11 @@ struct dpf_ctx {
   // serving loop's overlapping batches.
   std::multimap<uint64_t, void*> cache;
   uint64_t cached = 0;
+  // Mapped pinned host blocks (batches' results, builds' outcomes): allocating
+  // one takes longer than a small query, so freed ones are kept for reuse.
+  std::map<void*, uint64_t> pin_sizes;
+  std::multimap<uint64_t, void*> pin_cache;
+  uint64_t pin_cached = 0;
 };
 
 namespace {
@@ -239,10 +249,46 @@ void dev_free(dpf_ctx* c, void* p) {
   }
 }
 
+constexpr uint64_t kPinCacheMaxBytes = uint64_t(64) << 20;  // freed pinned bytes kept for reuse
+
+// Mapped pinned host memory, the same address on the host and the device.
+dpf_status pin_alloc(dpf_ctx* c, uint64_t bytes, void** out) {
+  uint64_t size = 4096;
+  while (size < bytes) size <<= 1;
+  auto it = c->pin_cache.find(size);
+  if (it != c->pin_cache.end()) {
+    *out = it->second;
+    c->pin_cache.erase(it);
+    c->pin_cached -= size;
+  } else {
+    const cudaError_t e = cudaHostAlloc(out, size, cudaHostAllocMapped | cudaHostAllocPortable);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      *out = nullptr;
+      return fail(DPF_ENOMEM, "cudaHostAlloc(%llu): %s", (unsigned long long)size, cudaGetErrorString(e));
+    }
+  }
+  c->pin_sizes[*out] = size;
+  return DPF_OK;
+}
+
+void pin_free(dpf_ctx* c, void* p) {
+  auto it = c->pin_sizes.find(p);
+  if (!p || it == c->pin_sizes.end()) return;
+  const uint64_t size = it->second;
+  c->pin_sizes.erase(it);
+  if (c->pin_cached + size > kPinCacheMaxBytes) {
+    cudaFreeHost(p);
+    return;
+  }
+  c->pin_cache.emplace(size, p);
+  c->pin_cached += size;
+}
+
 // Frees a table's device blocks (and an asynchronous build's launch buffers).
 static void free_table(dpf_ctx* c, HashTable& ht) {
   dev_free(c, ht.slots);
-  dev_free(c, ht.direct);
+  dev_free(c, ht.block ? ht.block : ht.direct);
   dev_free(c, ht.rank);
   dev_free(c, ht.stage);
   dev_free(c, ht.bq);
@@ -250,7 +296,7 @@ static void free_table(dpf_ctx* c, HashTable& ht) {
   if (ht.hstat) cudaFreeHost(ht.hstat);
   if (ht.done) cudaEventDestroy(ht.done);
   ht.slots = nullptr;
-  ht.direct = nullptr;
+  ht.direct = ht.block = nullptr;
   ht.rank = nullptr;
   ht.stage = nullptr;
   ht.bq = nullptr;
@@ -1210,10 +1256,9 @@ dpf_status release_prep(dpf_ctx* c, Prep* p) {
   if (p->gexec) cudaGraphExecDestroy(p->gexec);
   if (p->graph) cudaGraphDestroy(p->graph);
   if (p->ev) cudaEventDestroy(p->ev);
-  dev_free(c, p->dq);
-  dev_free(c, p->dqbegin);
-  dev_free(c, p->sched);
+  dev_free(c, p->dq);  // with the ticket table and the scheduler state behind it
   dev_free(c, p->scratch);
+  pin_free(c, p->results);
   dev_free(c, p->unf_scratch);
   return DPF_OK;
 }
@@ -1228,13 +1273,18 @@ cudaError_t launch_prep(Prep* p, cudaStream_t s) {
   if (p->unfused) {
     uint32_t n = 0;
     cudaError_t e = launch_unfused(p->U, s, &n);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(p->results, &p->sched->status, 4, cudaMemcpyDeviceToHost, s);
     p->launches = n;
     return e;
   }
   return launch_fused(p->L, s);
 }
 
-dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tuning* tuning, Prep** out) {
+// Prepares a batch.  Its plans are uploaded and its scratch cleared on `on`
+// (a launch that follows there needs no wait), or, when that is nullptr, on the
+// private stream, which is waited for.
+dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tuning* tuning, Prep** out,
+                   const cudaStream_t* on = nullptr) {
   if (!plans || n < 1 || n > 4096) return fail(DPF_EINVAL, "need 1..4096 plans");
   auto p = std::make_unique<Prep>();
   p->nq = n;
@@ -1252,9 +1302,11 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   bool any_warp_agg = false;
   bool host = false;
   std::vector<uint64_t> qbegin(2 * size_t(n) + 2);
-  // scratch layout per query: acc | done | out_n | out
-  std::vector<uint64_t> off_acc(n), off_done(n), off_outn(n), off_out(n);
-  uint64_t scratch = 0;
+  // scratch per query: acc | done; results per query: record count | records
+  std::vector<uint64_t> off_acc(n), off_done(n);
+  uint64_t scratch = 0, results = 64;
+  p->off_n.resize(size_t(n));
+  p->off_rec.resize(size_t(n));
   size_t max_tables = 0;
   uint32_t acc_slots = 0;
   // SMEM placement: what the opt-in shared memory leaves after the largest
@@ -1280,8 +1332,8 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     if (Q.use_smem_acc) acc_slots = std::max<uint32_t>(acc_slots, Q.domain * S1);
     off_acc[i] = scratch; scratch += align16(uint64_t(Q.domain) * S1 * 8);
     off_done[i] = scratch; scratch += 16;
-    off_outn[i] = scratch; scratch += 16;
-    off_out[i] = scratch; scratch += align16(uint64_t(std::max<uint32_t>(Q.domain, 1)) * sizeof(dpf_record));
+    p->off_n[size_t(i)] = results; results += 16;
+    p->off_rec[size_t(i)] = results; results += align16(uint64_t(std::max<uint32_t>(Q.domain, 1)) * sizeof(dpf_record));
   }
   // Staging ring: a launch stages all of its queries or none; a query can be
   // staged when its first step is an integer step over device-resident
@@ -1307,27 +1359,6 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   if (t.threads > 256 && (host || text || stage_bw))
     return fail(DPF_EINVAL, "CTAs of %u threads run device-resident batches without string-matcher steps, unstaged",
                 t.threads);
-  dpf_status st;
-  if ((st = dev_alloc(c, scratch, reinterpret_cast<void**>(&p->scratch)))) return st;
-  if ((st = dev_alloc_t(c, uint64_t(n), &p->dq)) || (st = dev_alloc_t(c, qbegin.size(), &p->dqbegin)) ||
-      (st = dev_alloc_t(c, 1, &p->sched))) {
-    release_prep(c, p.get());
-    return st;
-  }
-  for (int i = 0; i < n; ++i) {
-    DevQuery& Q = p->hq[i];
-    Q.acc = reinterpret_cast<unsigned long long*>(p->scratch + off_acc[i]);
-    Q.done = reinterpret_cast<unsigned int*>(p->scratch + off_done[i]);
-    Q.out_n = reinterpret_cast<unsigned int*>(p->scratch + off_outn[i]);
-    Q.out = p->scratch + off_out[i];
-  }
-  cudaError_t e = cudaMemsetAsync(p->scratch, 0, scratch, c->io);
-  if (e == cudaSuccess) e = cudaMemsetAsync(p->sched, 0, sizeof(Sched), c->io);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev, cudaEventDisableTiming);
-  if (e != cudaSuccess) {
-    release_prep(c, p.get());
-    return fail(DPF_ECUDA, "prepare: %s", cudaGetErrorString(e));
-  }
   // ctas_per_sm >= 4 selects the kernel build for four resident CTAs per SM
   // (64 registers) when four fit; otherwise the build for three (80)
   int min_blocks = kFusedMinBlocksLo;
@@ -1345,9 +1376,38 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   if (t.ctas_per_sm == 0 || int(t.ctas_per_sm) > per_sm || min_blocks == kFusedMinBlocksHi) t.ctas_per_sm = uint32_t(per_sm);
   layout_tickets(p->hq.data(), n, uint64_t(c->num_sms) * t.ctas_per_sm * (t.threads / 32), t.chunk_rows, fixed_chunk,
                  qbegin.data());
-  e = cudaMemcpyAsync(p->dq, p->hq.data(), sizeof(DevQuery) * n, cudaMemcpyHostToDevice, c->io);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(p->dqbegin, qbegin.data(), 8 * qbegin.size(), cudaMemcpyHostToDevice, c->io);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->io);
+  // one device block, uploaded by one copy: plans | ticket table | scheduler state (zero)
+  const uint64_t at_begin = sizeof(DevQuery) * uint64_t(n), at_sched = align16(at_begin + 8 * qbegin.size());
+  dpf_status st;
+  if ((st = dev_alloc(c, scratch, reinterpret_cast<void**>(&p->scratch))) ||
+      (st = dev_alloc(c, at_sched + sizeof(Sched), reinterpret_cast<void**>(&p->dq))) ||
+      (st = pin_alloc(c, results, reinterpret_cast<void**>(&p->results)))) {
+    const std::string msg = t_last_error;
+    release_prep(c, p.get());
+    return fail(st, "%s", msg.c_str());
+  }
+  p->dqbegin = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(p->dq) + at_begin);
+  p->sched = reinterpret_cast<Sched*>(reinterpret_cast<uint8_t*>(p->dq) + at_sched);
+  std::memset(p->results, 0, 64);
+  for (int i = 0; i < n; ++i) {
+    DevQuery& Q = p->hq[i];
+    Q.acc = reinterpret_cast<unsigned long long*>(p->scratch + off_acc[i]);
+    Q.done = reinterpret_cast<unsigned int*>(p->scratch + off_done[i]);
+    Q.out_n = reinterpret_cast<unsigned int*>(p->results + p->off_n[size_t(i)]);
+    Q.out = p->results + p->off_rec[size_t(i)];
+    *reinterpret_cast<uint32_t*>(p->results + p->off_n[size_t(i)]) = 0;
+  }
+  std::vector<uint8_t> up(at_sched + sizeof(Sched), 0);
+  std::memcpy(up.data(), p->hq.data(), at_begin);
+  std::memcpy(up.data() + at_begin, qbegin.data(), 8 * qbegin.size());
+  const cudaStream_t us = on ? *on : c->io;
+  cudaError_t e = cudaMemsetAsync(p->scratch, 0, scratch, us);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(p->dq, up.data(), up.size(), cudaMemcpyHostToDevice, us);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev, cudaEventDisableTiming);
+  if (e != cudaSuccess || !on) {
+    const cudaError_t e2 = cudaStreamSynchronize(us);  // nothing may still write blocks that are freed
+    if (e == cudaSuccess) e = e2;
+  }
   if (e != cudaSuccess) {
     release_prep(c, p.get());
     return fail(DPF_ECUDA, "prepare: %s", cudaGetErrorString(e));
@@ -1360,6 +1420,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   p->L.owned = qbegin[size_t(n)];
   p->L.pool = qbegin[2 * size_t(n) + 1];
   p->L.sched = p->sched;
+  p->L.status_out = reinterpret_cast<unsigned int*>(p->results);
   p->L.threads = int(t.threads);
   p->L.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(uint64_t(c->num_sms) * t.ctas_per_sm, p->L.owned + p->L.pool)));
   p->L.smem_tables = max_tables;
@@ -1402,11 +1463,12 @@ dpf_status read_result(dpf_ctx* c, Prep* p, int32_t i, dpf_record* buf, uint64_t
   if (!p->launched) return fail(DPF_EINVAL, "batch %d was never launched", p->id);
   dpf_status st = wait_event(p->ev, timeout_ms);
   if (st) return st;
-  uint32_t status = 0, n = 0;
-  CUDA_TRY(cudaMemcpyAsync(&status, &p->sched->status, 4, cudaMemcpyDeviceToHost, c->io));
-  CUDA_TRY(cudaMemcpyAsync(&n, p->hq[i].out_n, 4, cudaMemcpyDeviceToHost, c->io));
-  CUDA_TRY(cudaStreamSynchronize(c->io));
+  // the launch's kernels wrote its status, counts and records here
+  uint32_t status, n;
+  std::memcpy(&status, p->results, 4);
+  std::memcpy(&n, p->results + p->off_n[size_t(i)], 4);
   if (status) {
+    std::memset(p->results, 0, 4);
     cudaMemsetAsync(&p->sched->status, 0, 4, c->io);
     cudaStreamSynchronize(c->io);
     if (status & S_CORRUPT) return fail(DPF_ECORRUPT, "device reported corrupt data (status %u)", status);
@@ -1416,8 +1478,7 @@ dpf_status read_result(dpf_ctx* c, Prep* p, int32_t i, dpf_record* buf, uint64_t
   if (cap < n) return fail(DPF_ETRUNC, "need %u records", n);
   if (n) {
     if (!buf) return fail(DPF_EINVAL, "buf is NULL");
-    CUDA_TRY(cudaMemcpyAsync(buf, p->hq[i].out, uint64_t(n) * sizeof(dpf_record), cudaMemcpyDeviceToHost, c->io));
-    CUDA_TRY(cudaStreamSynchronize(c->io));
+    std::memcpy(buf, p->results + p->off_rec[size_t(i)], uint64_t(n) * sizeof(dpf_record));
   }
   return DPF_OK;
 }
@@ -1474,11 +1535,9 @@ dpf_status dpf_create(dpf_ctx** out, int32_t device, uint64_t hbm_budget, const 
   CUDA_TRY(cudaDeviceGetAttribute(&c->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
   CUDA_TRY(cudaStreamCreateWithFlags(&c->io, cudaStreamNonBlocking));
   dpf_status st;
-  if ((st = dev_alloc_t(c.get(), 1, &c->bsched)) || (st = dev_alloc_t(c.get(), 1, &c->bcount)) ||
-      (st = dev_alloc_t(c.get(), 2, &c->bkminmax)))
+  if ((st = dev_alloc_t(c.get(), 1, &c->bstat)) ||
+      (st = pin_alloc(c.get(), sizeof(BuildStat), reinterpret_cast<void**>(&c->bout))))
     return st;
-  CUDA_TRY(cudaMemsetAsync(c->bsched, 0, sizeof(Sched), c->io));
-  CUDA_TRY(cudaStreamSynchronize(c->io));
   *out = c.release();
   return DPF_OK;
 }
@@ -1493,10 +1552,10 @@ dpf_status dpf_destroy(dpf_ctx* c) {
     c->preps.clear();
     for (auto& kv : c->hts) free_table(c, kv.second);
     for (auto& kv : c->cols) free_column(c, kv.second);
-    dev_free(c, c->bsched);
-    dev_free(c, c->bcount);
-    dev_free(c, c->bkminmax);
+    dev_free(c, c->bstat);
     drop_cache(c);
+    pin_free(c, c->bout);
+    for (auto& kv : c->pin_cache) cudaFreeHost(kv.second);
     if (c->io) cudaStreamDestroy(c->io);
   }
   delete c;
@@ -1863,7 +1922,7 @@ static dpf_status alloc_table(dpf_ctx* c, const BuildSpec& bs, uint64_t kept, in
     L.krange = ht.capacity;
     e = cudaMemsetAsync(ht.rank, 0, 16 * nwords, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(ht.stage, 0, 16, s);
-  } else if (!bs.wide_payload && range <= std::max<uint64_t>(64 * kept, 1u << 20) && range <= kDirectMaxRange) {
+  } else if (!bs.wide_payload && range <= std::max<uint64_t>(64 * kept, kDirectAlways) && range <= kDirectMaxRange) {
     ht.kind = HT_DIRECT;
     ht.kmin = range ? int32_t(lo) : 0;
     ht.capacity = uint32_t(range);
@@ -1893,8 +1952,14 @@ static dpf_status build_status_error(uint32_t status, dpf_col_id key_col) {
   return fail(DPF_EINTERNAL, "hash build status %u", status);
 }
 
-// Exact sizing: a count pass finds the kept rows and their key range, the
-// host reads them back and sizes the table, then the insert pass fills it.
+// Exact sizing.  When the key column's load-time bounds span at most
+// kDirectAlways keys (and no budget limits the context's memory), the table is
+// a direct one whatever rows are kept: one pass fills a table over those
+// bounds, and the table is its part from the smallest to the largest key kept
+// (what an exactly sized one would hold).
+// Otherwise a count pass finds the kept rows and their key range, the host
+// reads them back and sizes the table, then the insert pass fills it.  Each
+// pass's outcome comes back in one copy.
 static dpf_status build_hash_impl(dpf_ctx* c, const dpf_build& B, void* stream, dpf_ht_id* out) {
   if (!c || !out) return fail(DPF_EINVAL, "NULL argument");
   std::lock_guard<std::recursive_mutex> lk(c->mu);
@@ -1904,44 +1969,70 @@ static dpf_status build_hash_impl(dpf_ctx* c, const dpf_build& B, void* stream, 
   dpf_status st = compile_build(c, B, bs);
   if (st) return st;
   HashTable& ht = bs.ht;
+  const Column& kc = c->cols[B.key_col];
   DevQuery* dq;
   if ((st = dev_alloc_t(c, 1, &dq))) return st;
   BuildLaunch L{};
   L.q = dq;
-  L.count = c->bcount;
-  L.sched = c->bsched;
+  L.stat = c->bstat;
   L.nrows = bs.Q.nrows;
   L.page_rows = bs.Q.page_rows;
   L.host_data = bs.host;
-  L.kminmax = c->bkminmax;
-  unsigned long long kept = 0;
-  int32_t minmax[2] = {INT32_MAX, INT32_MIN};
-  uint32_t status = 0;
+  L.measure = true;
   auto cleanup = [&](dpf_status r) {
     dev_free(c, dq);
     return r;
   };
+  const BuildStat zero{};
+  auto outcome = [&](cudaError_t e) {  // the enqueued pass's outcome, in c->bout
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c->bout, c->bstat, sizeof(BuildStat), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    return e;
+  };
   cudaError_t e = cudaMemcpyAsync(dq, &bs.Q, sizeof bs.Q, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->bcount, 0, 8, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->bsched, 0, sizeof(Sched), s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(c->bkminmax, minmax, 8, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = launch_build_count(L, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&kept, c->bcount, 8, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(minmax, c->bkminmax, 8, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return cleanup(fail(DPF_ECUDA, "hash build (count): %s", cudaGetErrorString(e)));
-  if ((st = alloc_table(c, bs, kept, minmax[0], minmax[1], ht, L, s))) {
-    free_table(c, ht);
-    return cleanup(st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(c->bstat, &zero, sizeof zero, cudaMemcpyHostToDevice, s);
+  bool done = false;
+  uint64_t kept = 0;
+  const uint64_t span = kc.vmin <= kc.vmax ? uint64_t(kc.vmax - kc.vmin + 1) : 0;
+  if (e == cudaSuccess && !bs.wide_payload && span != 0 && span <= kDirectAlways && c->budget == 0) {
+    st = alloc_table(c, bs, kc.nrows, kc.vmin, kc.vmax, ht, L, s);
+    if (st == DPF_OK) {
+      e = outcome(launch_build_insert(L, s));
+      done = true;
+      kept = c->bout->inserted;
+    } else {  // too large for what memory is left: size it exactly
+      free_table(c, ht);
+      ht.key_lo = 1;
+      ht.key_hi = 0;
+      L.direct = nullptr;
+    }
   }
-  ht.entries = kept;
-  e = launch_build_insert(L, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&status, &c->bsched->status, 4, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess || status) {
+  if (!done) {
+    if (e == cudaSuccess) e = outcome(launch_build_count(L, s));
+    if (e != cudaSuccess) return cleanup(fail(DPF_ECUDA, "hash build (count): %s", cudaGetErrorString(e)));
+    // the count pass's status bits (corrupt data) stay set for the insert pass
+    kept = c->bout->inserted;
+    if ((st = alloc_table(c, bs, kept, c->bout->key_lo(), c->bout->key_hi(), ht, L, s))) {
+      free_table(c, ht);
+      return cleanup(st);
+    }
+    L.measure = false;
+    e = outcome(launch_build_insert(L, s));
+  }
+  if (e != cudaSuccess || c->bout->sched.status) {
     free_table(c, ht);
     if (e != cudaSuccess) return cleanup(fail(DPF_ECUDA, "hash build (insert): %s", cudaGetErrorString(e)));
-    return cleanup(build_status_error(status, B.key_col));
+    return cleanup(build_status_error(c->bout->sched.status, B.key_col));
+  }
+  ht.entries = kept;
+  if (done) {  // the part of the table over the keys kept
+    const int64_t lo = c->bout->key_lo(), hi = c->bout->key_hi();
+    ht.key_lo = ht.entries ? int32_t(lo) : 1;
+    ht.key_hi = ht.entries ? int32_t(hi) : 0;
+    ht.block = ht.direct;
+    ht.direct += ht.entries ? lo - kc.vmin : 0;
+    ht.kmin = ht.entries ? int32_t(lo) : 0;
+    ht.capacity = ht.entries ? uint32_t(hi - lo + 1) : 0;
   }
   dev_free(c, ht.stage);  // the build has finished with it
   ht.stage = nullptr;
@@ -1979,8 +2070,7 @@ static dpf_status build_hash_async_impl(dpf_ctx* c, const dpf_build& B, void* st
     return st;
   }
   L.q = ht.bq;
-  L.sched = &ht.bstat->sched;
-  L.inserted = &ht.bstat->inserted;
+  L.stat = ht.bstat;
   L.nrows = bs.Q.nrows;
   L.page_rows = bs.Q.page_rows;
   L.host_data = bs.host;
@@ -2471,7 +2561,15 @@ dpf_status dpf_execute_plan(dpf_ctx* c, const dpf_plan* plans, int32_t n, void* 
   std::lock_guard<std::recursive_mutex> lk(c->mu);
   DeviceGuard g(c->device);
   Prep* p;
-  dpf_status st = prepare(c, plans, n, nullptr, &p);
+  // enqueued where the launch goes, unless that stream is being captured (the
+  // upload reads host memory of this call)
+  const cudaStream_t s = static_cast<cudaStream_t>(stream);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    cap = cudaStreamCaptureStatusActive;
+  }
+  dpf_status st = prepare(c, plans, n, nullptr, &p, cap == cudaStreamCaptureStatusNone ? &s : nullptr);
   if (st) return st;
   p->oneshot = true;
   st = dpf_launch(c, p->id, stream);

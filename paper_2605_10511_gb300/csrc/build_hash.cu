@@ -68,9 +68,9 @@ constexpr unsigned long long kEmptySlot = 0x0000000080000000ull;  // {INT32_MIN,
 // presence bits of a rank directory (a bit already set is a duplicate key)
 // and write {key offset, payload} to the staging list (a tile reserves one
 // slot per kept row with one atomic), from which rank_scatter places the
-// payloads once the ranks are known.  Modes 1-3
-// also add the rows they insert to L.inserted when it is set (a table sized
-// before its scan learns its entry count that way).
+// payloads once the ranks are known.  Every mode adds the rows it keeps to
+// L.stat and, with L.measure, their key range (a table sized before its scan
+// learns its entry count and range that way).
 template <bool kHost, int kMode>
 __global__ void __launch_bounds__(256) build_kernel(const DevQuery* __restrict__ qdev, BuildLaunch L,
                                                     unsigned int* status) {
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(256) build_kernel(const DevQuery* __restrict__
   const uint64_t npages = (Q.nrows + PR - 1) / PR;
   const uint64_t tiles_per_page = (PR / kMB + TB - 1) / TB;
   unsigned long long kept = 0;
-  int32_t kmin = INT32_MAX, kmax = INT32_MIN;
+  uint32_t hi = 0, lo = 0;  // the kept keys' range (BuildStat)
   for (uint64_t w = warp; w < npages * tiles_per_page; w += nwarps) {
     const uint64_t p = w / tiles_per_page;
     const uint32_t i0 = uint32_t(w % tiles_per_page) * TB;
@@ -122,8 +122,8 @@ __global__ void __launch_bounds__(256) build_kernel(const DevQuery* __restrict__
       if (!valid) continue;
       if (kMode == 0) {
         ++kept;
-        kmin = min(kmin, kv);
-        kmax = max(kmax, kv);
+        hi = max(hi, BuildStat::rank(kv));
+        lo = max(lo, ~BuildStat::rank(kv));
         continue;
       }
       // a rank build's slot of a row that inserts nothing holds a pair the
@@ -134,7 +134,11 @@ __global__ void __launch_bounds__(256) build_kernel(const DevQuery* __restrict__
         if (kMode == 3 && sslot < L.rank_cap) L.rank_stage[sslot] = make_uint2(0xffffffffu, 0u);
         continue;
       }
-      ++kept;  // rows inserted (read only when L.inserted is set)
+      ++kept;  // rows inserted
+      if (kMode == 2) {
+        hi = max(hi, BuildStat::rank(kv));
+        lo = max(lo, ~BuildStat::rank(kv));
+      }
       const uint32_t pay = (c0 & 0xffffu) | ((c1 & 0xffffu) << 16);
       if (kMode == 2 || kMode == 3) {
         const uint32_t off = uint32_t(kv) - uint32_t(L.kmin);
@@ -173,22 +177,16 @@ __global__ void __launch_bounds__(256) build_kernel(const DevQuery* __restrict__
     }
     __syncwarp();
   }
-  if (kMode == 0) {
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-      kept += __shfl_down_sync(kFull, kept, d);
-      kmin = min(kmin, __shfl_down_sync(kFull, kmin, d));
-      kmax = max(kmax, __shfl_down_sync(kFull, kmax, d));
-    }
+  for (int d = 16; d > 0; d >>= 1) kept += __shfl_down_sync(kFull, kept, d);
+  if (lane == 0 && kept) atomicAdd(&L.stat->inserted, kept);
+  if ((kMode == 0 || kMode == 2) && L.measure) {
+    hi = __reduce_max_sync(kFull, hi);
+    lo = __reduce_max_sync(kFull, lo);
     if (lane == 0 && kept) {
-      atomicAdd(L.count, kept);
-      atomicMin(L.kminmax, kmin);
-      atomicMax(L.kminmax + 1, kmax);
+      atomicMax(&L.stat->hi, hi);
+      atomicMax(&L.stat->lo, lo);
     }
-  } else if (L.inserted) {
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) kept += __shfl_down_sync(kFull, kept, d);
-    if (lane == 0 && kept) atomicAdd(L.inserted, kept);
   }
 }
 
@@ -294,8 +292,8 @@ int build_grid(uint64_t nrows, uint64_t page_rows) {
 template <int kMode>
 cudaError_t launch_build_mode(const BuildLaunch& L, cudaStream_t s) {
   const int g = build_grid(L.nrows, L.page_rows);
-  if (L.host_data) build_kernel<true, kMode><<<g, 256, 0, s>>>(L.q, L, &L.sched->status);
-  else build_kernel<false, kMode><<<g, 256, 0, s>>>(L.q, L, &L.sched->status);
+  if (L.host_data) build_kernel<true, kMode><<<g, 256, 0, s>>>(L.q, L, &L.stat->sched.status);
+  else build_kernel<false, kMode><<<g, 256, 0, s>>>(L.q, L, &L.stat->sched.status);
   return cudaGetLastError();
 }
 
@@ -312,7 +310,7 @@ cudaError_t launch_build_insert(const BuildLaunch& L, cudaStream_t s) {
     rank_fill<<<nblocks, 256, 0, s>>>(L.rank_dir, nwords, L.rank_sums);
     const int g = int(tmax<uint32_t>(1u, tmin<uint32_t>((L.rank_cap + 255) / 256, 2048u)));
     rank_scatter<<<g, 256, 0, s>>>(L.rank_dir, L.rank_stage, L.stage_n, L.rank_pay, L.rank_cap, L.krange,
-                                   &L.sched->status);
+                                   &L.stat->sched.status);
     return cudaGetLastError();
   }
   return L.direct ? launch_build_mode<2>(L, s) : launch_build_mode<1>(L, s);

@@ -506,8 +506,8 @@ template <bool kHost, int kMinBlocks, bool kText, bool kStage = false, int kThre
 __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQuery* __restrict__ queries,
                                                        const uint64_t* __restrict__ qbegin, int nq,
                                                        uint64_t owned, uint64_t pool, Sched* sched,
-                                                       uint32_t acc_slots, uint32_t tables_bytes,
-                                                       uint32_t stage_bw) {
+                                                       unsigned int* status_out, uint32_t acc_slots,
+                                                       uint32_t tables_bytes, uint32_t stage_bw) {
   __shared__ CtaState cs;
   uint32_t* sacc = shared_acc();
   uint8_t* stab = dyn + ((acc_slots * sizeof(unsigned long long) + 15) & ~size_t(15));
@@ -593,6 +593,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
     if (old == gridDim.x - 1) {
       sched->next = 0ull;
       sched->exited = 0u;
+      if (status_out) *status_out = atomicOr(&sched->status, 0u);  // every other CTA has left
       __threadfence();
     }
   }
@@ -614,7 +615,7 @@ cudaError_t launch_as(const FusedLaunch& L, size_t smem, uint32_t tb, cudaStream
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   k<<<L.grid, L.threads, smem, s>>>(
-      L.queries, L.qbegin, L.nq, L.owned, L.pool, L.sched, L.acc_slots, tb, L.stage_bw);
+      L.queries, L.qbegin, L.nq, L.owned, L.pool, L.sched, L.status_out, L.acc_slots, tb, L.stage_bw);
   return cudaGetLastError();
 }
 

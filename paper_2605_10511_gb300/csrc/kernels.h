@@ -39,6 +39,7 @@ constexpr int32_t kDefaultGroupAgg = 2;
 // directory (2 bits per key plus the kept payloads) up to 2^28 keys, open
 // addressing beyond.
 constexpr uint64_t kDirectMaxRange = uint64_t(1) << 22;
+constexpr uint64_t kDirectAlways = uint64_t(1) << 20;  // direct however few rows are kept
 constexpr uint64_t kRankMaxRange = uint64_t(1) << 28;
 // Shared-memory bytes of the code-level matcher tables of a PREFIX / CONTAINS
 // step with a pattern of plen bytes on an FSST column: for every matcher
@@ -61,6 +62,7 @@ struct FusedLaunch {
   int nq;
   uint64_t owned, pool;
   Sched* sched;
+  unsigned int* status_out;   // where the launch leaves its status word too (mapped host memory; or nullptr)
   int grid, threads;
   uint32_t acc_slots;   // int64 shared accumulators per CTA (max over the batch)
   size_t smem_tables;   // bytes of the CTA's join-table region
@@ -92,18 +94,21 @@ struct BuildLaunch {
   uint2* rank_stage;          //   scratch: {key offset, payload} of each inserted row, in insertion order
   unsigned long long* stage_n;  //   its count
   uint32_t rank_cap;          //   payload words (= staged pairs) the table holds
-  unsigned long long* count;  // device counter (count pass)
-  int32_t* kminmax;           // device {min, max} of kept keys (count pass)
-  unsigned long long* inserted;  // tables sized before the scan: rows the insert pass kept (or nullptr)
-  Sched* sched;               // status word
+  struct BuildStat* stat;     // status word and rows kept by the pass
+  bool measure;               // the pass also records the kept keys' range
   uint64_t nrows, page_rows;
   bool host_data;
 };
-// Device-side outcome of a table sized before its scan: the build kernels'
-// status bits and the rows the insert pass kept.
+// Device-side outcome of a build pass: its status bits, the rows it kept
+// (inserted, or counted) and their key range, kept by
+// atomicMax from zero bytes on: the largest rank(key), and the largest ~rank.
 struct BuildStat {
   Sched sched;
   unsigned long long inserted;
+  uint32_t hi, lo;
+  __host__ __device__ static uint32_t rank(int32_t key) { return uint32_t(key) ^ 0x80000000u; }
+  __host__ __device__ int32_t key_hi() const { return int32_t(hi ^ 0x80000000u); }
+  __host__ __device__ int32_t key_lo() const { return int32_t(~lo ^ 0x80000000u); }
 };
 cudaError_t launch_build_count(const BuildLaunch& L, cudaStream_t s);
 cudaError_t launch_build_insert(const BuildLaunch& L, cudaStream_t s);
