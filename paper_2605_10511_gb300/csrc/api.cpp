@@ -1064,13 +1064,16 @@ size_t place_tables(DevQuery& Q, size_t budget, bool first_only) {
     DevStep& S = Q.steps[s];
     if (S.kind != ST_PROBE) continue;
     S.smem_width = 0;
+    S.present = 0;
     if (first_only && s != 0) continue;
     if (S.ht_kind == HT_RANK) continue;  // probed in device memory (L2) only
-    const uint32_t w = S.ht_kind == HT_DIRECT ? width : 8u;
-    const size_t bytes = S.ht_kind == HT_DIRECT ? size_t(S.krange) * w : size_t(S.ht_mask + 1) * 8;
+    const bool present = s == 0 && S.ht_kind == HT_DIRECT && (S.mul0 | S.mul1) == 0;
+    const uint32_t w = present ? 1u : S.ht_kind == HT_DIRECT ? width : 8u;
+    const size_t bytes = S.ht_kind == HT_DIRECT ? size_t(S.krange) * w + present : size_t(S.ht_mask + 1) * 8;
     const size_t at = (used + 15) & ~size_t(15);
     if (at + bytes > budget) continue;
     S.smem_width = uint8_t(w);
+    S.present = present;
     S.smem_off = uint32_t(at);
     used = at + bytes;
   }

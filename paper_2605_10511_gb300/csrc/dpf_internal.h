@@ -117,7 +117,8 @@ struct DevStep {
                           // group-id contribution (all ones = absent);
                           // PREFIX / CONTAINS on an FSST column: 1 = the
                           // step's code-level matcher tables sit at smem_off
-  uint16_t pad_;
+  uint8_t present;        // smem_width 1: a byte per key and one more, 1 = present (PM_PRESENT)
+  uint8_t pad_;
   uint32_t smem_off;      // byte offset of the copy in the CTA's table region
   uint32_t mul0, mul1;    // gid multipliers of payload fields 0 and 1 (0 = unused)
   // Values a row needs to pass (a superset: [zlo, zhi] empty when nothing

@@ -468,8 +468,8 @@ __device__ void process_ticket(const DevQuery& Q, uint64_t chunk, const uint8_t*
 
 // Copies a query's shared-memory join tables into the CTA's table region:
 // open-addressing slots as they are, direct tables as 1/2/4-byte group-id
-// contributions (all ones = absent); builds the code-level matcher tables
-// of string steps on FSST columns.
+// contributions (all ones = absent) or presence bytes; builds the code-level
+// matcher tables of string steps on FSST columns.
 __device__ void load_smem_tables(const DevQuery& Q, uint8_t* stab) {
   for (uint32_t s = 0; s < Q.nsteps; ++s) {
     const DevStep& S = Q.steps[s];
@@ -485,6 +485,11 @@ __device__ void load_smem_tables(const DevQuery& Q, uint8_t* stab) {
       continue;
     }
     const uint32_t* src = static_cast<const uint32_t*>(S.ht);
+    if (S.present) {
+      for (uint32_t i = threadIdx.x; i <= S.krange; i += blockDim.x)
+        stab[S.smem_off + i] = i < S.krange && __ldg(src + i) != kAbsent ? 1 : 0;
+      continue;
+    }
     for (uint32_t i = threadIdx.x; i < S.krange; i += blockDim.x) {
       const uint32_t e = __ldg(src + i);
       const uint32_t c = (e & 0xffffu) * S.mul0 + (e >> 16) * S.mul1;

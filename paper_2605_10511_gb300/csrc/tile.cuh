@@ -232,11 +232,13 @@ __device__ __forceinline__ void tile_init(const PageState& P, uint32_t i0, uint3
 // = value of row 32k + lane of mini block t (the payload words are loaded
 // into v and decoded in place).  anym bit t = mini block t was decoded.
 // Specialised on the codec (FOR/DICT/STR lengths vs DELTA) so the unrolled
-// loops carry no per-value branch on it.
+// loops carry no per-value branch on it.  bias is added to every value (once,
+// to the mini block's base).
 template <bool kHost, bool kDelta, bool kStaged = false>
 __device__ __forceinline__ void decode_t(const DevQuery& Q, int c, const PageState& P, const TileHdr& Hd,
                                          uint32_t alive, int lane, uint32_t (&v)[TB][4], uint32_t& anym,
-                                         unsigned int* status, StagedPay sp = StagedPay{nullptr, 0, 0}) {
+                                         unsigned int* status, StagedPay sp = StagedPay{nullptr, 0, 0},
+                                         uint32_t bias = 0) {
   const uint8_t* pg = reinterpret_cast<const uint8_t*>(__shfl_sync(kFull, P.pg, c));
   const uint32_t* pay = reinterpret_cast<const uint32_t*>(pg + payload_offset(Q.cols[c].codec, P.prow));
   uint32_t hx[TB], hy[TB];
@@ -244,7 +246,7 @@ __device__ __forceinline__ void decode_t(const DevQuery& Q, int c, const PageSta
 #pragma unroll
   for (int t = 0; t < TB; ++t) {
     bool any = __any_sync(kFull, (alive >> (4 * t)) & 15u) != 0;
-    hx[t] = __shfl_sync(kFull, Hd.x, c * TB + t);
+    hx[t] = __shfl_sync(kFull, Hd.x, c * TB + t) + bias;
     hy[t] = __shfl_sync(kFull, kDelta ? Hd.z : Hd.y, c * TB + t);
     const uint32_t bw = hy[t] & 0xffu;
     if (any && bw > 32) {
@@ -757,7 +759,43 @@ __device__ __forceinline__ void tile_prefix(const DevQuery& Q, const DevStep& S,
   const uint8_t* bytes = pg + __shfl_sync(kFull, P.extra, S.col);
   const int4* sym = Q.cols[S.col].codec == C_FSST ? Q.cols[S.col].sym : nullptr;
   const uint8_t* tab = sym != nullptr && S.smem_width ? stab + S.smem_off : nullptr;
-  const bool lockstep = S.kind == ST_PREFIX && sym == nullptr;
+  if (S.kind == ST_PREFIX && sym == nullptr) {
+    // raw PREFIX: the warp compares byte i of all its rows' strings at once;
+    // a length that is long enough gives way to its string's offset
+    const uint32_t plen = S.plen;
+    uint32_t match = 0;
+#pragma unroll
+    for (int t = 0; t < TB; ++t) {
+      if (!((anym >> t) & 1u)) continue;
+      uint32_t st[4];
+      excl_scan128(len[t], lane, st);
+      const uint32_t mb_start = __shfl_sync(kFull, Hd.sstart, S.col * TB + t);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        match |= uint32_t(len[t][k] >= plen) << (4 * t + k);
+        len[t][k] = mb_start + st[k];
+      }
+    }
+    match &= T.alive;
+    for (uint32_t i = 0; i < plen; ++i) {
+      if (!__any_sync(kFull, match != 0)) break;
+      const uint8_t want = S.pfx[i];
+      uint32_t b[TB][4];
+#pragma unroll
+      for (int t = 0; t < TB; ++t)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          b[t][k] = ((match >> (4 * t + k)) & 1u) ? uint32_t(ld_u8<kHost>(bytes + (uint64_t(len[t][k]) + i))) : 256u;
+      uint32_t same = 0;
+#pragma unroll
+      for (int t = 0; t < TB; ++t)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) same |= uint32_t(b[t][k] == want) << (4 * t + k);
+      match &= same;
+    }
+    T.alive &= match;
+    return;
+  }
   uint32_t* queue = search + kSearchHits;
   uint32_t* result = queue + 3 * kLikeQueue;
   uint32_t waiting = 0;
@@ -780,46 +818,28 @@ __device__ __forceinline__ void tile_prefix(const DevQuery& Q, const DevStep& S,
     const uint32_t mb_start = __shfl_sync(kFull, Hd.sstart, S.col * TB + t);
     const uint8_t* mb = bytes + mb_start;
     uint32_t match = 0;
-    if (lockstep) {
-      // raw PREFIX: the warp compares byte i of all its rows' strings at once
-      const uint32_t plen = S.plen;
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (((T.alive >> (4 * t + k)) & 1u) && len[t][k] >= plen) match |= 1u << k;
-      for (uint32_t i = 0; i < plen; ++i) {
-        if (!__any_sync(kFull, match)) break;
-        const uint8_t want = S.pfx[i];
-        uint8_t b[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) b[k] = ((match >> k) & 1u) ? ld_u8<kHost>(mb + st[k] + i) : want;
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (b[k] != want) match &= ~(1u << k);
-      }
-    } else {
-      if constexpr (kText) {
-        if (coop) {
-          const uint32_t live = (T.alive >> (4 * t)) & 15u;
-          const uint4 st4 = make_uint4(st[0], st[1], st[2], st[3]);
-          const uint4 len4 = make_uint4(len[t][0], len[t][1], len[t][2], len[t][3]);
-          if (S.kind == ST_CONTAINS) {
-            match = sym != nullptr ? search_mb<kHost, true>(mb, st4, len4, S.pfx, S.plen, tab, search, lane)
-                                   : search_mb<kHost, false>(mb, st4, len4, S.pfx, S.plen, nullptr, search, lane);
-          } else {
-            const uint32_t run = uint32_t(S.in[1]);
-            match = run == 0 ? live
-                             : search_mb<kHost, false>(mb, st4, len4, S.pfx + S.in[0], run, nullptr, search, lane);
-            waiting = like_push<kHost>(S, bytes, mb_start, st, len[t], match & live, t, queue, result, waiting, lane);
-          }
+    if constexpr (kText) {
+      if (coop) {
+        const uint32_t live = (T.alive >> (4 * t)) & 15u;
+        const uint4 st4 = make_uint4(st[0], st[1], st[2], st[3]);
+        const uint4 len4 = make_uint4(len[t][0], len[t][1], len[t][2], len[t][3]);
+        if (S.kind == ST_CONTAINS) {
+          match = sym != nullptr ? search_mb<kHost, true>(mb, st4, len4, S.pfx, S.plen, tab, search, lane)
+                                 : search_mb<kHost, false>(mb, st4, len4, S.pfx, S.plen, nullptr, search, lane);
         } else {
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (((T.alive >> (4 * t + k)) & 1u) && string_match<kHost>(S, mb + st[k], len[t][k], sym, tab))
-              match |= 1u << k;
+          const uint32_t run = uint32_t(S.in[1]);
+          match = run == 0 ? live
+                           : search_mb<kHost, false>(mb, st4, len4, S.pfx + S.in[0], run, nullptr, search, lane);
+          waiting = like_push<kHost>(S, bytes, mb_start, st, len[t], match & live, t, queue, result, waiting, lane);
         }
       } else {
-        if (lane == 0) atomicOr(status, S_INTERNAL);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (((T.alive >> (4 * t + k)) & 1u) && string_match<kHost>(S, mb + st[k], len[t][k], sym, tab))
+            match |= 1u << k;
       }
+    } else {
+      if (lane == 0) atomicOr(status, S_INTERNAL);
     }
     T.alive &= ~((~match & 15u) << (4 * t));
   }
@@ -838,9 +858,13 @@ __device__ __forceinline__ void tile_prefix(const DevQuery& Q, const DevStep& S,
 
 // Probe modes: direct table copied into shared memory as 1/2/4-byte group-id
 // contributions, direct or rank-directory table in global memory, open
-// addressing (shared or global slots).
-enum ProbeMode : int { PM_S1 = 0, PM_S2 = 1, PM_S4 = 2, PM_GDIRECT = 3, PM_OPEN = 4 };
+// addressing (shared or global slots); and, for a first step that adds no
+// contribution, a direct table copied as one byte per key, 1 = present, with a
+// 0 behind the last key: a row's bit is then the byte at the smaller of its
+// key offset and the table's size, with no test of bounds or of absence.
+enum ProbeMode : int { PM_S1 = 0, PM_S2 = 1, PM_S4 = 2, PM_GDIRECT = 3, PM_OPEN = 4, PM_PRESENT = 9 };
 __device__ __forceinline__ int probe_mode(const DevStep& S) {
+  if (S.present) return PM_PRESENT;
   if (S.ht_kind == HT_OPEN) return PM_OPEN;
   return S.smem_width == 1 ? PM_S1 : S.smem_width == 2 ? PM_S2 : S.smem_width == 4 ? PM_S4 : PM_GDIRECT;
 }
@@ -1046,7 +1070,7 @@ __device__ __forceinline__ bool staged_mb_decode(const TileHdr& Hd, int c, int t
 
 // The step's test on the four values of mini block t: bits k of the result
 // = row 32k + lane passes (and, with kGid, its group-id contribution added).
-// kOp 0..4 = probe modes, 5 = group key, 6 = RANGE, 7 = NOTRANGE, 8 = IN.
+// kOp 0..4, 9 = probe modes, 5 = group key, 6 = RANGE, 7 = NOTRANGE, 8 = IN.
 template <int kOp, bool kGid>
 __device__ __forceinline__ uint32_t staged_mb_test(const DevStep& S, const uint8_t* stab, const uint32_t (&v)[4],
                                                    uint32_t live, uint32_t (&gid)[4], unsigned int* status) {
@@ -1087,6 +1111,10 @@ __device__ __forceinline__ uint32_t staged_mb_test(const DevStep& S, const uint8
 #pragma unroll
       for (int k = 0; k < 4; ++k) gid[k] += (pay[k] & 0xffffu) * S.mul0 + (pay[k] >> 16) * S.mul1;
     }
+  } else if (kOp == PM_PRESENT) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      keep |= uint32_t(stab[S.smem_off + tmin<uint32_t>(v[k] - uint32_t(S.kmin), S.krange)]) << k;
   } else if (kOp == 5) {
     if (kGid) {
 #pragma unroll
@@ -1134,6 +1162,7 @@ __device__ __forceinline__ void dense_step_t(const DevQuery& Q, const DevStep& S
     switch (S.kind) {
       case ST_PROBE:
         switch (probe_mode(S)) {
+          case PM_PRESENT: staged_dense<kDelta, false, PM_PRESENT>(S, Hd, T, stab, sp, lane, status); break;
           case PM_S1: staged_dense<kDelta, kGid, PM_S1>(S, Hd, T, stab, sp, lane, status); break;
           case PM_S2: staged_dense<kDelta, kGid, PM_S2>(S, Hd, T, stab, sp, lane, status); break;
           case PM_S4: staged_dense<kDelta, kGid, PM_S4>(S, Hd, T, stab, sp, lane, status); break;
@@ -1155,10 +1184,25 @@ __device__ __forceinline__ void dense_step_t(const DevQuery& Q, const DevStep& S
   }
   uint32_t v[TB][4];
   uint32_t anym;
-  decode_t<kHost, kDelta, kStaged>(Q, S.col, P, Hd, T.alive, lane, v, anym, status, sp);
+  // lo <= x <= hi  <=>  (x - lo) <= (hi - lo) as unsigned; a presence table is
+  // indexed from its smallest key: the subtraction is the decode's bias
+  const bool range = S.kind == ST_RANGE || S.kind == ST_NOTRANGE;
+  const uint32_t bias = range ? 0u - uint32_t(S.lo) : S.kind == ST_PROBE && S.present ? 0u - uint32_t(S.kmin) : 0u;
+  decode_t<kHost, kDelta, kStaged>(Q, S.col, P, Hd, T.alive, lane, v, anym, status, sp, bias);
   switch (S.kind) {
     case ST_PROBE:
       switch (probe_mode(S)) {
+        case PM_PRESENT: {  // mini blocks that were not decoded have no live row
+          const uint8_t* tab = stab + S.smem_off;
+          const uint32_t top = S.krange;
+          uint32_t keep = 0;
+#pragma unroll
+          for (int t = 0; t < TB; ++t)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) keep |= uint32_t(tab[tmin<uint32_t>(v[t][k], top)]) << (4 * t + k);
+          T.alive &= keep;
+          break;
+        }
         case PM_S1: dense_probe<PM_S1, kGid>(S, stab, v, anym, T, status); break;
         case PM_S2: dense_probe<PM_S2, kGid>(S, stab, v, anym, T, status); break;
         case PM_S4: dense_probe<PM_S4, kGid>(S, stab, v, anym, T, status); break;
@@ -1187,15 +1231,13 @@ __device__ __forceinline__ void dense_step_t(const DevQuery& Q, const DevStep& S
       return;
     case ST_RANGE:
     case ST_NOTRANGE: {
-      const bool neg = S.kind == ST_NOTRANGE;
-      // lo <= x <= hi  <=>  (x - lo) <= (hi - lo) as unsigned
-      const uint32_t lo = uint32_t(S.lo), span = uint32_t(S.hi) - uint32_t(S.lo);
+      const uint32_t span = uint32_t(S.hi) - uint32_t(S.lo);
       uint32_t keep = 0;
 #pragma unroll
       for (int t = 0; t < TB; ++t)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) keep |= uint32_t(((v[t][k] - lo) <= span) != neg) << (4 * t + k);
-      T.alive &= keep;
+        for (int k = 0; k < 4; ++k) keep |= uint32_t(v[t][k] <= span) << (4 * t + k);
+      T.alive &= S.kind == ST_NOTRANGE ? ~keep : keep;
       return;
     }
     default: {  // IN (FALSE compiles to IN with an empty list)
