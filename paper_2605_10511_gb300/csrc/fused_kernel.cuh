@@ -137,8 +137,9 @@ __device__ void finish_query(const DevQuery& Q, uint32_t mine, CtaState& cs) {
   __syncthreads();
 }
 
-// The accumulators a warp adds to: the CTA's shared ones, or the query's
-// global int64 ones when the domain does not fit.  A shared
+// One accumulator slot of the groups that a warp adds to, in registers (taken
+// once before a list's rounds, like PointCol): the CTA's shared accumulators,
+// or the query's global int64 ones when the domain does not fit.  A shared
 // int64 accumulator is kept as two 32-bit halves, all low halves first
 // (slot-major: slot * domain + group, so that neighbouring groups lie in
 // different banks), then all high halves.  32-bit shared atomics are done by
@@ -146,16 +147,24 @@ __device__ void finish_query(const DevQuery& Q, uint32_t mine, CtaState& cs) {
 // a 64-bit one is a compare-and-swap loop that repeats for each of them.  An
 // add needs the high half only when it carries (or the value itself has high
 // bits), so most adds are one 32-bit atomic; the sum is exact modulo 2^64.
-__device__ __forceinline__ void acc_add(const DevQuery& Q, uint32_t gid, uint32_t slot, unsigned long long x) {
-  if (!Q.use_smem_acc) {
-    atomicAdd(Q.acc + uint64_t(gid) * (1 + Q.naggs) + slot, x);
+struct AccSlot {
+  unsigned long long* g;       // global accumulators of the slot, a group every `slots`
+  uint32_t at, to_hi, slots;   // shared: index of the slot's group 0; distance to the high halves
+  bool shared, warp;           // warp: warp-aggregated updates
+  __device__ __forceinline__ AccSlot(const DevQuery& Q, uint32_t slot)
+      : g(Q.acc + slot), at(slot * Q.domain), to_hi(Q.domain * (1 + Q.naggs)), slots(1 + Q.naggs),
+        shared(Q.use_smem_acc != 0), warp(Q.warp_agg != 0) {}
+};
+__device__ __forceinline__ void acc_add(const AccSlot& A, uint32_t gid, unsigned long long x) {
+  if (!A.shared) {
+    atomicAdd(A.g + uint64_t(gid) * A.slots, x);
     return;
   }
-  uint32_t* p = shared_acc() + slot * Q.domain + gid;
+  uint32_t* p = shared_acc() + A.at + gid;
   const uint32_t lo = uint32_t(x);
   const uint32_t old = atomicAdd(p, lo);
   const uint32_t hi = uint32_t(x >> 32) + uint32_t(old + lo < lo);
-  if (hi) atomicAdd(p + Q.domain * (1 + Q.naggs), hi);
+  if (hi) atomicAdd(p + A.to_hi, hi);
 }
 
 // Warp-aggregated group-by update (hash aggregation of Kernel #3, Sec. 3.1),
@@ -169,8 +178,8 @@ __device__ __forceinline__ void acc_add(const DevQuery& Q, uint32_t gid, uint32_
 // the 64-bit value; otherwise the value is an int32, whose low 16 bits and
 // signed high 16 bits are summed).  Warp-uniform call.
 template <bool kWide>
-__device__ __forceinline__ void lead_group_add(const DevQuery& Q, uint32_t gid, uint32_t slot, unsigned long long x,
-                                               bool valid, int lane) {
+__device__ __forceinline__ void lead_group_add(const AccSlot& A, uint32_t gid, unsigned long long x, bool valid,
+                                               int lane) {
   const uint32_t vm = __ballot_sync(kFull, valid);
   if (vm == 0) return;
   const int lead = __ffs(vm) - 1;
@@ -191,68 +200,70 @@ __device__ __forceinline__ void lead_group_add(const DevQuery& Q, uint32_t gid, 
       const int32_t s_hi = int32_t(__reduce_add_sync(m, uint32_t(v >> 16)));  // |sum| < 2^20
       t = (unsigned long long)((long long)s_lo + (long long)s_hi * 65536ll);
     }
-    if (lane == lead) acc_add(Q, g0, slot, t);
+    if (lane == lead) acc_add(A, g0, t);
   } else if (valid) {
-    acc_add(Q, gid, slot, x);
+    acc_add(A, gid, x);
   }
 }
 
-// A grouped update: warp-aggregated by the leading group (Q.warp_agg) or one
-// atomic per row.
+// A grouped update: warp-aggregated by the leading group or one atomic per row.
 template <bool kWide>
-__device__ __forceinline__ void group_add(const DevQuery& Q, uint32_t gid, uint32_t slot,
-                                          unsigned long long x, bool valid, int lane) {
-  if (Q.warp_agg) lead_group_add<kWide>(Q, gid, slot, x, valid, lane);
-  else if (valid) acc_add(Q, gid, slot, x);
+__device__ __forceinline__ void group_add(const AccSlot& A, uint32_t gid, unsigned long long x, bool valid, int lane) {
+  if (A.warp) lead_group_add<kWide>(A, gid, x, valid, lane);
+  else if (valid) acc_add(A, gid, x);
+}
+
+// Adds a warp's per-lane sums (an ungrouped aggregate) to group 0.
+__device__ __forceinline__ void single_add(const AccSlot& A, unsigned long long sum, int lane) {
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) sum += __shfl_down_sync(kFull, sum, d);
+  if (lane == 0 && sum != 0) acc_add(A, 0, sum);
+}
+
+// Group id of a list entry, and whether the row takes part: a group id beyond
+// the domain is a corrupt dictionary code, which drops the row.
+__device__ __forceinline__ uint32_t entry_group(uint32_t e, uint32_t domain, bool& valid, unsigned int* status) {
+  const uint32_t gid = e >> kRowBits;
+  if (valid && gid >= domain) {
+    atomicOr(status, S_CORRUPT);
+    valid = false;
+  }
+  return gid;
 }
 
 // One aggregate over a warp's list, specialised on its operation (dpf_agg_op)
 // and on how its operands are read: kPoint = FOR/DICT columns, one bit field
 // per row; otherwise any codec through row_value (DELTA decodes densely).
+// count: the pass counts the rows too (slot 0), which saves a pass of its own.
 template <bool kHost, int kOp, bool kPoint>
 __device__ __forceinline__ void agg_pass(const DevQuery& Q, const PageState& P, uint32_t seg_mb,
-                                         const uint32_t* list, uint32_t n, int lane,
-                                         uint32_t slot, int ca, int cb, bool single, unsigned int* status) {
-  constexpr int U = kPoint ? kListUnroll : 1;  // rounds whose loads are issued together
+                                         const uint32_t* list, uint32_t n, int lane, uint32_t slot, int ca, int cb,
+                                         bool single, bool count, unsigned int* status) {
+  constexpr bool kTwo = kOp == DPF_AGG_SUM_MUL || kOp == DPF_AGG_SUM_SUB;
+  const AccSlot A(Q, slot);
+  const uint32_t domain = Q.domain;
+  const PointCol Ca = point_col(Q, ca, P, seg_mb), Cb = kTwo ? point_col(Q, cb, P, seg_mb) : Ca;
   long long sum = 0;
-  for (uint32_t i0 = 0; i0 < n; i0 += 32 * U) {
-    uint32_t r[U], gid[U];
-    bool valid[U];
-    int32_t va[U], vb[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      valid[u] = i0 + 32u * u + lane < n;
-      const uint32_t e = valid[u] ? list[i0 + 32u * u + lane] : 0u;
-      r[u] = e & ((1u << kRowBits) - 1u);
-      gid[u] = e >> kRowBits;
-      if (!single && gid[u] >= Q.domain) valid[u] = false;  // reported by list_aggregate
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      va[u] = vb[u] = 0;
-      va[u] = int32_t(kPoint ? point_value<kHost>(Q, ca, P, seg_mb, r[u], valid[u])
-                             : row_value<kHost>(Q, ca, P, seg_mb, r[u], valid[u], lane, status));
-      if (kOp == DPF_AGG_SUM_MUL || kOp == DPF_AGG_SUM_SUB)
-        vb[u] = int32_t(kPoint ? point_value<kHost>(Q, cb, P, seg_mb, r[u], valid[u])
-                               : row_value<kHost>(Q, cb, P, seg_mb, r[u], valid[u], lane, status));
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      long long x = va[u];
-      if (kOp == DPF_AGG_SUM_MUL)
-        x = (long long)((unsigned long long)(long long)va[u] * (unsigned long long)(long long)vb[u]);
-      else if (kOp == DPF_AGG_SUM_SUB)
-        x = (long long)va[u] - (long long)vb[u];
-      if (single) sum += valid[u] ? x : 0;
-      else group_add<kOp == DPF_AGG_SUM_MUL || kOp == DPF_AGG_SUM_SUB>(Q, gid[u], slot,
-                                                                      (unsigned long long)x, valid[u], lane);
-    }
+  for (uint32_t i0 = 0; i0 < n; i0 += 32) {
+    bool valid = i0 + lane < n;
+    const uint32_t e = valid ? list[i0 + lane] : 0u;
+    const uint32_t r = e & ((1u << kRowBits) - 1u);
+    const uint32_t gid = entry_group(e, domain, valid, status);
+    if (count && valid) atomicAdd(shared_acc() + gid, 1u);
+    const int32_t va = int32_t(kPoint ? point_at<kHost>(Ca, r)
+                                      : row_value<kHost>(Q, ca, P, seg_mb, r, valid, lane, status));
+    int32_t vb = 0;
+    if (kTwo)
+      vb = int32_t(kPoint ? point_at<kHost>(Cb, r) : row_value<kHost>(Q, cb, P, seg_mb, r, valid, lane, status));
+    long long x = va;
+    if (kOp == DPF_AGG_SUM_MUL)
+      x = (long long)((unsigned long long)(long long)va * (unsigned long long)(long long)vb);
+    else if (kOp == DPF_AGG_SUM_SUB)
+      x = (long long)va - (long long)vb;
+    if (single) sum += valid ? x : 0;
+    else group_add<kTwo>(A, gid, (unsigned long long)x, valid, lane);
   }
-  if (single) {
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) sum += __shfl_down_sync(kFull, sum, d);
-    if (lane == 0 && sum != 0) acc_add(Q, 0, slot, (unsigned long long)sum);
-  }
+  if (single) single_add(A, (unsigned long long)sum, lane);
 }
 
 // An aggregate with a FOR64 operand: one survivor per lane, int64 operands,
@@ -261,40 +272,39 @@ __device__ __forceinline__ void agg_pass(const DevQuery& Q, const PageState& P, 
 // allocation as it was.
 template <bool kHost, int kOp>
 __device__ __forceinline__ void agg_pass_wide(const DevQuery& Q, const PageState& P, uint32_t seg_mb,
-                                           const uint32_t* list, uint32_t n, int lane,
-                                           uint32_t slot, int ca, int cb, bool single, unsigned int* status) {
+                                           const uint32_t* list, uint32_t n, int lane, uint32_t slot, int ca, int cb,
+                                           bool single, bool count, unsigned int* status) {
+  const AccSlot A(Q, slot);
+  const uint32_t domain = Q.domain;
   unsigned long long sum = 0;
   for (uint32_t i0 = 0; i0 < n; i0 += 32) {
     bool valid = i0 + lane < n;
     const uint32_t e = valid ? list[i0 + lane] : 0u;
-    const uint32_t r = e & ((1u << kRowBits) - 1u), gid = e >> kRowBits;
-    if (!single && gid >= Q.domain) valid = false;  // reported by list_aggregate
+    const uint32_t r = e & ((1u << kRowBits) - 1u);
+    const uint32_t gid = entry_group(e, domain, valid, status);
+    if (count && valid) atomicAdd(shared_acc() + gid, 1u);
     const unsigned long long a = (unsigned long long)value64<kHost>(Q, ca, P, seg_mb, r, valid, lane, status);
     unsigned long long b = 0;
     if (kOp == DPF_AGG_SUM_MUL || kOp == DPF_AGG_SUM_SUB)
       b = (unsigned long long)value64<kHost>(Q, cb, P, seg_mb, r, valid, lane, status);
     const unsigned long long x = kOp == DPF_AGG_SUM ? a : (kOp == DPF_AGG_SUM_MUL ? a * b : a - b);
     if (single) sum += valid ? x : 0ull;
-    else group_add<true>(Q, gid, slot, x, valid, lane);
+    else group_add<true>(A, gid, x, valid, lane);
   }
-  if (single) {
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) sum += __shfl_down_sync(kFull, sum, d);
-    if (lane == 0 && sum != 0) acc_add(Q, 0, slot, sum);
-  }
+  if (single) single_add(A, sum, lane);
 }
 
 template <bool kHost, int kOp>
 __device__ __forceinline__ void agg_dispatch(const DevQuery& Q, const PageState& P, uint32_t seg_mb,
-                                             const uint32_t* list, uint32_t n, int lane,
-                                             uint32_t slot, int ca, int cb, bool single, unsigned int* status) {
+                                             const uint32_t* list, uint32_t n, int lane, uint32_t slot, int ca, int cb,
+                                             bool single, bool count, unsigned int* status) {
   if (Q.cols[ca].codec == C_FOR64 || (kOp != DPF_AGG_SUM && Q.cols[cb].codec == C_FOR64)) {
-    agg_pass_wide<kHost, kOp>(Q, P, seg_mb, list, n, lane, slot, ca, cb, single, status);
+    agg_pass_wide<kHost, kOp>(Q, P, seg_mb, list, n, lane, slot, ca, cb, single, count, status);
     return;
   }
   const bool point = Q.cols[ca].codec != C_DELTA && (kOp == DPF_AGG_SUM || Q.cols[cb].codec != C_DELTA);
-  if (point) agg_pass<kHost, kOp, true>(Q, P, seg_mb, list, n, lane, slot, ca, cb, single, status);
-  else agg_pass<kHost, kOp, false>(Q, P, seg_mb, list, n, lane, slot, ca, cb, single, status);
+  if (point) agg_pass<kHost, kOp, true>(Q, P, seg_mb, list, n, lane, slot, ca, cb, single, count, status);
+  else agg_pass<kHost, kOp, false>(Q, P, seg_mb, list, n, lane, slot, ca, cb, single, count, status);
 }
 
 // Aggregation over a warp's survivor list (Kernel #3 hash aggregation;
@@ -309,36 +319,42 @@ __device__ __forceinline__ void list_aggregate(const DevQuery& Q, const PageStat
                                                const uint32_t* list, uint32_t n, int lane,
                                                unsigned int* status) {
   const bool single = Q.domain == 1;
+  bool count = false;  // the next aggregate's pass counts the rows too
   if (single) {
-    if (lane == 0) acc_add(Q, 0, 0, (unsigned long long)n);
+    if (lane == 0) acc_add(AccSlot(Q, 0), 0, (unsigned long long)n);
   } else {
-    // a shared count needs no high half while the table has fewer than 2^32 rows
-    const bool narrow = Q.use_smem_acc && (Q.nrows >> 32) == 0 && !Q.warp_agg;
-    for (uint32_t i0 = 0; i0 < n; i0 += 32) {
-      bool valid = i0 + lane < n;
-      const uint32_t gid = valid ? list[i0 + lane] >> kRowBits : 0u;
-      if (valid && gid >= Q.domain) {
-        atomicOr(status, S_CORRUPT);  // a corrupt dictionary code
-        valid = false;
+    // a shared count needs no high half while the table has fewer than 2^32
+    // rows: then the first aggregate's pass makes it
+    bool other = false;
+    for (uint32_t a = 0; a < Q.naggs; ++a) other = other || Q.agg_op[a] != DPF_AGG_COUNT;
+    count = Q.use_smem_acc && (Q.nrows >> 32) == 0 && !Q.warp_agg;
+    if (!count || !other) {
+      const AccSlot A(Q, 0);
+      const uint32_t domain = Q.domain;
+      for (uint32_t i0 = 0; i0 < n; i0 += 32) {
+        bool valid = i0 + lane < n;
+        const uint32_t gid = entry_group(valid ? list[i0 + lane] : 0u, domain, valid, status);
+        if (!count) group_add<false>(A, gid, 1ull, valid, lane);
+        else if (valid) atomicAdd(shared_acc() + gid, 1u);
       }
-      if (!narrow) group_add<false>(Q, gid, 0, 1ull, valid, lane);
-      else if (valid) atomicAdd(shared_acc() + gid, 1u);
+      count = false;
     }
   }
   for (uint32_t a = 0; a < Q.naggs; ++a) {
     const int ca = Q.agg_a[a], cb = Q.agg_b[a];
     switch (Q.agg_op[a]) {
-      case DPF_AGG_COUNT: break;  // the row count (slot 0)
+      case DPF_AGG_COUNT: continue;  // the row count (slot 0)
       case DPF_AGG_SUM:
-        agg_dispatch<kHost, DPF_AGG_SUM>(Q, P, seg_mb, list, n, lane, 1 + a, ca, cb, single, status);
+        agg_dispatch<kHost, DPF_AGG_SUM>(Q, P, seg_mb, list, n, lane, 1 + a, ca, cb, single, count, status);
         break;
       case DPF_AGG_SUM_MUL:
-        agg_dispatch<kHost, DPF_AGG_SUM_MUL>(Q, P, seg_mb, list, n, lane, 1 + a, ca, cb, single, status);
+        agg_dispatch<kHost, DPF_AGG_SUM_MUL>(Q, P, seg_mb, list, n, lane, 1 + a, ca, cb, single, count, status);
         break;
       default:
-        agg_dispatch<kHost, DPF_AGG_SUM_SUB>(Q, P, seg_mb, list, n, lane, 1 + a, ca, cb, single, status);
+        agg_dispatch<kHost, DPF_AGG_SUM_SUB>(Q, P, seg_mb, list, n, lane, 1 + a, ca, cb, single, count, status);
         break;
     }
+    count = false;
   }
 }
 

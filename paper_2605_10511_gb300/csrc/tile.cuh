@@ -1390,6 +1390,38 @@ __device__ __forceinline__ uint32_t point_value(const DevQuery& Q, int c, const 
   return h.x + x;
 }
 
+// FOR/DICT column c of the list's segment (mini blocks seg_mb.. of the page):
+// its headers and its packed words.  A list loop takes this once, before its
+// rounds: the plan lies in shared memory, as the list does, so a field read
+// inside the loop is read again after every list write.  Warp-uniform call.
+struct PointCol {
+  const uint2* hdr;
+  const uint32_t* pay;
+};
+__device__ __forceinline__ PointCol point_col(const DevQuery& Q, int c, const PageState& P, uint32_t seg_mb) {
+  const uint8_t* pg = reinterpret_cast<const uint8_t*>(__shfl_sync(kFull, P.pg, c));
+  PointCol C;
+  C.hdr = reinterpret_cast<const uint2*>(pg + kPageHdr) + seg_mb;
+  C.pay = reinterpret_cast<const uint32_t*>(pg + payload_offset(Q.cols[c].codec, P.prow));
+  return C;
+}
+
+// Its value at row r of the segment (r must be one of its rows: lanes without
+// a survivor pass 0): the mini block's header (an L1 hit: the tile's headers
+// were just loaded) and one bit field of its packed payload (two words when
+// the field straddles them).
+template <bool kHost>
+__device__ __forceinline__ uint32_t point_at(const PointCol& C, uint32_t r) {
+  const uint2 h = ld_u2<kHost>(C.hdr + (r >> 7));
+  const uint32_t bw = tmin<uint32_t>(h.y & 0xffu, 32u);
+  const uint32_t bit = (r & (kMB - 1)) * bw, sh = bit & 31u;
+  const uint32_t* p = C.pay + ((h.y >> 8) + (bit >> 5));
+  const uint32_t lo = bw != 0 ? ld_u32<kHost>(p) : 0u;
+  const uint32_t hi = sh + bw > 32 ? ld_u32<kHost>(p + 1) : 0u;
+  const uint32_t x = __funnelshift_r(lo, hi, sh);
+  return h.x + (bw < 32 ? x & ((1u << bw) - 1u) : x);
+}
+
 // Dense decode of one mini block mb of column c whose header is read from
 // the page (lane i < bw loads word k*bw + i): v[k] = value of row 32k + lane.
 template <bool kHost>
