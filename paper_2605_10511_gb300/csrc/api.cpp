@@ -1127,9 +1127,13 @@ uint64_t plans_signature(dpf_ctx* c, const dpf_plan* plans, int32_t n) {
 
 // Fields left 0 take the tuning dpf_autotune stored for these plans, else the
 // defaults.
-// Returns whether something named the ticket size (else kDefaultChunkRows is
-// the largest one and layout_tickets chooses).
-bool fill_tuning_defaults(dpf_ctx* c, dpf_tuning& t, const dpf_plan* plans, int32_t n) {
+// Which fields nothing named: the library chooses them for the batch (chunk:
+// kDefaultChunkRows is the largest ticket and layout_tickets chooses; threads:
+// 256 unless the wide build suits the query better).
+struct OpenFields {
+  bool chunk, threads;
+};
+OpenFields fill_tuning_defaults(dpf_ctx* c, dpf_tuning& t, const dpf_plan* plans, int32_t n) {
   if (t.chunk_rows == 0 || t.threads == 0 || t.ht_placement == 0 || t.ctas_per_sm == 0 || t.staging == 0 ||
       t.group_agg == 0) {
     auto it = c->tune_cache.find(plans_signature(c, plans, n));
@@ -1149,13 +1153,13 @@ bool fill_tuning_defaults(dpf_ctx* c, dpf_tuning& t, const dpf_plan* plans, int3
   if (t.ctas_per_sm == 0) t.ctas_per_sm = d.ctas_per_sm;
   if (t.staging == 0) t.staging = d.staging;
   if (t.group_agg == 0) t.group_agg = d.group_agg;
-  const bool fixed_chunk = t.chunk_rows != 0;
+  const OpenFields open{t.chunk_rows == 0, t.threads == 0 && t.ctas_per_sm == 0};
   if (t.chunk_rows == 0) t.chunk_rows = kDefaultChunkRows;
   if (t.threads == 0) t.threads = 256;
   if (t.ht_placement == 0) t.ht_placement = DPF_HT_AUTO;
   if (t.staging == 0) t.staging = kDefaultStaging;
   if (t.group_agg == 0) t.group_agg = kDefaultGroupAgg;
-  return fixed_chunk;
+  return open;
 }
 
 // A flat JSON object of launch-configuration fields (dpf_set_tuning): the
@@ -1294,7 +1298,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   p->hq.resize(size_t(n));
   dpf_tuning t{};
   if (tuning) t = *tuning;
-  const bool fixed_chunk = fill_tuning_defaults(c, t, plans, n);
+  const OpenFields open = fill_tuning_defaults(c, t, plans, n);
   if (t.chunk_rows % (kMbPerWarpTile * kMB) != 0 || t.chunk_rows > (1u << 24))
     return fail(DPF_EINVAL, "chunk_rows %u must be a multiple of %u and at most 2^24", t.chunk_rows, kMbPerWarpTile * kMB);
   if (t.threads != 128 && t.threads != 256 && t.threads != 512 && t.threads != 1024)
@@ -1377,7 +1381,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     return fail(DPF_EINVAL, "fused kernel does not fit on an SM with %u threads and %zu table bytes", t.threads, max_tables);
   }
   if (t.ctas_per_sm == 0 || int(t.ctas_per_sm) > per_sm || min_blocks == kFusedMinBlocksHi) t.ctas_per_sm = uint32_t(per_sm);
-  layout_tickets(p->hq.data(), n, uint64_t(c->num_sms) * t.ctas_per_sm * (t.threads / 32), t.chunk_rows, fixed_chunk,
+  layout_tickets(p->hq.data(), n, uint64_t(c->num_sms) * t.ctas_per_sm * (t.threads / 32), t.chunk_rows, !open.chunk,
                  qbegin.data());
   // one device block, uploaded by one copy: plans | ticket table | scheduler state (zero)
   const uint64_t at_begin = sizeof(DevQuery) * uint64_t(n), at_sched = align16(at_begin + 8 * qbegin.size());

@@ -19,11 +19,13 @@ constexpr int kFusedMinBlocksLo = 3;
 constexpr int kFusedMinBlocksHi = 4;
 // Rows of one scheduling ticket (one warp's unit of work) unless tuned.
 constexpr uint32_t kDefaultChunkRows = 4096;
+// Rows from which one query takes the 1,024-thread build unless tuned.
+constexpr uint64_t kWideRows = uint64_t(1) << 23;
 // Shared memory of one warp's survivor list (1,024 entries).
 constexpr uint32_t kListBytesPerWarp = 1024 * 4;
 // Words of one warp's scratch of the cooperative string search (search_mb),
 // in launches that have a string-matcher step.
-constexpr uint32_t kSearchWords = 336;
+constexpr uint32_t kSearchWords = 384;
 // Estimated selectivity of the first step from which step 1's mini blocks
 // are prefetched into L2 during the dense tiles (DevQuery::pf_step).
 constexpr double kPrefetchMinSel = 0.03;
@@ -43,8 +45,8 @@ constexpr uint64_t kDirectAlways = uint64_t(1) << 20;  // direct however few row
 constexpr uint64_t kRankMaxRange = uint64_t(1) << 28;
 // Shared-memory bytes of the code-level matcher tables of a PREFIX / CONTAINS
 // step with a pattern of plen bytes on an FSST column: for every matcher
-// state 0..plen, the next state after one symbol code (256 entries) and
-// after one literal byte (256 entries).
+// state below plen, the next state after one symbol code (256 entries) and
+// after one literal byte (256 entries), and behind the former a flag per code.
 inline uint32_t fsst_match_bytes(uint32_t plen) { return (plen + 1) * 512u; }
 
 // Cuts the n queries of a launch into tickets for `warps` resident warps: sets

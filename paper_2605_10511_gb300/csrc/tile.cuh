@@ -380,8 +380,10 @@ __device__ __forceinline__ bool string_scan(const DevStep& S, const uint8_t* s, 
 // for every state q < plen, the entry after symbol code c at tab[q * 256 + c]
 // and after escaped literal byte b at tab[(plen + 1) * 256 + q * 256 + b];
 // an entry is the next state, kFsstHit (the pattern was completed inside the
-// symbol) or kFsstDead (a PREFIX mismatch).  The string's bytes are read as
-// aligned 4-byte words (inside the 16-byte padded page).
+// symbol) or kFsstDead (a PREFIX mismatch).  tab[plen * 256 + c] is 1 for the
+// codes that leave the empty state (and the escape code), where a match can
+// start.  The string's bytes are read as aligned 4-byte words (inside the
+// 16-byte padded page).
 constexpr uint8_t kFsstHit = 0x80, kFsstDead = 0x7f;
 template <bool kHost>
 __device__ __forceinline__ bool fsst_table_match(const DevStep& S, const uint8_t* s, uint32_t len, const uint8_t* tab) {
@@ -446,6 +448,7 @@ __device__ __forceinline__ void build_fsst_matcher(const DevStep& S, const int4*
       }
     }
     tab[i] = uint8_t(e);
+    if (q == 0) tab[n + c] = e != 0;
   }
 }
 
@@ -502,25 +505,12 @@ __device__ __forceinline__ bool string_match(const DevStep& S, const uint8_t* s,
 // own range.  Bytes are taken kSearchWin at a time, so strings of any length
 // fit the scratch.
 constexpr uint32_t kSearchWin = 4096;
-constexpr uint32_t kSearchAhead = 2 * kMaxPrefix;           // bytes an FSST match may run past its first code
-constexpr uint32_t kSearchHits = kSearchWin / 32;            // words of the hit bitmap
-constexpr uint32_t kSearchStarts = (kSearchWin + kSearchAhead) / 32;  // FSST: words of the row-start bitmap
-constexpr uint32_t kLikeQueue = 64;                          // LIKE: candidate rows {offset, length, row}, then
+constexpr uint32_t kSearchHits = kSearchWin / 32;  // words of the hit bitmap
+constexpr uint32_t kCodeQueue = 512 / 2;           // FSST: words of a round's queue of 16-bit positions
+constexpr uint32_t kLikeQueue = 64;                // LIKE: candidate rows {offset, length, row}, then
 constexpr uint32_t kLikeWords = 3 * kLikeQueue + kMB * TB / 32;  // one result bit per row of the tile
-static_assert(kSearchHits + kLikeWords == kSearchWords && kSearchStarts <= kLikeWords,
+static_assert(kSearchHits + kCodeQueue == kSearchWords && kLikeWords <= kCodeQueue,
               "the host's per-warp shared-memory figure");
-
-// Whether bitmap bits [lo, hi) hold a set bit.
-__device__ __forceinline__ bool any_bit(const uint32_t* bits, uint32_t lo, uint32_t hi) {
-  if (lo >= hi) return false;
-  const uint32_t last = (hi - 1) >> 5;
-  uint32_t w = lo >> 5, x = bits[w] & (0xffffffffu << (lo & 31u));
-  while (w < last) {
-    if (x) return true;
-    x = bits[++w];
-  }
-  return (x & (0xffffffffu >> (31u - ((hi - 1) & 31u)))) != 0;
-}
 
 // Occurrences of pat[0..plen), plen >= 1, starting in the 16 bytes at p (bit
 // o: at p[o]); avail = bytes of the mini block from p on.  The first four
@@ -549,100 +539,92 @@ __device__ __forceinline__ uint32_t find_raw(const uint8_t* p, uint64_t avail, c
   return m;
 }
 
-// Bytes of a 16-byte chunk that are literals (the byte after an escape),
-// given esc = its bytes equal to the escape code and whether its first byte
-// is one; *out = whether the next chunk's first byte is.
-__device__ __forceinline__ uint32_t literals(uint32_t esc, bool first, bool* out) {
-  uint32_t lit = first ? 1u : 0u;
-  esc &= ~lit;
+// Literals of a 16-byte chunk (the bytes after an escape code) when its first
+// byte is a code, given esc = its bytes equal to the escape code; bit 16 = the
+// next chunk's first byte is one.
+__device__ __forceinline__ uint32_t literals(uint32_t esc) {
+  uint32_t lit = 0;
   while (esc) {
     const uint32_t b = esc & (0u - esc);
     lit |= b << 1;
     esc &= ~(b | (b << 1));
   }
-  *out = (lit >> 16) & 1u;
-  return lit & 0xffffu;
+  return lit;
 }
 
-// Code positions among the 16 bytes at p where a match of the pattern starts
-// (bit o), for a warp's 32 consecutive chunks; *carry = whether the first
-// chunk starts with a literal, then whether the next 32 do.  skip = leading
-// bytes of the chunk before the mini block, avail = its bytes from p on
-// (0: the lane has no chunk).  A match is found from the code its first byte
-// lies in: the matcher run from its empty state at every code whose table
-// entry leaves that state (a bit row of few codes), for at most plen codes (an
-// occurrence starting inside the first code ends within them), up to the
-// row's end (starts: a bit per row start, from this chunk's window on).
+// Whether a match of the pattern starts in the code at p (avail bytes from p
+// on): the matcher run from its empty state, for at most plen codes, since an
+// occurrence starting inside the first code ends within them.
 template <bool kHost>
-__device__ __forceinline__ uint32_t find_fsst(const uint8_t* p, uint32_t at, uint32_t skip, uint64_t avail, bool* carry,
-                                              const uint8_t* tab, uint32_t plen, const uint32_t* starts, int lane) {
-  uint4 v = make_uint4(0, 0, 0, 0);
-  if (avail) v = ld_u4<kHost>(reinterpret_cast<const uint4*>(p));
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-  uint32_t m = 0, seen = 0;
-#pragma unroll
-  for (int o = 0; o < 16; ++o) {
-    const uint32_t e = tab[(w[o >> 2] >> (8 * (o & 3))) & 0xffu];
-    seen |= e;
-    m |= uint32_t(e != 0) << o;
-  }
-  const uint32_t keep = avail == 0 ? 0u : (0xffffu << skip) & (avail >= 16 ? 0xffffu : (1u << uint32_t(avail)) - 1u);
-  m &= keep;
-  // kFsstDead (bit 6) is the escape code's entry; matcher states stay below 32
-  if (__any_sync(kFull, (seen & 0x40u) != 0) || *carry) {
-    uint32_t esc = 0;
-#pragma unroll
-    for (int o = 0; o < 16; ++o) esc |= uint32_t(((w[o >> 2] >> (8 * (o & 3))) & 0xffu) == kFsstEscape) << o;
-    esc &= keep;
-    bool o0, o1;
-    const uint32_t lit0 = literals(esc, false, &o0), lit1 = literals(esc, true, &o1);
-    // the chunk maps "starts with a literal" (0 / 1) to the next chunk's;
-    // a warp scan composes the maps
-    uint32_t f = uint32_t(o0) | (uint32_t(o1) << 1);
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t g = __shfl_up_sync(kFull, f, d);  // the map of the chunks before
-      if (lane >= d) f = ((f >> (g & 1u)) & 1u) | (((f >> ((g >> 1) & 1u)) & 1u) << 1);
-    }
-    const uint32_t before = __shfl_up_sync(kFull, f, 1);
-    const bool in = lane == 0 ? *carry : ((before >> uint32_t(*carry)) & 1u) != 0;
-    *carry = (__shfl_sync(kFull, f, 31) >> uint32_t(*carry)) & 1u;
-    m &= ~(in ? lit1 : lit0);
-  }
+__device__ __forceinline__ bool fsst_match_at(const uint8_t* p, uint64_t avail, const uint8_t* tab, uint32_t plen) {
   const uint8_t* btab = tab + (plen + 1) * 256;
-  uint32_t hits = 0;
-  while (m) {
-    const uint32_t o = uint32_t(__ffs(m) - 1);
-    m &= m - 1;
-    uint32_t q = 0;
-    uint64_t i = o;
-    for (uint32_t n = 0; n < plen; ++n) {
-      const uint32_t c = ld_u8<kHost>(p + i++);
-      const uint32_t e = c == kFsstEscape ? btab[q * 256 + ld_u8<kHost>(p + i++)] : tab[q * 256 + c];
-      if (e & kFsstHit) {
-        hits |= 1u << o;
-        break;
-      }
-      q = e;
-      if (q == 0 || i >= avail) break;
-      const uint32_t b = at + uint32_t(i);
-      if ((starts[b >> 5] >> (b & 31u)) & 1u) break;
-    }
+  uint32_t q = 0;
+  uint64_t i = 0;
+  for (uint32_t n = 0; n < plen && i < avail; ++n) {
+    const uint32_t c = ld_u8<kHost>(p + i++);
+    const uint32_t e = c == kFsstEscape ? btab[q * 256 + ld_u8<kHost>(p + i++)] : tab[q * 256 + c];
+    if (e & kFsstHit) return true;
+    q = e;
+    if (q == 0) return false;
   }
-  return hits;
+  return false;
+}
+
+// A bit per byte of the 16-byte chunk v where a code may start a match
+// (tab's flag row); *esc = its bytes equal to the escape code.
+__device__ __forceinline__ uint32_t fsst_flags(uint4 v, const uint8_t* flag, uint32_t* esc) {
+  static_assert(kFsstEscape == 255, "an escape byte has every bit set");
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  uint32_t m = 0;
+  *esc = 0;
+#pragma unroll
+  for (int o = 0; o < 16; ++o) m |= uint32_t(flag[(w[o >> 2] >> (8 * (o & 3))) & 0xffu]) << o;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    // bit 7 of each byte of z: the byte of w is 255; gathered by a product
+    const uint32_t z = ((w[i] & 0x7f7f7f7fu) + 0x01010101u) & w[i] & 0x80808080u;
+    *esc |= (((z >> 7) * 0x10204080u) >> 28) << (4 * i);
+  }
+  return m;
+}
+
+// The bytes of a warp's 32 consecutive chunks that are literals, esc = the
+// lane's bytes equal to the escape code; *carry = whether the first chunk
+// starts with one, then whether the next 32 do.
+__device__ __forceinline__ uint32_t warp_literals(uint32_t esc, bool* carry, int lane) {
+  const uint32_t lit = literals(esc);
+  // behind a chunk that ends with an escape its first byte is a literal, which
+  // changes the others only if that byte looks like an escape
+  const uint32_t shifted = (esc & 1u) ? literals(esc & ~1u) | 1u : lit | 1u;
+  if (!*carry && !__any_sync(kFull, ((lit | shifted) >> 16) != 0)) return lit;
+  // the chunk maps "starts with a literal" (0 / 1) to the next chunk's; a
+  // warp scan composes the maps
+  uint32_t f = (lit >> 16) | ((shifted >> 16) << 1);
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t g = __shfl_up_sync(kFull, f, d);  // the map of the chunks before
+    if (lane >= d) f = ((f >> (g & 1u)) & 1u) | (((f >> ((g >> 1) & 1u)) & 1u) << 1);
+  }
+  const uint32_t before = __shfl_up_sync(kFull, f, 1);
+  const bool in = lane == 0 ? *carry : ((before >> uint32_t(*carry)) & 1u) != 0;
+  *carry = (__shfl_sync(kFull, f, 31) >> uint32_t(*carry)) & 1u;
+  return in ? shifted : lit;
 }
 
 // Rows of one mini block (bit k: row 32k + lane, string bytes at mb + st[k],
-// len[k] of them) that hold the pattern pat[0..plen), plen >= 1: kFsst with
-// the code-level matcher tables tab, else compared with the raw bytes.  Out of
-// line: inlined it would be compiled once per mini block of the tile.
+// len[k] of them) that hold the pattern pat[0..plen), plen >= 1; total = the
+// mini block's bytes.  kFsst: with the code-level matcher tables tab, else
+// compared with the raw bytes.  FSST takes a round's flagged codes (few)
+// through a queue, so that the matcher runs on full warps; it is run there up
+// to the mini block's end, and once more up to its own by a row that a hit
+// falls into.
 template <bool kHost, bool kFsst>
-__device__ __noinline__ uint32_t search_mb(const uint8_t* mb, uint4 st4, uint4 len4, const uint8_t* pat, uint32_t plen,
-                                           const uint8_t* tab, uint32_t* scratch, int lane) {
-  const uint32_t st[4] = {st4.x, st4.y, st4.z, st4.w}, len[4] = {len4.x, len4.y, len4.z, len4.w};
+__device__ __forceinline__ uint32_t search_mb(const uint8_t* mb, const uint32_t (&st)[4], const uint32_t (&len)[4],
+                                              uint32_t total, const uint8_t* pat, uint32_t plen, const uint8_t* tab,
+                                              uint32_t* scratch, int lane) {
   uint32_t* hits = scratch;
-  uint32_t* starts = scratch + kSearchHits;
-  const uint32_t total = __shfl_sync(kFull, st[3] + len[3], 31), skew = uint32_t(reinterpret_cast<uintptr_t>(mb)) & 15u;
+  uint16_t* queue = reinterpret_cast<uint16_t*>(scratch + kSearchHits);
+  const uint32_t skew = uint32_t(reinterpret_cast<uintptr_t>(mb)) & 15u;
   const uint64_t end = uint64_t(skew) + total;
   uint32_t pat4 = 0, mask4 = 0, match = 0;
   if (!kFsst) {
@@ -656,26 +638,44 @@ __device__ __noinline__ uint32_t search_mb(const uint8_t* mb, uint4 st4, uint4 l
     const uint8_t* wp = mb - skew + w0;
     const uint64_t left = end - w0;
     const uint32_t wend = uint32_t(tmin<uint64_t>(left, kSearchWin));
-    if (kFsst) {
-      for (uint32_t i = lane; i < kSearchStarts; i += 32) starts[i] = 0;
-      __syncwarp();
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint64_t s = uint64_t(skew) + st[k] - w0;  // wraps below the window
-        if (s < kSearchWin + kSearchAhead) atomicOr(starts + (s >> 5), 1u << (s & 31u));
-      }
-      __syncwarp();
-    }
     for (uint32_t c0 = 0; c0 * 16 < wend; c0 += 32) {
       const uint32_t c = c0 + lane, at = c * 16;
-      uint32_t m = 0;
-      if (kFsst) {
-        const uint32_t skip = w0 == 0 && c == 0 ? skew : 0u;
-        m = find_fsst<kHost>(wp + at, at, skip, at < wend ? left - at : 0u, &carry, tab, plen, starts, lane);
-      } else if (at < wend) {
-        m = find_raw<kHost>(wp + at, left - at, pat, plen, pat4, mask4);
+      if (!kFsst) {
+        if (at < wend)
+          reinterpret_cast<uint16_t*>(hits)[c] =
+              uint16_t(find_raw<kHost>(wp + at, left - at, pat, plen, pat4, mask4));
+        continue;
       }
-      if (at < wend) reinterpret_cast<uint16_t*>(hits)[c] = uint16_t(m);
+      uint4 v = make_uint4(0, 0, 0, 0);
+      uint32_t keep = 0;
+      if (at < wend) {
+        v = ld_u4<kHost>(reinterpret_cast<const uint4*>(wp + at));
+        keep = (0xffffu << (w0 == 0 && c == 0 ? skew : 0u)) & (wend - at >= 16 ? 0xffffu : (1u << (wend - at)) - 1u);
+        reinterpret_cast<uint16_t*>(hits)[c] = 0;
+      }
+      uint32_t esc;
+      uint32_t m = fsst_flags(v, tab + plen * 256, &esc) & keep;
+      esc &= keep;
+      if (__any_sync(kFull, esc != 0) || carry) m &= ~warp_literals(esc, &carry, lane);
+      const uint32_t cnt = __popc(m);
+      uint32_t at_q = cnt;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, at_q, d);
+        if (lane >= d) at_q += y;
+      }
+      const uint32_t queued = __shfl_sync(kFull, at_q, 31);
+      at_q -= cnt;
+      while (m) {
+        queue[at_q++] = uint16_t(at + uint32_t(__ffs(m) - 1));
+        m &= m - 1;
+      }
+      __syncwarp();
+      for (uint32_t j = lane; j < queued; j += 32) {
+        const uint32_t i = queue[j];
+        if (fsst_match_at<kHost>(wp + i, left - i, tab, plen)) atomicOr(hits + (i >> 5), 1u << (i & 31u));
+      }
+      __syncwarp();
     }
     __syncwarp();
 #pragma unroll
@@ -683,8 +683,24 @@ __device__ __noinline__ uint32_t search_mb(const uint8_t* mb, uint4 st4, uint4 l
       // an occurrence in the raw bytes starts at most len - plen into the row
       const uint32_t span = kFsst ? len[k] : (len[k] >= plen ? len[k] - plen + 1 : 0u);
       const int64_t s = int64_t(skew) + int64_t(st[k]) - int64_t(w0), e = s + int64_t(span);
-      const uint32_t lo = uint32_t(tmax<int64_t>(s, 0)), hi = uint32_t(tmax<int64_t>(tmin<int64_t>(e, wend), 0));
-      if (s < int64_t(wend) && !((match >> k) & 1u) && any_bit(hits, lo, hi)) match |= 1u << k;
+      if (s >= int64_t(wend) || e <= 0 || span == 0 || ((match >> k) & 1u)) continue;
+      const uint32_t lo = uint32_t(tmax<int64_t>(s, 0)), hi = uint32_t(tmin<int64_t>(e, wend));
+      const uint32_t last = (hi - 1) >> 5;
+      bool hit = false;
+      for (uint32_t w = lo >> 5; w <= last && !hit; ++w) {
+        uint32_t x = hits[w];
+        if (w == lo >> 5) x &= 0xffffffffu << (lo & 31u);
+        if (w == last) x &= 0xffffffffu >> (31u - ((hi - 1) & 31u));
+        if (!kFsst) {
+          hit = x != 0;
+        } else {
+          for (; x && !hit; x &= x - 1) {
+            const uint32_t i = w * 32 + uint32_t(__ffs(x) - 1);
+            hit = fsst_match_at<kHost>(wp + i, uint64_t(e - int64_t(i)), tab, plen);
+          }
+        }
+      }
+      match |= uint32_t(hit) << k;
     }
     __syncwarp();
   }
@@ -738,9 +754,108 @@ __device__ __forceinline__ uint32_t like_push(const DevStep& S, const uint8_t* b
   return n;
 }
 
-// PREFIX / CONTAINS step over a string column, dense: lengths decoded, their
-// exclusive scan gives each string's start, then each live row's string is
-// matched.  kText = false compiles the raw-PREFIX path only (the general
+// Starts of a mini block's 128 strings from the bw-bit fields f of their
+// lengths (length = base + field): st[k] = bytes before row 32k + lane;
+// returns the fields' sum.  Fields of at most 11 bits are summed two to a
+// register (128 of them stay below 2^16 a half).
+__device__ __forceinline__ uint32_t string_starts(const uint32_t (&f)[4], uint32_t base, uint32_t bw, int lane,
+                                                  uint32_t (&st)[4]) {
+  uint32_t sum;
+  if (bw <= 11) {
+    uint32_t a = f[0] | (f[1] << 16), b = f[2] | (f[3] << 16);
+    const uint32_t a0 = a, b0 = b;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t x = __shfl_up_sync(kFull, a, d), y = __shfl_up_sync(kFull, b, d);
+      if (lane >= d) {
+        a += x;
+        b += y;
+      }
+    }
+    const uint32_t ta = __shfl_sync(kFull, a, 31), tb = __shfl_sync(kFull, b, 31);
+    a -= a0;
+    b -= b0;
+    const uint32_t s1 = ta & 0xffffu, s2 = s1 + (ta >> 16), s3 = s2 + (tb & 0xffffu);
+    st[0] = a & 0xffffu;
+    st[1] = s1 + (a >> 16);
+    st[2] = s2 + (b & 0xffffu);
+    st[3] = s3 + (b >> 16);
+    sum = s3 + (tb >> 16);
+  } else {
+    excl_scan128(f, lane, st);
+    sum = __shfl_sync(kFull, st[3] + f[3], 31);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) st[k] += base * uint32_t(32 * k + lane);
+  return sum;
+}
+
+// CONTAINS, or a general LIKE, dense, with the warp's scratch: one mini block
+// at a time, its strings' starts and lengths in registers, searched
+// cooperatively (search_mb).
+template <bool kHost, bool kFsst>
+__device__ __forceinline__ void tile_search(const DevQuery& Q, const DevStep& S, const PageState& P, const TileHdr& Hd,
+                                            TileState& T, int lane, unsigned int* status, const uint8_t* tab,
+                                            uint32_t* search) {
+  const int col = S.col;
+  const uint32_t plen = S.plen, kind = S.kind, run_at = uint32_t(S.in[0]), run = uint32_t(S.in[1]);
+  const uint8_t* pg = reinterpret_cast<const uint8_t*>(__shfl_sync(kFull, P.pg, col));
+  const uint8_t* bytes = pg + __shfl_sync(kFull, P.extra, col);
+  const uint32_t* pay = reinterpret_cast<const uint32_t*>(pg + payload_offset(C_STR, P.prow));
+  uint32_t* queue = search + kSearchHits;
+  uint32_t* result = queue + 3 * kLikeQueue;
+  const bool like = !kFsst && kind == ST_LIKE;
+  uint32_t waiting = 0;
+  if (like) {
+    if (lane < int(kMB * TB / 32)) result[lane] = 0;
+    __syncwarp();
+  }
+#pragma unroll 1
+  for (int t = 0; t < TB; ++t) {
+    const uint32_t live = (T.alive >> (4 * t)) & 15u;
+    if (!__any_sync(kFull, live != 0)) continue;
+    const uint32_t base = __shfl_sync(kFull, Hd.x, col * TB + t), wob = __shfl_sync(kFull, Hd.y, col * TB + t);
+    const uint32_t mb_start = __shfl_sync(kFull, Hd.sstart, col * TB + t), bw = wob & 0xffu;
+    if (bw > 32) {
+      if (lane == 0) atomicOr(status, S_CORRUPT);
+      T.alive &= ~(15u << (4 * t));
+      continue;
+    }
+    uint32_t len[4], st[4];
+    const uint32_t* src = pay + (wob >> 8) + lane;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) len[k] = uint32_t(lane) < bw ? ld_u32<kHost>(src + uint32_t(k) * bw) : 0u;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      len[k] = unpack_lane(len[k], bw, lane);
+      if (!((live >> k) & 1u)) len[k] = 0;  // a row past the page's last has no bytes
+    }
+    const uint32_t rows = __reduce_add_sync(kFull, uint32_t(__popc(live)));
+    const uint32_t total = string_starts(len, base, bw, lane, st) + base * rows;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) len[k] = (live >> k) & 1u ? len[k] + base : 0u;
+    uint32_t match;
+    if (!like) {
+      match = search_mb<kHost, kFsst>(bytes + mb_start, st, len, total, S.pfx, plen, tab, search, lane);
+    } else {
+      match = run == 0 ? live
+                       : search_mb<kHost, kFsst>(bytes + mb_start, st, len, total, S.pfx + run_at, run, tab, search, lane);
+      waiting = like_push<kHost>(S, bytes, mb_start, st, len, match & live, t, queue, result, waiting, lane);
+    }
+    T.alive &= ~((~match & 15u) << (4 * t));
+  }
+  if (like) {
+    like_round<kHost>(S, bytes, queue, result, waiting, lane);
+#pragma unroll
+    for (int j = 0; j < 4 * TB; ++j)
+      if (!((result[j] >> lane) & 1u)) T.alive &= ~(1u << j);
+    __syncwarp();
+  }
+}
+
+// PREFIX / CONTAINS / LIKE step over a string column, dense: lengths decoded,
+// their exclusive scan gives each string's start, then each live row's string
+// is matched.  kText = false compiles the raw-PREFIX path only (the general
 // matcher of CONTAINS and FSST is left out of the kernel's code); the host
 // launches that build only for batches without such steps, and a step it
 // cannot run drops its rows and reports S_INTERNAL.  With the warp's scratch
@@ -752,13 +867,20 @@ template <bool kHost, bool kText = true>
 __device__ __forceinline__ void tile_prefix(const DevQuery& Q, const DevStep& S, const PageState& P,
                                             const TileHdr& Hd, TileState& T, int lane, unsigned int* status,
                                             const uint8_t* stab, uint32_t* search) {
+  const int4* sym = Q.cols[S.col].codec == C_FSST ? Q.cols[S.col].sym : nullptr;
+  const uint8_t* tab = sym != nullptr && S.smem_width ? stab + S.smem_off : nullptr;
+  if constexpr (kText) {
+    if (search != nullptr && S.plen != 0 && S.kind != ST_PREFIX && (sym == nullptr || tab != nullptr)) {
+      if (sym != nullptr) tile_search<kHost, true>(Q, S, P, Hd, T, lane, status, tab, search);
+      else tile_search<kHost, false>(Q, S, P, Hd, T, lane, status, nullptr, search);
+      return;
+    }
+  }
   uint32_t len[TB][4];
   uint32_t anym;
   tile_decode<kHost>(Q, S.col, P, Hd, T.alive, lane, len, anym, status);
   const uint8_t* pg = reinterpret_cast<const uint8_t*>(__shfl_sync(kFull, P.pg, S.col));
   const uint8_t* bytes = pg + __shfl_sync(kFull, P.extra, S.col);
-  const int4* sym = Q.cols[S.col].codec == C_FSST ? Q.cols[S.col].sym : nullptr;
-  const uint8_t* tab = sym != nullptr && S.smem_width ? stab + S.smem_off : nullptr;
   if (S.kind == ST_PREFIX && sym == nullptr) {
     // raw PREFIX: the warp compares byte i of all its rows' strings at once;
     // a length that is long enough gives way to its string's offset
@@ -796,63 +918,22 @@ __device__ __forceinline__ void tile_prefix(const DevQuery& Q, const DevStep& S,
     T.alive &= match;
     return;
   }
-  uint32_t* queue = search + kSearchHits;
-  uint32_t* result = queue + 3 * kLikeQueue;
-  uint32_t waiting = 0;
-  const bool coop = kText && search != nullptr && S.plen != 0 &&
-                    ((S.kind == ST_CONTAINS && (sym == nullptr || tab != nullptr)) || (S.kind == ST_LIKE && sym == nullptr));
-  if (kText && coop && S.kind == ST_LIKE) {
-    if (lane < int(kMB * TB / 32)) result[lane] = 0;
-    __syncwarp();
-  }
 #pragma unroll
   for (int t = 0; t < TB; ++t) {
     if (!((anym >> t) & 1u)) continue;
-    if (coop) {  // rows past the page's last have no bytes (their field decodes to the mini block's base)
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (!((T.alive >> (4 * t + k)) & 1u)) len[t][k] = 0;
-    }
     uint32_t st[4];
     excl_scan128(len[t], lane, st);
-    const uint32_t mb_start = __shfl_sync(kFull, Hd.sstart, S.col * TB + t);
-    const uint8_t* mb = bytes + mb_start;
+    const uint8_t* mb = bytes + __shfl_sync(kFull, Hd.sstart, S.col * TB + t);
     uint32_t match = 0;
     if constexpr (kText) {
-      if (coop) {
-        const uint32_t live = (T.alive >> (4 * t)) & 15u;
-        const uint4 st4 = make_uint4(st[0], st[1], st[2], st[3]);
-        const uint4 len4 = make_uint4(len[t][0], len[t][1], len[t][2], len[t][3]);
-        if (S.kind == ST_CONTAINS) {
-          match = sym != nullptr ? search_mb<kHost, true>(mb, st4, len4, S.pfx, S.plen, tab, search, lane)
-                                 : search_mb<kHost, false>(mb, st4, len4, S.pfx, S.plen, nullptr, search, lane);
-        } else {
-          const uint32_t run = uint32_t(S.in[1]);
-          match = run == 0 ? live
-                           : search_mb<kHost, false>(mb, st4, len4, S.pfx + S.in[0], run, nullptr, search, lane);
-          waiting = like_push<kHost>(S, bytes, mb_start, st, len[t], match & live, t, queue, result, waiting, lane);
-        }
-      } else {
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (((T.alive >> (4 * t + k)) & 1u) && string_match<kHost>(S, mb + st[k], len[t][k], sym, tab))
-            match |= 1u << k;
-      }
+      for (int k = 0; k < 4; ++k)
+        if (((T.alive >> (4 * t + k)) & 1u) && string_match<kHost>(S, mb + st[k], len[t][k], sym, tab))
+          match |= 1u << k;
     } else {
       if (lane == 0) atomicOr(status, S_INTERNAL);
     }
     T.alive &= ~((~match & 15u) << (4 * t));
-  }
-  if constexpr (kText) {
-    if (coop && S.kind == ST_LIKE) {
-      like_round<kHost>(S, bytes, queue, result, waiting, lane);
-#pragma unroll
-      for (int t = 0; t < TB; ++t)
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (!((result[4 * t + k] >> lane) & 1u)) T.alive &= ~(1u << (4 * t + k));
-      __syncwarp();
-    }
   }
 }
 
