@@ -1366,6 +1366,17 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   if (t.threads > 256 && (host || text || stage_bw))
     return fail(DPF_EINVAL, "CTAs of %u threads run device-resident batches without string-matcher steps, unstaged",
                 t.threads);
+  // One large query over device-resident integers runs best as one CTA of
+  // 1,024 threads per SM (64 registers, 32 warps; one copy of its tables and
+  // accumulators to fill and flush): star join of 67 M rows 229 -> 205 us,
+  // chain of 17 M 102 -> 90, group-by of 10 M 88 -> 85.  Below kWideRows the
+  // 3 x 256 build (80 registers) wins, 32 against 35 us for a star of 5 M
+  // rows, as it does for a raw prefix at any size (207 against 211 us), and in
+  // a batch, whose CTAs change queries (223 against 345 us).
+  if (open.threads && n == 1 && !host && !text && !stage_bw && t.ht_placement == DPF_HT_AUTO &&
+      p->hq[0].nrows >= kWideRows && (p->hq[0].nsteps == 0 || p->hq[0].steps[0].kind != ST_PREFIX) &&
+      fused_blocks_per_sm(1024, acc_slots, max_tables, host, kFusedMinBlocksLo, stage_bw, text) >= 1)
+    t.threads = 1024;
   // ctas_per_sm >= 4 selects the kernel build for four resident CTAs per SM
   // (64 registers) when four fit; otherwise the build for three (80)
   int min_blocks = kFusedMinBlocksLo;
