@@ -348,6 +348,24 @@ dpf_status upload(dpf_ctx* c, void* dst, const void* src, uint64_t bytes) {
   return DPF_OK;
 }
 
+// Device blocks of one call, freed when it ends.
+struct Staging {
+  dpf_ctx* c;
+  std::vector<void*> blocks;
+  ~Staging() {
+    cudaStreamSynchronize(c->io);  // nothing of the call may still use them
+    for (void* p : blocks) dev_free(c, p);
+  }
+  template <class T>
+  bool get(uint64_t count, T** out) {
+    void* p;
+    if (dev_alloc(c, count * sizeof(T), &p)) return false;
+    blocks.push_back(p);
+    *out = static_cast<T*>(p);
+    return true;
+  }
+};
+
 void free_column(dpf_ctx* c, Column& col) {
   if (col.placement == DPF_PLACE_HOST_PINNED) {
     if (col.host_blob) cudaFreeHost(col.host_blob);
@@ -1587,6 +1605,23 @@ dpf_status dpf_memory_used(dpf_ctx* c, uint64_t* bytes) {
   return DPF_OK;
 }
 
+// The device copies of a column's page directory, zone map and dictionary
+// (col.page_off, zones, col.dict).
+static dpf_status attach_metadata(dpf_ctx* c, Column& col, std::vector<int2>& zones) {
+  dpf_status st;
+  const uint64_t npages = col.npages;
+  if ((st = dev_alloc_t(c, npages + 1, &col.d_page_off)) ||
+      (st = upload(c, col.d_page_off, col.page_off.data(), 8 * (npages + 1))) ||
+      (st = dev_alloc_t(c, std::max<uint64_t>(npages, 1), &col.d_zone)) ||
+      (st = upload(c, col.d_zone, zones.data(), sizeof(int2) * npages)))
+    return st;
+  col.zones = std::move(zones);
+  if (col.codec == C_DICT &&
+      ((st = dev_alloc_t(c, col.dict.size(), &col.d_dict)) || (st = upload(c, col.d_dict, col.dict.data(), 4 * col.dict.size()))))
+    return st;
+  return DPF_OK;
+}
+
 dpf_status dpf_load_encoded(dpf_ctx* c, const dpf_column_desc* d, const uint8_t* pages, uint64_t size,
                             const uint64_t* page_off, const uint64_t* row_prefix, uint64_t nrows,
                             const int32_t* dict, uint64_t dict_n, dpf_col_id* out) {
@@ -1658,18 +1693,9 @@ dpf_status dpf_load_encoded(dpf_ctx* c, const dpf_column_desc* d, const uint8_t*
     col.blob = static_cast<uint8_t*>(dp);
     if ((st = upload(c, col.blob, pages, size))) { free_column(c, col); return st; }
   }
-  if ((st = dev_alloc_t(c, npages + 1, &col.d_page_off)) || (st = upload(c, col.d_page_off, page_off, 8 * (npages + 1))) ||
-      (st = dev_alloc_t(c, std::max<uint64_t>(npages, 1), &col.d_zone)) ||
-      (st = upload(c, col.d_zone, zones.data(), sizeof(int2) * npages))) {
+  if ((st = attach_metadata(c, col, zones))) {
     free_column(c, col);
     return st;
-  }
-  col.zones = std::move(zones);
-  if (codec == C_DICT) {
-    if ((st = dev_alloc_t(c, dict_n, &col.d_dict)) || (st = upload(c, col.d_dict, dict, 4 * dict_n))) {
-      free_column(c, col);
-      return st;
-    }
   }
   if (codec == C_FSST) {
     col.nsym = dict_n / 3;
@@ -1686,11 +1712,137 @@ dpf_status dpf_load_encoded(dpf_ctx* c, const dpf_column_desc* d, const uint8_t*
   return DPF_OK;
 }
 
+// Loads a column by encoding it on the device (encode_dev.cu): the same page
+// images, bounds and dictionary as the host encoder gives.  Returns false,
+// with nothing left behind, when it does not apply (a small column, pages in
+// host memory, FSST, a dictionary over a wide range, no memory for the raw
+// values beside the pages) or meets anything wrong: the host path then loads
+// the column or reports the error.
+static bool load_column_device(dpf_ctx* c, const dpf_column_desc* d, const void* values, const uint64_t* offs,
+                               uint64_t nrows, dpf_col_id* out) {
+  const uint32_t codec = uint32_t(d->codec), P = d->page_rows ? d->page_rows : kDefaultPageRows;
+  if (d->placement != DPF_PLACE_DEVICE || nrows < (codec == C_DICT ? kDeviceDictRows : kDeviceEncodeRows) || P % kMB || P > kMaxPageRows || !values) return false;
+  if (codec != C_FOR && codec != C_DELTA && codec != C_DICT && codec != C_FOR64 && codec != C_STR) return false;
+  if (codec == C_STR && (!offs || offs[nrows] < offs[0])) return false;
+  Staging tmp{c, {}};
+  const cudaStream_t s = c->io;
+  EncodeDev E{};
+  E.codec = codec;
+  E.page_rows = P;
+  E.nrows = nrows;
+  E.npages = (nrows + P - 1) / P;
+  E.nmb = (E.npages - 1) * (P / kMB) + (nrows - (E.npages - 1) * P + kMB - 1) / kMB;
+  if (E.npages > (1u << 30)) return false;
+  const uint64_t raw = codec == C_STR ? offs[nrows] - offs[0] : (codec == C_FOR64 ? 8 : 4) * nrows;
+  uint8_t* draw;
+  if (!tmp.get(raw, &draw) || !tmp.get(E.nmb, &E.mb) || !tmp.get(E.npages, &E.pages)) return false;
+  const uint8_t* src = static_cast<const uint8_t*>(values) + (codec == C_STR ? offs[0] : 0);
+  if (raw && cudaMemcpyAsync(draw, src, raw, cudaMemcpyHostToDevice, s) != cudaSuccess) return false;
+  E.v32 = reinterpret_cast<const int32_t*>(draw);
+  E.v64 = reinterpret_cast<const long long*>(draw);
+  E.bytes = draw;
+  if (codec == C_STR) {
+    unsigned long long* doffs;
+    if (!tmp.get(nrows + 1, &doffs) || !tmp.get(E.nmb, &E.mb_bytes)) return false;
+    if (cudaMemcpyAsync(doffs, offs, 8 * (nrows + 1), cudaMemcpyHostToDevice, s) != cudaSuccess) return false;
+    E.offs = doffs;
+  }
+  Column col;
+  if (codec == C_DICT) {
+    struct Head {
+      uint32_t hi, lo;
+      unsigned long long count;
+    } h{};
+    Head* dh;
+    constexpr uint32_t kCap = 65536;
+    int32_t* dvals;
+    uint32_t* words;  // bitmap | ranks
+    if (!tmp.get(1, &dh) || !tmp.get(kCap, &dvals) || cudaMemsetAsync(dh, 0, sizeof(Head), s) != cudaSuccess) return false;
+    if (launch_dict_range(E.v32, nrows, &dh->hi, &dh->lo, s) != cudaSuccess ||
+        cudaMemcpyAsync(&h, dh, sizeof h, cudaMemcpyDeviceToHost, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
+      return false;
+    BuildStat r{};
+    r.hi = h.hi;
+    r.lo = h.lo;
+    const int64_t lo = r.key_lo(), range = int64_t(r.key_hi()) - lo + 1;
+    if (range < 1 || uint64_t(range) > kDeviceDictRange) return false;
+    const uint32_t nwords = uint32_t((range + 31) / 32);
+    if (!tmp.get(2 * uint64_t(nwords), &words) || cudaMemsetAsync(words, 0, 4ull * nwords, s) != cudaSuccess) return false;
+    if (launch_dict_values(E.v32, nrows, int32_t(lo), nwords, words, words + nwords, dvals, kCap, &dh->count, s) != cudaSuccess ||
+        cudaMemcpyAsync(&h, dh, sizeof h, cudaMemcpyDeviceToHost, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess ||
+        h.count == 0 || h.count > kCap)
+      return false;
+    col.dict.resize(h.count);
+    if (cudaMemcpyAsync(col.dict.data(), dvals, 4 * h.count, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        launch_dict_codes(reinterpret_cast<int32_t*>(draw), nrows, int32_t(lo), words, words + nwords, s) != cudaSuccess)
+      return false;
+  }
+  std::vector<EncodePage> pages(E.npages);
+  if (launch_encode_plan(E, s) != cudaSuccess ||
+      cudaMemcpyAsync(pages.data(), E.pages, sizeof(EncodePage) * E.npages, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return false;
+  col.codec = int32_t(codec);
+  col.placement = d->placement;
+  col.table = d->table;
+  col.page_rows = P;
+  col.nrows = nrows;
+  col.npages = E.npages;
+  col.page_off.resize(E.npages + 1);
+  col.row_prefix.resize(E.npages);
+  std::vector<int2> zones(E.npages, make_int2(INT32_MIN, INT32_MAX));
+  const bool bounds = codec != C_STR && codec != C_FOR64;
+  int64_t clo = INT64_MAX, chi = INT64_MIN;
+  uint64_t off = 0, string_region = 0;
+  for (uint64_t p = 0; p < E.npages; ++p) {
+    const EncodePage& q = pages[p];
+    if (q.bad) return false;
+    col.page_off[p] = off;
+    col.row_prefix[p] = std::min<uint64_t>(nrows, (p + 1) * uint64_t(P));
+    off += q.bytes;
+    string_region += q.bytes - q.extra;
+    if (!bounds) continue;
+    clo = std::min<int64_t>(clo, q.lo);
+    chi = std::max<int64_t>(chi, q.hi);
+    col.max_bw = std::max(col.max_bw, q.max_bw);
+    if (q.lo >= INT32_MIN && q.hi <= INT32_MAX) zones[p] = make_int2(int32_t(q.lo), int32_t(q.hi));
+  }
+  col.page_off[E.npages] = off;
+  if (bounds) {
+    col.vmin = std::max<int64_t>(clo, INT32_MIN);
+    col.vmax = std::min<int64_t>(chi, INT32_MAX);
+  }
+  col.bytes = off;
+  col.raw_bytes = codec == C_STR ? string_region + 8 * nrows : raw;
+  void* blob;
+  if (dev_alloc(c, off, &blob)) return false;
+  col.blob = static_cast<uint8_t*>(blob);
+  if (attach_metadata(c, col, zones) == DPF_OK && cudaMemsetAsync(col.blob, 0, off, s) == cudaSuccess) {
+    E.blob = col.blob;
+    E.page_off = col.d_page_off;
+    if (launch_encode_write(E, s) == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess) {
+      col.id = c->next_col++;
+      *out = col.id;
+      c->cols[col.id] = std::move(col);
+      return true;
+    }
+  }
+  cudaStreamSynchronize(s);
+  free_column(c, col);
+  return false;
+}
+
 dpf_status dpf_load_column(dpf_ctx* c, const dpf_column_desc* d, const void* values, const uint64_t* str_offsets,
                            uint64_t nrows, dpf_col_id* out) {
   if (!c || !d || !out) return fail(DPF_EINVAL, "NULL argument");
   const uint32_t P = d->page_rows ? d->page_rows : kDefaultPageRows;
   if (nrows == 0 || P == 0) return fail(DPF_EINVAL, "nrows must be > 0");
+  {
+    std::lock_guard<std::recursive_mutex> lk(c->mu);
+    DeviceGuard g(c->device);
+    if (load_column_device(c, d, values, str_offsets, nrows, out)) return DPF_OK;
+    cudaGetLastError();
+  }
   const uint64_t npages = (nrows + P - 1) / P;
   std::vector<uint64_t> page_off(npages + 1), row_prefix(npages);
   uint64_t size = 0, dict_n = 0;

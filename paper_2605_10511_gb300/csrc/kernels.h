@@ -117,6 +117,51 @@ cudaError_t launch_build_insert(const BuildLaunch& L, cudaStream_t s);
 cudaError_t launch_init_table(uint2* table, uint32_t slots, cudaStream_t s);
 cudaError_t launch_init_direct(uint32_t* table, uint32_t n, cudaStream_t s);
 
+// Device-side encode of a loaded column (encode_dev.cu): raw values in device
+// memory to the page images that dpf_encode_column writes.
+struct EncodeMb {          // a mini block: FOR64's base is {base, first} as one int64, low half first
+  int32_t base, first;
+  uint32_t bw, word_off;   // word_off: 4-byte (FOR64: 8-byte) words into the page's payload
+};
+struct EncodePage {
+  uint64_t bytes;          // size of the page image
+  long long lo, hi;        // value bounds from its headers (FOR / DICT / DELTA)
+  uint32_t max_bw, extra, bad, pad_;  // extra: offset of the byte region; bad: lengths the format cannot hold
+};
+struct EncodeDev {
+  uint32_t codec, page_rows;
+  uint64_t nrows, npages, nmb;
+  const int32_t* v32;      // FOR / DELTA values, DICT codes
+  const long long* v64;    // FOR64
+  const uint8_t* bytes;    // STR: bytes from the first string on, and
+  const unsigned long long* offs;  // the caller's row offsets (the first may be non-zero)
+  EncodeMb* mb;            // [nmb]
+  unsigned long long* mb_bytes;  // STR: [nmb] string bytes, then the mini block's byte start in its page
+  EncodePage* pages;       // [npages]
+  uint8_t* blob;           // write: the pages, zeroed
+  const uint64_t* page_off;
+};
+cudaError_t launch_encode_plan(const EncodeDev& E, cudaStream_t s);   // fills mb and pages
+cudaError_t launch_encode_write(const EncodeDev& E, cudaStream_t s);  // fills blob
+// Dictionary of int32 values: their range (ranks of BuildStat), the distinct
+// ones in ascending order (at most cap are written; bitmap and rank: nwords
+// words over [lo, lo + 32 nwords), bitmap zeroed) and, in place, their codes.
+cudaError_t launch_dict_range(const int32_t* v, uint64_t n, uint32_t* hi, uint32_t* lo, cudaStream_t s);
+cudaError_t launch_dict_values(const int32_t* v, uint64_t n, int32_t lo, uint32_t nwords, uint32_t* bitmap, uint32_t* rank,
+                               int32_t* values, uint32_t cap, unsigned long long* count, cudaStream_t s);
+cudaError_t launch_dict_codes(int32_t* v, uint64_t n, int32_t lo, const uint32_t* bitmap, const uint32_t* rank,
+                              cudaStream_t s);
+// Columns of at least this many rows are encoded on the device when they are
+// to live there: at 8,192 rows the host encoder takes 50 to 57 us (FOR, DELTA,
+// FOR64) where the device's launches take 60, at 65,536 rows it is behind at
+// every codec; its sort of a dictionary's values takes 280 us at 2,000 rows
+// against the device's 140.
+constexpr uint64_t kDeviceEncodeRows = 16384;
+constexpr uint64_t kDeviceDictRows = 1024;
+// Widest value range of a dictionary made on the device (its bitmap is ranked
+// by one CTA).
+constexpr uint64_t kDeviceDictRange = uint64_t(1) << 20;
+
 // Unfused per-operator chain (baseline).  Buffers for every intermediate:
 // decoded columns, predicate flags, two ping-pong (row id, group id) lists
 // and the device-side list lengths.

@@ -1,0 +1,60 @@
+"""Columns that a load encodes on the device have the pages that the host
+encoder writes, byte for byte: every such codec, widths from 0 to full,
+negative and wrapping values, ragged page tails, string offsets that start
+above 0, empty strings; and what the encoder refuses is still refused."""
+
+import numpy as np
+import pytest
+
+import paper_2605_10511_gb300 as dpf
+
+pytestmark = pytest.mark.gpu
+
+
+def _columns(n, rng):
+    spans = [(5, 5), (-3, 4), (900, 105001), (-2**31, 2**31 - 1), (2**31 - 2, 2**31 - 1)]
+    for lo, hi in spans:
+        v = rng.integers(lo, hi, n, endpoint=True).astype(np.int32)
+        yield {"codec": "for", "values": v}
+        yield {"codec": "delta", "values": v if lo == -3 else np.sort(v)}
+    vals = rng.integers(-30000, 30000, int(rng.integers(1, 3000))).astype(np.int32)
+    yield {"codec": "dict", "values": vals[rng.integers(0, vals.size, n)]}
+    yield {"codec": "dict", "values": (vals[rng.integers(0, vals.size, n)] * 70000).astype(np.int32)}  # a wide range
+    for lo, hi in [(7, 7), (-5, 5), (-2**40, 2**40), (-2**63, 2**63 - 1)]:
+        yield {"codec": "for64", "values": rng.integers(lo, hi, n, dtype=np.int64, endpoint=True)}
+    for top in (1, 2, 45, 300):
+        off = np.zeros(n + 1, np.uint64)
+        off[1:] = np.cumsum(rng.integers(0, top, n).astype(np.uint64))
+        off += np.uint64(top % 7)
+        yield {"codec": "str", "bytes": rng.integers(0, 256, int(off[-1]) + 3, dtype=np.uint8), "offsets": off}
+
+
+@pytest.mark.parametrize("n", [1023, 1024, 1025, 16383, 16384, 16385, 100_003])
+@pytest.mark.parametrize("page_rows", [128, 4096, 65536])
+def test_pages_equal_the_host_encoders(n, page_rows):
+    rng = np.random.default_rng(n + page_rows)
+    with dpf.Context(0) as ctx:
+        base = ctx.memory_used()
+        for col in _columns(n, rng):
+            enc = dpf.encode_column(col, page_rows)
+            cid = ctx.load_column(col, table=1, page_rows=page_rows)
+            assert np.array_equal(ctx.column_bytes(cid), enc["blob"]), (col["codec"], n, page_rows)
+            host = ctx.load_encoded(enc, table=1)
+            assert ctx.column_info(cid) == ctx.column_info(host), col["codec"]
+            ctx.drop_column(host)
+            ctx.drop_column(cid)
+        assert ctx.memory_used() == base
+
+
+def test_refusals_stay():
+    off = np.arange(40001, dtype=np.uint64)
+    off[100] = 0
+    bad = [{"codec": "dict", "values": np.arange(70_000, dtype=np.int32)},
+           {"codec": "str", "bytes": np.zeros(50_000, np.uint8), "offsets": off}]
+    with dpf.Context(0) as ctx:
+        base = ctx.memory_used()
+        for col in bad:
+            with pytest.raises(dpf.DpfError) as e:
+                ctx.load_column(col, table=1)
+            assert e.value.status == -1  # DPF_EINVAL
+        assert ctx.memory_used() == base
