@@ -1040,6 +1040,8 @@ dpf_status compile_plan(dpf_ctx* c, const dpf_plan& P, DevQuery& Q, bool* host,
   }
   Q.nsteps = uint32_t(steps.size());
   for (size_t i = 0; i < steps.size(); ++i) Q.steps[i] = steps[order[i]];
+  Q.live = Q.nsteps == 0 ? 1.0f
+                         : float(zone_fraction(c->cols[cs.ids[Q.steps[0].col]], Q.steps[0].zlo, Q.steps[0].zhi));
   // When the first step keeps enough rows (>= 3 % estimated), most 32-byte
   // sectors of step 1's column hold a survivor's field anyway: prefetch its
   // mini blocks into L2 while the dense tiles run, so that step's

@@ -143,12 +143,14 @@ struct alignas(16) DevQuery {
   uint32_t page_rows;
   uint32_t chunk_rows;
   // Tickets of the query (layout_tickets): the first tail_first are owned by
-  // CTAs and cover chunk_rows rows each; the others are in the pool and cover
-  // tail_rows rows each, from row tail_first * chunk_rows on (tail_rows == 0:
-  // every ticket is owned).
+  // CTAs and cover chunk_rows rows each, one after the other through the table,
+  // or page_tickets of them per page (the page's last one fewer rows), so that
+  // none crosses a page.  The others are in the pool and cover tail_rows rows
+  // each, from row tail_row on.
   uint64_t nchunks;
-  uint64_t tail_first;
-  uint32_t tail_rows;
+  uint64_t tail_first, tail_row;
+  uint32_t page_tickets, tail_rows;
+  float live;                  // host: fraction of the rows in pages that the first step's range meets
   uint32_t stage;              // > 0: the first step's mini blocks are staged in the warp's
                                // shared-memory ring, whose slots hold up to `stage` bits a value
   // aggregation: slot 0 = count, slot 1 + a = aggregate a

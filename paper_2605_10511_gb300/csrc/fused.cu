@@ -39,14 +39,38 @@ double row_cost(const DevQuery& Q) {
 // over at least its last `tail` rows (none: tail == 0).
 void cut(DevQuery& Q, uint64_t big, uint64_t small, uint64_t tail) {
   Q.chunk_rows = uint32_t(big);
+  Q.page_tickets = 0;
   if (tail == 0 || small >= big) {
     Q.tail_first = Q.nchunks = (Q.nrows + big - 1) / big;
-    Q.tail_rows = 0;
+    Q.tail_row = Q.nrows;
+    Q.tail_rows = uint32_t(big);
     return;
   }
   Q.tail_first = (Q.nrows - std::min(Q.nrows, tail)) / big;
+  Q.tail_row = Q.tail_first * big;
   Q.tail_rows = uint32_t(small);
-  Q.nchunks = Q.tail_first + (Q.nrows - Q.tail_first * big + small - 1) / small;
+  Q.nchunks = Q.tail_first + (Q.nrows - Q.tail_row + small - 1) / small;
+}
+
+// One ticket per warp, of about per_warp rows.  A ticket that crosses a page
+// is two runs of tiles, one after the other, which costs about as long as 256
+// more cheap rows (a scan of 1 M rows: 17 against 14 us); so when a page's
+// equal tickets are not much larger than that, none crosses a page.
+void cut_once(DevQuery& Q, uint64_t per_warp, uint64_t warps) {
+  const uint64_t P = Q.page_rows, big = round_up(per_warp, kMB);
+  cut(Q, big, 0, 0);
+  if (big >= P) return;
+  for (uint64_t per = (P + big - 1) / big; per > 0; --per) {
+    const uint64_t rows = round_up((P + per - 1) / per, kMB), n = (P + rows - 1) / rows;  // n <= per tickets a page
+    if (double(rows) > double(big) + 256.0 / row_cost(Q)) return;
+    const uint64_t count = Q.nrows / P * n + (Q.nrows % P + rows - 1) / rows;
+    if (count > std::max(warps, Q.nchunks)) continue;
+    Q.chunk_rows = uint32_t(rows);
+    Q.page_tickets = uint32_t(n);
+    Q.tail_first = Q.nchunks = count;
+    Q.tail_rows = uint32_t(rows);
+    return;
+  }
 }
 
 }  // namespace
@@ -55,12 +79,15 @@ void cut(DevQuery& Q, uint64_t big, uint64_t small, uint64_t tail) {
 // than by its rows, so a launch is fastest when every warp gets the same few
 // tickets:
 //  - a query of at most chunk_rows rows per warp is cut into one ticket per
-//    warp (whole mini blocks); there is no pool;
+//    warp (whole mini blocks); there is no pool.  Rows of pages that the first
+//    step's range misses do not count (Q.live): a table of which a seventh is
+//    read has seven tickets per warp;
 //  - a larger one into equal tickets of at most chunk_rows, the same number
 //    for every warp, and a pool of two 512-row tickets per warp, which even
 //    out the warps' different speeds;
 //  - a batch likewise over all its queries, tickets of equal cost, a tenth of
-//    a warp's work in each of two pool tickets.
+//    a warp's work in each of two pool tickets; a query with skipped pages is
+//    in the pool as a whole, since they would fall to few CTAs.
 // With a fixed ticket size (a tuning names it) the last rows, two tickets of
 // an eighth per warp, make the pool, in a batch one per warp and query.
 void layout_tickets(DevQuery* Q, int n, uint64_t warps, uint32_t chunk_rows, bool fixed, uint64_t* begin) {
@@ -74,23 +101,29 @@ void layout_tickets(DevQuery* Q, int n, uint64_t warps, uint32_t chunk_rows, boo
       cut(Q[i], chunk, small, std::max(rows, n > 1 ? std::min(Q[i].nrows, warps * small) : 0));
     }
   } else if (n == 1) {
-    const uint64_t per_warp = (Q->nrows + warps - 1) / warps, pool = 2 * tile;
+    const uint64_t read = std::max<uint64_t>(1, uint64_t(double(Q->nrows) * Q->live));
+    const uint64_t per_warp = (read + warps - 1) / warps, pool = 2 * tile;
     if (per_warp <= chunk) {
-      cut(*Q, round_up(per_warp, kMB), 0, 0);
+      cut_once(*Q, per_warp, warps);
     } else {
       const uint64_t own = per_warp - pool, k = (own + chunk - 1) / chunk;
       cut(*Q, round_up((own + k - 1) / k, tile), tile, warps * pool);
     }
   } else {
     double total = 0;
-    for (int i = 0; i < n; ++i) total += double(Q[i].nrows) * row_cost(Q[i]);
+    for (int i = 0; i < n; ++i) total += double(Q[i].nrows) * Q[i].live * row_cost(Q[i]);
     const double per_warp = total / double(warps);
-    const double k = std::ceil(0.8 * per_warp / double(chunk));
+    const double k = std::max(1.0, std::ceil(0.8 * per_warp / double(chunk)));
     for (int i = 0; i < n; ++i) {
       const double c = row_cost(Q[i]);
       const uint64_t big = std::min(chunk, round_up(uint64_t(0.8 * per_warp / k / c) + 1, kMB));
       const uint64_t small = std::min(big, round_up(uint64_t(0.1 * per_warp / c) + 1, kMB));
       cut(Q[i], big, small, uint64_t(0.2 * double(Q[i].nrows)));
+      if (Q[i].live < 0.75f) {
+        Q[i].tail_first = Q[i].tail_row = 0;
+        Q[i].tail_rows = uint32_t(big);
+        Q[i].nchunks = (Q[i].nrows + big - 1) / big;
+      }
     }
   }
   uint64_t owned = 0, pool = 0;

@@ -389,9 +389,8 @@ __device__ __forceinline__ FirstCol first_col(const DevQuery& Q, const PageState
   return f;
 }
 
-// One ticket: the rows [chunk*chunk_rows, +chunk_rows) of Q's fact table
-// (a smaller range for the pool's tickets: tail_first / tail_rows), processed
-// by one warp, cut at page boundaries into tiles.  A page whose
+// One ticket (layout_tickets): a range of rows of Q's fact table, processed by
+// one warp, cut at page boundaries into tiles.  A page whose
 // zone map misses the first step's value range is skipped whole; inside a
 // page, mini blocks whose headers miss it are skipped by the first step.
 // Each tile loads its headers as it starts (the other resident warps hide
@@ -403,10 +402,17 @@ __device__ void process_ticket(const DevQuery& Q, uint64_t chunk, const uint8_t*
                                uint32_t* list, int lane, unsigned int* status,
                                uint8_t* ring) {
   const uint64_t PR = Q.page_rows;
-  uint64_t r0 = chunk * Q.chunk_rows, r1 = r0 + Q.chunk_rows;
-  if (Q.tail_rows != 0 && chunk >= Q.tail_first) {  // one of the pool's
-    r0 = Q.tail_first * Q.chunk_rows + (chunk - Q.tail_first) * Q.tail_rows;
+  uint64_t r0, r1;
+  if (chunk >= Q.tail_first) {  // one of the pool's
+    r0 = Q.tail_row + (chunk - Q.tail_first) * Q.tail_rows;
     r1 = r0 + Q.tail_rows;
+  } else if (Q.page_tickets) {
+    const uint64_t p = chunk / Q.page_tickets;
+    r0 = p * PR + (chunk - p * Q.page_tickets) * Q.chunk_rows;
+    r1 = tmin<uint64_t>(r0 + Q.chunk_rows, (p + 1) * PR);
+  } else {
+    r0 = chunk * Q.chunk_rows;
+    r1 = r0 + Q.chunk_rows;
   }
   r1 = tmin<uint64_t>(Q.nrows, r1);
   const bool gid0 = Q.nsteps != 0 && step_adds_gid(Q.steps[0]);
@@ -535,9 +541,11 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
   uint32_t* lists = reinterpret_cast<uint32_t*>(stab + tables_bytes);
   // Warps draw tickets on their own (one ticket = a range of rows of one
   // query, processed by one warp), so no CTA barrier separates tickets.  Each
-  // CTA owns an equal run of the launch's `owned` tickets, which its warps
-  // draw with a shared-memory counter: it stays on one query, or few, of a
-  // batch, and a small launch's warps need no global atomic.  Then its warps
+  // CTA owns an equal share of the launch's `owned` tickets, which its warps
+  // draw with a shared-memory counter, so a small launch's warps need no
+  // global atomic: every gridDim-th ticket of a single query (a clustered
+  // table's skipped pages then fall to every CTA alike), a run of a batch's (it
+  // stays on one query, or few).  Then its warps
   // draw from the `pool` of small tickets all CTAs share (sched->next), so
   // that they finish together.  The CTA meets only when its warps' tickets
   // leave the current query: it flushes that query's accumulators and moves to
@@ -555,9 +563,10 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
   auto draw = [&](unsigned long long& t) -> int {
     unsigned int x = 0;
     if (lane == 0) x = atomicAdd(&cs.drawn, 1u);
-    t = own0 + __shfl_sync(kFull, x, 0);
+    x = __shfl_sync(kFull, x, 0);
+    t = nq == 1 ? uint64_t(x) * gridDim.x + blockIdx.x : own0 + x;
     const uint64_t* begin = qbegin;
-    const bool mine = t < own1;
+    const bool mine = t < (nq == 1 ? owned : own1);
     if (!mine) {
       if (pool == 0) return INT_MAX;
       if (lane == 0) t = atomicAdd(&sched->next, 1ull);
