@@ -969,20 +969,32 @@ dpf_status compile_plan(dpf_ctx* c, const dpf_plan& P, DevQuery& Q, bool* host,
   // Step order from a small cost model (the result does not depend on it: a
   // conjunction, and group-id contributions add).  The first step runs
   // densely over the rows of the pages its zone map keeps (the pages whose
-  // value bounds meet the step's range; the kernel skips the others
-  // unread) at a cost of about its column's bits per row; every later step
-  // runs over the survivors of the steps before it at about kSparseCost
-  // bit-equivalents per survivor (a sector read and a probe).  For a given
-  // first step, later filters go most selective first; group keys come
+  // value bounds meet the step's range; the kernel skips the others unread);
+  // every later step runs over the survivors of the steps before it.  For a
+  // given first step, later filters go most selective first; group keys come
   // last.  The plan's own first filter is kept unless another first step is
   // estimated 5 % cheaper.
-  constexpr double kSparseCost = 64.0;
+  // The dense step's work is mostly the same for every row, its column's bits
+  // a small part; a survivor of it costs about six rows; a first probe's table
+  // is copied by every CTA, or probed in device memory when it is large (star
+  // of 67 M rows: first by the 10 % join on 11 bits 208 us, by the 4 % join on
+  // 15 bits and 30,000 keys 195 us; of 5 M rows: 31 and 38 us).  Over the host
+  // link the column's bits are what a row costs (17 M rows: 370 and 400 us).
+  const double kSparseCost = cs.host ? 64.0 : 100.0;
+  constexpr double kTableCost = 1500.0, kSmemTableKeys = 48.0 * 1024, kGlobalProbe = 8.0;
   std::vector<size_t> filters, keys;
   for (size_t i = 0; i < steps.size(); ++i) (steps[i].kind == ST_KEY ? keys : filters).push_back(i);
   std::vector<double> bits(steps.size(), 32.0);
   for (size_t i = 0; i < steps.size(); ++i) {
     const Column& col = c->cols[cs.ids[steps[i].col]];
     if (col.nrows) bits[i] = 8.0 * double(col.bytes) / double(col.nrows) + (steps[i].kind == ST_PROBE ? 4.0 : 0.0);
+    if (!cs.host) {
+      bits[i] = 12.0 + 0.3 * bits[i];
+      if (steps[i].kind == ST_PROBE) {
+        const double keys = steps[i].ht_kind == HT_DIRECT ? double(steps[i].krange) : 1e9;
+        bits[i] += keys <= kSmemTableKeys ? kTableCost * keys / double(std::max<uint64_t>(cs.nrows, 1u << 20)) : kGlobalProbe;
+      }
+    }
     bits[i] *= zone_fraction(col, steps[i].zlo, steps[i].zhi);
   }
   auto plan_cost = [&](size_t first, std::vector<size_t>* out) {
@@ -1089,7 +1101,8 @@ size_t place_tables(DevQuery& Q, size_t budget, bool first_only) {
     if (S.ht_kind == HT_RANK) continue;  // probed in device memory (L2) only
     const bool present = s == 0 && S.ht_kind == HT_DIRECT && (S.mul0 | S.mul1) == 0;
     const uint32_t w = present ? 1u : S.ht_kind == HT_DIRECT ? width : 8u;
-    const size_t bytes = S.ht_kind == HT_DIRECT ? size_t(S.krange) * w + present : size_t(S.ht_mask + 1) * 8;
+    const size_t bytes = S.ht_kind == HT_DIRECT ? size_t(S.krange) * w + present  // and a 0 behind the last key
+                                                : size_t(S.ht_mask + 1) * 8;
     const size_t at = (used + 15) & ~size_t(15);
     if (at + bytes > budget) continue;
     S.smem_width = uint8_t(w);

@@ -507,9 +507,20 @@ __device__ void load_smem_tables(const DevQuery& Q, uint8_t* stab) {
       continue;
     }
     const uint32_t* src = static_cast<const uint32_t*>(S.ht);
-    if (S.present) {
-      for (uint32_t i = threadIdx.x; i <= S.krange; i += blockDim.x)
-        stab[S.smem_off + i] = i < S.krange && __ldg(src + i) != kAbsent ? 1 : 0;
+    if (S.present) {  // eight coalesced loads together
+      for (uint32_t i0 = threadIdx.x; i0 <= S.krange; i0 += 8 * blockDim.x) {
+        uint32_t e[8];
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k) {
+          const uint32_t i = i0 + k * blockDim.x;
+          e[k] = i < S.krange ? __ldg(src + i) : kAbsent;
+        }
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k) {
+          const uint32_t i = i0 + k * blockDim.x;
+          if (i <= S.krange) stab[S.smem_off + i] = e[k] != kAbsent;
+        }
+      }
       continue;
     }
     for (uint32_t i = threadIdx.x; i < S.krange; i += blockDim.x) {
