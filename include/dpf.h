@@ -73,9 +73,11 @@ dpf_status dpf_create(dpf_ctx** out, int32_t device, uint64_t hbm_budget,
 /* Waits for the context's work, frees every object it owns. */
 dpf_status dpf_destroy(dpf_ctx* ctx);
 /* Device bytes held by the context's live objects (columns, hash tables,
- * prepared batches).  Without allocation hooks, freed blocks of up to 64 MiB
- * (1 GiB in all) are kept for reuse and not counted here; with a budget, live
- * plus kept bytes stay within it.  dpf_destroy returns all of them. */
+ * prepared batches; their results lie in pinned host memory).  Without
+ * allocation hooks, freed blocks of up to 1 GiB (8 GiB in all) are kept for
+ * reuse and not counted here; with a budget, live plus kept bytes stay within
+ * it.  Of the pinned result blocks at most 64 MiB are kept when freed.
+ * dpf_destroy returns all of them. */
 dpf_status dpf_memory_used(dpf_ctx* ctx, uint64_t* bytes);
 /* CUDA device the context is bound to. */
 dpf_status dpf_context_device(dpf_ctx* ctx, int32_t* device);
@@ -146,8 +148,14 @@ dpf_status dpf_load_encoded(dpf_ctx* ctx, const dpf_column_desc* desc, const uin
                             uint64_t nrows, const int32_t* dict, uint64_t dict_n,
                             dpf_col_id* out);
 
-/* Encodes on the host (dpf_encode_column) and uploads (dpf_load_encoded).
- * The caller keeps ownership of `values` / `str_offsets`. */
+/* Encodes the column and loads its pages, which are those of
+ * dpf_encode_column byte for byte.  FOR, DELTA, FOR64 and STR columns of at
+ * least 16,384 rows and DICT columns of at least 1,024 (values spanning at
+ * most 2^20) that are placed in device memory are encoded on the device; the
+ * call then holds their raw values there while it runs, and encodes on the
+ * host when they do not fit.  Everything else is encoded on the host and
+ * uploaded (dpf_load_encoded).  The caller keeps ownership of `values` /
+ * `str_offsets`. */
 dpf_status dpf_load_column(dpf_ctx* ctx, const dpf_column_desc* desc, const void* values,
                            const uint64_t* str_offsets, uint64_t nrows, dpf_col_id* out);
 
@@ -341,10 +349,13 @@ typedef struct dpf_plan {
 enum dpf_ht_place { DPF_HT_AUTO = 0, DPF_HT_SMEM = 1, DPF_HT_GLOBAL = 2 };
 typedef struct dpf_tuning {
   uint32_t chunk_rows;   /* rows per scheduling ticket (one warp's unit of work):
-                            multiple of 512, at most 2^24; default 4096        */
+                            multiple of 512, at most 2^24; 0 = chosen for the
+                            batch (equal tickets of at most 4096 rows)         */
   uint32_t threads;      /* threads per CTA: 128 or 256; 512 or 1024 (2 / 1 CTAs
                             per SM) for device-resident, unstaged batches
-                            without CONTAINS / FSST steps                    */
+                            without CONTAINS / FSST steps; 0 = 1024 for one
+                            such query of at least 2^23 rows whose first step
+                            is not a string's, else 256                      */
   int32_t ht_placement;  /* enum dpf_ht_place                                     */
   uint32_t ctas_per_sm;  /* persistent CTAs per SM: 0 = as many as fit of the
                             kernel build for 3 resident 256-thread CTAs

@@ -2760,6 +2760,7 @@ dpf_status dpf_execute_plan(dpf_ctx* c, const dpf_plan* plans, int32_t n, void* 
   st = dpf_launch(c, p->id, stream);
   if (st) {
     const std::string msg = t_last_error;
+    if (cap == cudaStreamCaptureStatusNone) cudaStreamSynchronize(s);  // its upload may still write blocks that are freed
     dpf_release(c, p->id);
     return fail(st, "%s", msg.c_str());
   }

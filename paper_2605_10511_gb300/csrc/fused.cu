@@ -35,6 +35,8 @@ double row_cost(const DevQuery& Q) {
   }
 }
 
+double read_part(const DevQuery& Q) { return std::max(double(Q.live), 0.125); }
+
 // One query: owned tickets of `big` rows, then pool tickets of `small` rows
 // over at least its last `tail` rows (none: tail == 0).
 void cut(DevQuery& Q, uint64_t big, uint64_t small, uint64_t tail) {
@@ -81,7 +83,8 @@ void cut_once(DevQuery& Q, uint64_t per_warp, uint64_t warps) {
 //  - a query of at most chunk_rows rows per warp is cut into one ticket per
 //    warp (whole mini blocks); there is no pool.  Rows of pages that the first
 //    step's range misses do not count (Q.live): a table of which a seventh is
-//    read has seven tickets per warp;
+//    read has seven tickets per warp, eight at most, as a ticket that skips
+//    its page costs a load too;
 //  - a larger one into equal tickets of at most chunk_rows, the same number
 //    for every warp, and a pool of two 512-row tickets per warp, which even
 //    out the warps' different speeds;
@@ -101,7 +104,7 @@ void layout_tickets(DevQuery* Q, int n, uint64_t warps, uint32_t chunk_rows, boo
       cut(Q[i], chunk, small, std::max(rows, n > 1 ? std::min(Q[i].nrows, warps * small) : 0));
     }
   } else if (n == 1) {
-    const uint64_t read = std::max<uint64_t>(1, uint64_t(double(Q->nrows) * Q->live));
+    const uint64_t read = std::max<uint64_t>(1, uint64_t(double(Q->nrows) * read_part(*Q)));
     const uint64_t per_warp = (read + warps - 1) / warps, pool = 2 * tile;
     if (per_warp <= chunk) {
       cut_once(*Q, per_warp, warps);
@@ -111,7 +114,7 @@ void layout_tickets(DevQuery* Q, int n, uint64_t warps, uint32_t chunk_rows, boo
     }
   } else {
     double total = 0;
-    for (int i = 0; i < n; ++i) total += double(Q[i].nrows) * Q[i].live * row_cost(Q[i]);
+    for (int i = 0; i < n; ++i) total += double(Q[i].nrows) * read_part(Q[i]) * row_cost(Q[i]);
     const double per_warp = total / double(warps);
     const double k = std::max(1.0, std::ceil(0.8 * per_warp / double(chunk)));
     for (int i = 0; i < n; ++i) {
