@@ -821,8 +821,9 @@ struct ColumnSet {
   }
 };
 
+// alone: the plan is the launch's only one and may run in the 1,024-thread build.
 dpf_status compile_plan(dpf_ctx* c, const dpf_plan& P, DevQuery& Q, bool* host,
-                        std::vector<const HashTable*>& probes) {
+                        std::vector<const HashTable*>& probes, bool alone) {
   std::memset(&Q, 0, sizeof Q);
   ColumnSet cs{c, Q};
   if (P.n_preds < 0 || P.n_preds > DPF_MAX_PREDS || P.n_joins < 0 || P.n_joins > DPF_MAX_JOINS ||
@@ -981,7 +982,7 @@ dpf_status compile_plan(dpf_ctx* c, const dpf_plan& P, DevQuery& Q, bool* host,
   // 15 bits and 30,000 keys 195 us; of 5 M rows: 31 and 38 us).  Over the host
   // link the column's bits are what a row costs (17 M rows: 370 and 400 us).
   const double kSparseCost = cs.host ? 64.0 : 100.0;
-  constexpr double kTableCost = 1500.0, kSmemTableKeys = 48.0 * 1024, kGlobalProbe = 8.0;
+  constexpr double kTableCost = 1500.0, kSmemTableKeys = 48.0 * 1024, kSharedSmKeys = 16.0 * 1024, kGlobalProbe = 8.0;
   std::vector<size_t> filters, keys;
   for (size_t i = 0; i < steps.size(); ++i) (steps[i].kind == ST_KEY ? keys : filters).push_back(i);
   std::vector<double> bits(steps.size(), 32.0);
@@ -992,7 +993,9 @@ dpf_status compile_plan(dpf_ctx* c, const dpf_plan& P, DevQuery& Q, bool* host,
       bits[i] = 12.0 + 0.3 * bits[i];
       if (steps[i].kind == ST_PROBE) {
         const double keys = steps[i].ht_kind == HT_DIRECT ? double(steps[i].krange) : 1e9;
-        bits[i] += keys <= kSmemTableKeys ? kTableCost * keys / double(std::max<uint64_t>(cs.nrows, 1u << 20)) : kGlobalProbe;
+        bits[i] += keys <= kSmemTableKeys ? kTableCost * keys / double(std::max<uint64_t>(cs.nrows, 1u << 20)) : 0.0;
+        // a large table in three CTAs' shared memory leaves the later probes little L1
+        if (keys > (alone ? kSmemTableKeys : kSharedSmKeys)) bits[i] += kGlobalProbe;
       }
     }
     bits[i] *= zone_fraction(col, steps[i].zlo, steps[i].zhi);
@@ -1052,6 +1055,15 @@ dpf_status compile_plan(dpf_ctx* c, const dpf_plan& P, DevQuery& Q, bool* host,
   }
   Q.nsteps = uint32_t(steps.size());
   for (size_t i = 0; i < steps.size(); ++i) Q.steps[i] = steps[order[i]];
+  {
+    double cost = steps.empty() ? 12.0 : bits[order[0]], surv = 1.0;
+    for (size_t i = 0; i < order.size(); ++i) {
+      if (i > 0) cost += surv * kSparseCost;
+      surv *= std::min(1.0, sel[order[i]]);
+    }
+    for (uint32_t a = 0; a < Q.naggs; ++a) cost += Q.agg_op[a] == DPF_AGG_COUNT ? 0.0 : surv * kSparseCost;
+    Q.cost = float(cost / 27.0);  // the star join: 16 for its dense step, 11 for the survivors
+  }
   Q.live = Q.nsteps == 0 ? 1.0f
                          : float(zone_fraction(c->cols[cs.ids[Q.steps[0].col]], Q.steps[0].zlo, Q.steps[0].zhi));
   // When the first step keeps enough rows (>= 3 % estimated), most 32-byte
@@ -1360,7 +1372,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     DevQuery& Q = p->hq[i];
     bool h = false;
     std::vector<const HashTable*> probes;
-    dpf_status st = compile_plan(c, plans[i], Q, &h, probes);
+    dpf_status st = compile_plan(c, plans[i], Q, &h, probes, n == 1);
     if (st) return fail(st, "plan %d: %s", i, t_last_error.c_str());
     host |= h;
     const size_t used = place_tables(Q, table_budget, t.ht_placement == DPF_HT_AUTO);
@@ -1425,7 +1437,8 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     return fail(DPF_EINVAL, "fused kernel does not fit on an SM with %u threads and %zu table bytes", t.threads, max_tables);
   }
   if (t.ctas_per_sm == 0 || int(t.ctas_per_sm) > per_sm || min_blocks == kFusedMinBlocksHi) t.ctas_per_sm = uint32_t(per_sm);
-  layout_tickets(p->hq.data(), n, uint64_t(c->num_sms) * t.ctas_per_sm * (t.threads / 32), t.chunk_rows, !open.chunk,
+  p->L.strided =
+      layout_tickets(p->hq.data(), n, uint64_t(c->num_sms) * t.ctas_per_sm * (t.threads / 32), t.chunk_rows, !open.chunk,
                  qbegin.data());
   // one device block, uploaded by one copy: plans | ticket table | scheduler state (zero)
   const uint64_t at_begin = sizeof(DevQuery) * uint64_t(n), at_sched = align16(at_begin + 8 * qbegin.size());
@@ -1544,7 +1557,7 @@ namespace dpf {
 dpf_status noalloc_compile(dpf_ctx* c, const dpf_plan* plan, DevQuery* Q, size_t* smem_tables, bool* host,
                            int* device, int* num_sms) {
   std::vector<const HashTable*> probes;
-  dpf_status st = compile_plan(c, *plan, *Q, host, probes);
+  dpf_status st = compile_plan(c, *plan, *Q, host, probes, false);
   if (st) return st;
   const size_t used = place_tables(*Q, size_t(48 * 1024), true);
   *smem_tables = used;
@@ -2534,7 +2547,7 @@ dpf_status dpf_plan_footprint(dpf_ctx* c, const dpf_plan* plan, uint64_t* bytes)
   DevQuery Q;
   bool host = false;
   std::vector<const HashTable*> probes;
-  dpf_status st = compile_plan(c, *plan, Q, &host, probes);
+  dpf_status st = compile_plan(c, *plan, Q, &host, probes, true);
   if (st) return st;
   const uint64_t S1 = 1 + Q.naggs;
   *bytes = align16(uint64_t(Q.domain) * S1 * 8) + 32 + align16(uint64_t(std::max<uint32_t>(Q.domain, 1)) * sizeof(dpf_record)) +

@@ -150,6 +150,7 @@ struct alignas(16) DevQuery {
   uint64_t nchunks;
   uint64_t tail_first, tail_row;
   uint32_t page_tickets, tail_rows;
+  float cost;                  // host: estimated cost of a row, 1 = a star join's
   float live;                  // host: fraction of the rows in pages that the first step's range meets
   uint32_t stage;              // > 0: the first step's mini blocks are staged in the warp's
                                // shared-memory ring, whose slots hold up to `stage` bits a value

@@ -543,7 +543,7 @@ __device__ void load_smem_tables(const DevQuery& Q, uint8_t* stab) {
 template <bool kHost, int kMinBlocks, bool kText, bool kStage = false, int kThreads = 256>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQuery* __restrict__ queries,
                                                        const uint64_t* __restrict__ qbegin, int nq,
-                                                       uint64_t owned, uint64_t pool, Sched* sched,
+                                                       uint64_t owned, uint64_t pool, bool strided, Sched* sched,
                                                        unsigned int* status_out, uint32_t acc_slots,
                                                        uint32_t tables_bytes, uint32_t stage_bw) {
   __shared__ CtaState cs;
@@ -554,9 +554,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
   // query, processed by one warp), so no CTA barrier separates tickets.  Each
   // CTA owns an equal share of the launch's `owned` tickets, which its warps
   // draw with a shared-memory counter, so a small launch's warps need no
-  // global atomic: every gridDim-th ticket of a single query (a clustered
-  // table's skipped pages then fall to every CTA alike), a run of a batch's (it
-  // stays on one query, or few).  Then its warps
+  // global atomic: every gridDim-th one (strided: a clustered table's skipped
+  // pages fall to every CTA alike), or a run of a batch's (it stays on one
+  // query, or few).  Then its warps
   // draw from the `pool` of small tickets all CTAs share (sched->next), so
   // that they finish together.  The CTA meets only when its warps' tickets
   // leave the current query: it flushes that query's accumulators and moves to
@@ -575,9 +575,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
     unsigned int x = 0;
     if (lane == 0) x = atomicAdd(&cs.drawn, 1u);
     x = __shfl_sync(kFull, x, 0);
-    t = nq == 1 ? uint64_t(x) * gridDim.x + blockIdx.x : own0 + x;
+    t = strided ? uint64_t(x) * gridDim.x + blockIdx.x : own0 + x;
     const uint64_t* begin = qbegin;
-    const bool mine = t < (nq == 1 ? owned : own1);
+    const bool mine = t < (strided ? owned : own1);
     if (!mine) {
       if (pool == 0) return INT_MAX;
       if (lane == 0) t = atomicAdd(&sched->next, 1ull);
@@ -656,7 +656,7 @@ cudaError_t launch_as(const FusedLaunch& L, size_t smem, uint32_t tb, cudaStream
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   k<<<L.grid, L.threads, smem, s>>>(
-      L.queries, L.qbegin, L.nq, L.owned, L.pool, L.sched, L.status_out, L.acc_slots, tb, L.stage_bw);
+      L.queries, L.qbegin, L.nq, L.owned, L.pool, L.strided, L.sched, L.status_out, L.acc_slots, tb, L.stage_bw);
   return cudaGetLastError();
 }
 

@@ -53,7 +53,8 @@ inline uint32_t fsst_match_bytes(uint32_t plen) { return (plen + 1) * 512u; }
 // each query's chunk_rows, tail_first, tail_rows and nchunks and fills begin
 // (2 n + 2 entries, FusedLaunch::qbegin).  chunk_rows = the largest ticket;
 // fixed: every owned ticket has that size (a tuning that names it).
-void layout_tickets(DevQuery* Q, int n, uint64_t warps, uint32_t chunk_rows, bool fixed, uint64_t* begin);
+// Returns whether CTAs own every gridDim-th ticket (FusedLaunch::strided).
+bool layout_tickets(DevQuery* Q, int n, uint64_t warps, uint32_t chunk_rows, bool fixed, uint64_t* begin);
 
 // Fused persistent kernel over a batch of compiled queries (Sec. 3.2).
 // qbegin[0..nq] = first owned ticket of each query (qbegin[nq] = owned),
@@ -63,6 +64,7 @@ struct FusedLaunch {
   const uint64_t* qbegin;
   int nq;
   uint64_t owned, pool;
+  bool strided;         // a CTA owns every gridDim-th ticket, else a run of them
   Sched* sched;
   unsigned int* status_out;   // where the launch leaves its status word too (mapped host memory; or nullptr)
   int grid, threads;

@@ -132,7 +132,7 @@ extern "C" dpf_status dpf_execute_noalloc(dpf_ctx* ctx, const dpf_plan* plan, vo
   const int per_sm = fused_blocks_per_sm(L.threads, L.acc_slots, smem_tables, host, L.min_blocks, 0, L.text);
   if (per_sm < 1) return fail(DPF_EINVAL, "dpf_execute_noalloc: fused kernel does not fit on an SM");
   uint64_t qbegin[4];
-  layout_tickets(&Q, 1, uint64_t(num_sms) * per_sm * (L.threads / 32), kDefaultChunkRows, false, qbegin);
+  L.strided = layout_tickets(&Q, 1, uint64_t(num_sms) * per_sm * (L.threads / 32), kDefaultChunkRows, false, qbegin);
   L.owned = qbegin[1];
   L.pool = qbegin[3];
   L.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(uint64_t(num_sms) * per_sm, Q.nchunks)));

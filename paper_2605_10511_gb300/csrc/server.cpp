@@ -140,6 +140,8 @@ void dpf_server::finish_slot(Slot& s) {
   done_cv.notify_all();
 }
 
+static constexpr double kGatherUs = 40.0;
+
 void dpf_server::run() {
   std::unique_lock<std::mutex> lk(mu);
   for (;;) {
@@ -156,9 +158,13 @@ void dpf_server::run() {
       finish_slot(s);  // also reports a failed launch through dpf_read_result
       lk.lock();
     }
-    // launches: FIFO, while a slot is free and the head of the queue fits
+    // launches: FIFO, while a slot is free and the head of the queue fits.
+    // Beside a batch that runs, a short queue waits kGatherUs for company: the
+    // running kernel holds the SMs, so a launch of its own gains nothing
+    // (preparing a batch used to take that long).
     for (Slot& s : slots) {
       if (s.busy || pending.empty()) continue;
+      if (any_busy && pending.size() < cfg.max_batch && !stop && now_us() - pending.front()->submit_us < kGatherUs) break;
       std::vector<std::shared_ptr<Request>> batch;
       uint64_t bytes = 0;
       while (!pending.empty() && batch.size() < cfg.max_batch) {
