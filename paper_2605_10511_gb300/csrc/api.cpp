@@ -1062,7 +1062,8 @@ dpf_status compile_plan(dpf_ctx* c, const dpf_plan& P, DevQuery& Q, bool* host,
       surv *= std::min(1.0, sel[order[i]]);
     }
     for (uint32_t a = 0; a < Q.naggs; ++a) cost += Q.agg_op[a] == DPF_AGG_COUNT ? 0.0 : surv * kSparseCost;
-    Q.cost = float(cost / 27.0);  // the star join: 16 for its dense step, 11 for the survivors
+    // 1 = the star join: 16 for its dense step, 11 for the survivors; a query that reads no page costs its tickets
+    Q.cost = float(std::max(0.25, cost / 27.0));
   }
   Q.live = Q.nsteps == 0 ? 1.0f
                          : float(zone_fraction(c->cols[cs.ids[Q.steps[0].col]], Q.steps[0].zlo, Q.steps[0].zhi));

@@ -127,7 +127,7 @@ bool layout_tickets(DevQuery* Q, int n, uint64_t warps, uint32_t chunk_rows, boo
     const double per_warp = total / double(warps);
     const double k = std::max(1.0, std::ceil(0.8 * per_warp / double(chunk)));
     for (int i = 0; i < n; ++i) {
-      const double c = Q[i].cost;
+      const double c = std::max(0.25, double(Q[i].cost));
       const uint64_t big = std::min(chunk, round_up(uint64_t(0.8 * per_warp / k / c) + 1, kMB));
       const uint64_t small = std::min(big, round_up(uint64_t(0.1 * per_warp / c) + 1, kMB));
       cut(Q[i], big, small, uint64_t(0.2 * double(Q[i].nrows)));
