@@ -61,7 +61,8 @@ struct Column {
   int32_t* d_dict = nullptr;
   std::vector<uint64_t> page_off, row_prefix;
   std::vector<int32_t> dict;
-  int64_t vmin = 0, vmax = -1;    // value bounds from the mini block headers (planner statistics)
+  int64_t vmin = 0, vmax = -1;    // value bounds from the mini block headers (planner statistics, table sizes)
+  bool bounded = false;           // vmin..vmax hold every value: no page's bounds leave int32
   std::vector<int2> zones;        // host copy of the zone map (planner statistics)
   uint32_t max_bw = 0;            // FOR/DICT/DELTA: widest mini block (bits)
   uint64_t nsym = 0;              // FSST: symbols in the table
@@ -687,14 +688,36 @@ dpf_status compile_pred(const Column& c, const dpf_pred& p, DevStep& S, int col_
 // within 127 steps of the mini block's first value, each step in
 // [min(0, dmin), max(0, dmin + 2^bw - 1)]; a page whose bound leaves int32
 // (values may have wrapped) gets the full range.  STR: the full range.
+// ColumnBounds takes the pages' bounds in turn.
+struct ColumnBounds {
+  int64_t lo = INT64_MAX, hi = INT64_MIN;
+  bool inside = true;  // no page's bounds leave int32
+  // Page p's bounds: its zone, and the column's.
+  void add(int64_t page_lo, int64_t page_hi, int2* zone) {
+    lo = std::min(lo, page_lo);
+    hi = std::max(hi, page_hi);
+    if (page_lo >= INT32_MIN && page_hi <= INT32_MAX) *zone = make_int2(int32_t(page_lo), int32_t(page_hi));
+    else inside = false;
+  }
+  // A DELTA column with a page whose values may have wrapped gets the full
+  // range; a FOR column's upper bound is rounded up to a power of two, so one
+  // beyond int32 says nothing of its values when they were encoded from int32
+  // (it is cut), and all the same no table is laid out by it (bounded).
+  void set(Column* c, uint32_t codec) const {
+    if (lo > hi) return;
+    c->bounded = inside;
+    const bool wraps = codec == C_DELTA && !inside;
+    c->vmin = wraps ? INT32_MIN : std::max<int64_t>(lo, INT32_MIN);
+    c->vmax = wraps ? INT32_MAX : std::min<int64_t>(hi, INT32_MAX);
+  }
+};
 void value_bounds(uint32_t codec, const uint8_t* pages, const uint64_t* page_off, uint64_t npages, uint64_t nrows,
-                  uint32_t P, int64_t* vmin, int64_t* vmax, std::vector<int2>* zones, uint32_t* max_bw) {
-  *vmin = 0;
-  *vmax = -1;
+                  uint32_t P, Column* col, std::vector<int2>* zones) {
+  uint32_t* max_bw = &col->max_bw;
   *max_bw = 0;
   zones->assign(npages, make_int2(INT32_MIN, INT32_MAX));
   if (is_str_codec(codec) || codec == C_FOR64) return;  // no 32-bit bounds (never a step's column)
-  int64_t clo = INT64_MAX, chi = INT64_MIN;
+  ColumnBounds cb;
   for (uint64_t p = 0; p < npages; ++p) {
     const uint8_t* pg = pages + page_off[p];
     const uint32_t rows = uint32_t(std::min<uint64_t>(P, nrows - p * uint64_t(P)));
@@ -717,15 +740,9 @@ void value_bounds(uint32_t codec, const uint8_t* pages, const uint64_t* page_off
         hi = std::max(hi, base + (bw >= 32 ? int64_t(0xffffffffll) : (int64_t(1) << bw) - 1));
       }
     }
-    if (lo > hi) continue;
-    clo = std::min(clo, lo);
-    chi = std::max(chi, hi);
-    if (lo >= INT32_MIN && hi <= INT32_MAX) (*zones)[p] = make_int2(int32_t(lo), int32_t(hi));
+    if (lo <= hi) cb.add(lo, hi, &(*zones)[p]);
   }
-  if (clo <= chi) {
-    *vmin = std::max<int64_t>(clo, INT32_MIN);
-    *vmax = std::min<int64_t>(chi, INT32_MAX);
-  }
+  cb.set(col, codec);
 }
 
 // Fraction of a column's rows in pages whose zone map meets [lo, hi]: the
@@ -1691,7 +1708,7 @@ dpf_status dpf_load_encoded(dpf_ctx* c, const dpf_column_desc* d, const uint8_t*
   col.row_prefix.assign(row_prefix, row_prefix + npages);
   if (codec == C_DICT) col.dict.assign(dict, dict + dict_n);
   std::vector<int2> zones;
-  value_bounds(codec, pages, page_off, npages, nrows, P, &col.vmin, &col.vmax, &zones, &col.max_bw);
+  value_bounds(codec, pages, page_off, npages, nrows, P, &col, &zones);
   if (is_str_codec(codec)) {
     uint64_t sb = 0;
     for (uint64_t p = 0; p < npages; ++p) {
@@ -1821,7 +1838,7 @@ static bool load_column_device(dpf_ctx* c, const dpf_column_desc* d, const void*
   col.row_prefix.resize(E.npages);
   std::vector<int2> zones(E.npages, make_int2(INT32_MIN, INT32_MAX));
   const bool bounds = codec != C_STR && codec != C_FOR64;
-  int64_t clo = INT64_MAX, chi = INT64_MIN;
+  ColumnBounds cb;
   uint64_t off = 0, string_region = 0;
   for (uint64_t p = 0; p < E.npages; ++p) {
     const EncodePage& q = pages[p];
@@ -1831,16 +1848,11 @@ static bool load_column_device(dpf_ctx* c, const dpf_column_desc* d, const void*
     off += q.bytes;
     string_region += q.bytes - q.extra;
     if (!bounds) continue;
-    clo = std::min<int64_t>(clo, q.lo);
-    chi = std::max<int64_t>(chi, q.hi);
+    cb.add(q.lo, q.hi, &zones[p]);
     col.max_bw = std::max(col.max_bw, q.max_bw);
-    if (q.lo >= INT32_MIN && q.hi <= INT32_MAX) zones[p] = make_int2(int32_t(q.lo), int32_t(q.hi));
   }
   col.page_off[E.npages] = off;
-  if (bounds) {
-    col.vmin = std::max<int64_t>(clo, INT32_MIN);
-    col.vmax = std::min<int64_t>(chi, INT32_MAX);
-  }
+  cb.set(&col, codec);
   col.bytes = off;
   col.raw_bytes = codec == C_STR ? string_region + 8 * nrows : raw;
   void* blob;
@@ -2152,7 +2164,7 @@ static dpf_status build_status_error(uint32_t status, dpf_col_id key_col) {
 }
 
 // Exact sizing.  When the key column's load-time bounds span at most
-// kDirectAlways keys (and no budget limits the context's memory), the table is
+// kDirectAlways keys and hold every key (and no budget limits the context's memory), the table is
 // a direct one whatever rows are kept: one pass fills a table over those
 // bounds, and the table is its part from the smallest to the largest key kept
 // (what an exactly sized one would hold).
@@ -2192,7 +2204,7 @@ static dpf_status build_hash_impl(dpf_ctx* c, const dpf_build& B, void* stream, 
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->bstat, &zero, sizeof zero, cudaMemcpyHostToDevice, s);
   bool done = false;
   uint64_t kept = 0;
-  const uint64_t span = kc.vmin <= kc.vmax ? uint64_t(kc.vmax - kc.vmin + 1) : 0;
+  const uint64_t span = kc.bounded && kc.vmin <= kc.vmax ? uint64_t(kc.vmax - kc.vmin + 1) : 0;
   if (e == cudaSuccess && !bs.wide_payload && span != 0 && span <= kDirectAlways && c->budget == 0) {
     st = alloc_table(c, bs, kc.nrows, kc.vmin, kc.vmax, ht, L, s);
     if (st == DPF_OK) {

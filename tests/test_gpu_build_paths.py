@@ -48,6 +48,44 @@ def test_both_paths_give_the_same_table(span, keep):
     assert info[0] == info[1]
 
 
+@pytest.mark.parametrize("n", [3000, 20_000])  # encoded on the host, and on the device
+@pytest.mark.parametrize("asynchronous", [False, True])
+def test_delta_keys_that_wrap(n, asynchronous):
+    """Keys that run past the largest int32 to the smallest (DELTA adds modulo
+    2^32), inside the last mini block: no header names a negative one, and the
+    column's bounds are the whole of int32 all the same."""
+    at = np.arange(n, dtype=np.int64)
+    keys = (2**31 - 3 - 7 * (n - 25) + 7 * at).astype(np.uint32).astype(np.int32)
+    assert keys.min() < 0 < keys.max() and -2**31 not in keys
+    fk = keys[np.random.default_rng(n).integers(0, n, 9001)]
+    w = {"name": f"wrap_{n}_{asynchronous}", "fact": "f",
+         "tables": {"d": {"rows": n, "page_rows": 1024, "cols": {"k": {"codec": "delta", "values": keys},
+                                                                 "p": {"codec": "dict", "values": (at % 7).astype(np.int32)}}},
+                    "f": {"rows": fk.size, "page_rows": 1024, "cols": {"fk": {"codec": "for", "values": fk}}}},
+         "query": {"preds": [], "group": [{"join": 0, "field": 0}], "aggs": [{"op": "count"}],
+                   "joins": [{"fk": "fk", "dim": "d", "key": "k", "payload": ["p"], "preds": []}]}}
+    want = oracle.run_query(w, from_encoded=False)
+    e = dpf.Engine(device=0)
+    try:
+        got = e.run(w, asynchronous=asynchronous)
+        assert got.shape == want.shape and all(np.array_equal(got[f], want[f]) for f in ("key", "count", "val"))
+    finally:
+        e.close()
+
+
+def test_for_pages_whose_fields_wrap():
+    """A mini block of another writer, its base near the largest int32: base +
+    field wraps, and every key is found."""
+    n = 128
+    enc = dpf.encode_column({"codec": "for", "values": 2 * np.arange(n, dtype=np.int32)}, 128)
+    enc["blob"][16:20].view(np.int32)[0] = 2**31 - 99
+    keys = (2 * np.arange(n, dtype=np.int64) + 2**31 - 99).astype(np.uint32).astype(np.int32)
+    assert keys.min() < 0 < keys.max() and -2**31 not in keys
+    with dpf.Context(0) as ctx:
+        k = ctx.load_encoded(enc, table=1)
+        assert ctx.hash_info(ctx.build_hash(k))["entries"] == n
+
+
 def test_duplicate_keys_are_refused_by_both():
     keys = np.array([1, 5, 9, 5], np.int32)
     for budget in (0, 1 << 30):
