@@ -430,8 +430,9 @@ dpf_status dpf_capture_graph(dpf_ctx* ctx, dpf_prep_id prep, void* stream);
 dpf_status dpf_launch_graph(dpf_ctx* ctx, dpf_prep_id prep, void* stream);
 /* Waits (up to timeout_ms; < 0 = forever) for the last launch of `prep`
  * and copies query i's records, ascending by key tuple, to host `buf`.
- * DPF_ETRUNC if cap < needed (*n_out = needed).  Device status words turn
- * into DPF_ECORRUPT / DPF_EINTERNAL. */
+ * DPF_ETRUNC if cap < needed (*n_out = needed).  A device status word turns
+ * into DPF_ECORRUPT / DPF_EINTERNAL: it is the launch's, so every query of
+ * the batch reports it, on every read, until another launch has run. */
 dpf_status dpf_read_result(dpf_ctx* ctx, dpf_prep_id prep, int32_t i, dpf_record* buf,
                            uint64_t cap, uint64_t* n_out, int32_t timeout_ms);
 /* Tuning the batch will launch with (after defaults and cache lookup;

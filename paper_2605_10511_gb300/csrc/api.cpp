@@ -1344,6 +1344,7 @@ cudaError_t launch_prep(Prep* p, cudaStream_t s) {
     uint32_t n = 0;
     cudaError_t e = launch_unfused(p->U, s, &n);
     if (e == cudaSuccess) e = cudaMemcpyAsync(p->results, &p->sched->status, 4, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(&p->sched->status, 0, 4, s);
     p->launches = n;
     return e;
   }
@@ -1539,7 +1540,7 @@ dpf_status wait_event(cudaEvent_t ev, int32_t timeout_ms) {
   }
 }
 
-dpf_status read_result(dpf_ctx* c, Prep* p, int32_t i, dpf_record* buf, uint64_t cap, uint64_t* n_out,
+dpf_status read_result(Prep* p, int32_t i, dpf_record* buf, uint64_t cap, uint64_t* n_out,
                        int32_t timeout_ms) {
   if (i < 0 || i >= p->nq) return fail(DPF_EINVAL, "query index %d out of range", i);
   if (!p->launched) return fail(DPF_EINVAL, "batch %d was never launched", p->id);
@@ -1549,10 +1550,7 @@ dpf_status read_result(dpf_ctx* c, Prep* p, int32_t i, dpf_record* buf, uint64_t
   uint32_t status, n;
   std::memcpy(&status, p->results, 4);
   std::memcpy(&n, p->results + p->off_n[size_t(i)], 4);
-  if (status) {
-    std::memset(p->results, 0, 4);
-    cudaMemsetAsync(&p->sched->status, 0, 4, c->io);
-    cudaStreamSynchronize(c->io);
+  if (status) {  // of the whole launch: every query of it reports the error
     if (status & S_CORRUPT) return fail(DPF_ECORRUPT, "device reported corrupt data (status %u)", status);
     return fail(DPF_EINTERNAL, "device reported an internal error (status %u)", status);
   }
@@ -2502,7 +2500,7 @@ dpf_status dpf_autotune(dpf_ctx* c, const dpf_plan* plans, int32_t n, void* stre
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
     uint32_t status = 0;
-    if (e == cudaSuccess) e = cudaMemcpy(&status, &p->sched->status, 4, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) std::memcpy(&status, p->results, 4);
     dpf_tuning used = p->tuning;
     release_prep(c, p);
     c->preps.erase(id);
@@ -2628,7 +2626,7 @@ dpf_status dpf_read_result(dpf_ctx* c, dpf_prep_id id, int32_t i, dpf_record* bu
   DeviceGuard g(c->device);
   Prep* p = find_prep(c, id);
   if (!p) return fail(DPF_EINVAL, "unknown batch %d", id);
-  return read_result(c, p, i, buf, cap, n_out, timeout_ms);
+  return read_result(p, i, buf, cap, n_out, timeout_ms);
 }
 
 dpf_status dpf_prepare_unfused(dpf_ctx* c, const dpf_plan* plan, dpf_prep_id* out) {
@@ -2802,7 +2800,7 @@ dpf_status dpf_fetch_result(dpf_ctx* c, dpf_query_id id, dpf_record* buf, uint64
   Prep* p = find_prep(c, dpf_prep_id(id >> 20));
   const int32_t i = int32_t(id & 0xfffff);
   if (!p || !p->oneshot || i >= p->nq || p->fetched[i]) return fail(DPF_ENOTFOUND, "unknown or fetched query id %lld", (long long)id);
-  dpf_status st = read_result(c, p, i, buf, cap, n_out, timeout_ms);
+  dpf_status st = read_result(p, i, buf, cap, n_out, timeout_ms);
   if (st) return st;
   p->fetched[i] = 1;
   if (std::all_of(p->fetched.begin(), p->fetched.end(), [](char f) { return f != 0; })) {

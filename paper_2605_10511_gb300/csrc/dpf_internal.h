@@ -188,7 +188,7 @@ inline bool needs_string_matcher(const DevQuery& Q) {
 struct Sched {
   unsigned long long next;     // ticket counter
   unsigned int exited;         // CTAs that left the persistent loop
-  unsigned int status;         // StatusBits
+  unsigned int status;         // StatusBits of the launch that runs
 };
 
 }  // namespace dpf

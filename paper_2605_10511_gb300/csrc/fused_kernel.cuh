@@ -634,7 +634,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
     if (old == gridDim.x - 1) {
       sched->next = 0ull;
       sched->exited = 0u;
-      if (status_out) *status_out = atomicOr(&sched->status, 0u);  // every other CTA has left
+      // every other CTA has left: the launch's status word, and a clean one for the next
+      if (status_out) *status_out = atomicExch(&sched->status, 0u);
       __threadfence();
     }
   }

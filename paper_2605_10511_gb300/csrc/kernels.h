@@ -66,7 +66,7 @@ struct FusedLaunch {
   uint64_t owned, pool;
   bool strided;         // a CTA owns every gridDim-th ticket, else a run of them
   Sched* sched;
-  unsigned int* status_out;   // where the launch leaves its status word too (mapped host memory; or nullptr)
+  unsigned int* status_out;   // where the launch leaves its status word (mapped host memory); nullptr: in sched
   int grid, threads;
   uint32_t acc_slots;   // int64 shared accumulators per CTA (max over the batch)
   size_t smem_tables;   // bytes of the CTA's join-table region

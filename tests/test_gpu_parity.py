@@ -296,6 +296,40 @@ def test_fsst_codes_outside_the_table_are_rejected(eng):
     assert ex.value.status == -9  # DPF_ECORRUPT
 
 
+@pytest.mark.parametrize("unfused", [False, True])
+def test_a_launch_that_met_corrupt_data_fails_every_read(unfused):
+    """A dictionary code beyond the dictionary drops its row: no query of that
+    launch returns records, however often it is read; launching again does not
+    clear it, and a batch without the page is not touched by it."""
+    n = 3000
+    g = np.array([10, 20, 30], np.int32)[np.arange(n) % 3]
+    enc = dpf.encode_column({"codec": "dict", "values": g}, 1024)
+    pay = (16 + 1024 // 128 * 8 + 15) // 16 * 16
+    assert enc["blob"][20] == 2              # mini block 0: two bits a code
+    enc["blob"][pay] |= 3                    # row 0's code becomes 3
+    w = {"name": "bad_code", "fact": "fact", "tables": {"fact": {"rows": n, "page_rows": 1024, "cols": {
+        "g": {"codec": "dict", "values": g}}}},
+        "query": {"preds": [], "joins": [], "group": [{"col": "g"}], "aggs": [{"op": "count"}]}}
+    clean = synth.scan_filter_aggregate(rows=5000, page_rows=1024)
+    e = dpf.Engine(device=0)
+    try:
+        e.tables[(w["name"], "fact")] = 77
+        e.cols[(w["name"], "fact", "g")] = e.ctx.load_encoded(enc, table=77)
+        e.load_workload(clean)
+        ok = e.plan(clean)
+        prep = e.ctx.prepare_unfused(e.plan(w)) if unfused else e.ctx.prepare([ok, e.plan(w), ok])
+        for _ in range(2):
+            e.ctx.launch(prep)
+            for i in [0, 0] if unfused else [0, 1, 2, 1, 0]:
+                with pytest.raises(dpf.DpfError) as ex:
+                    e.ctx.read_result(prep, i)
+                assert ex.value.status == -9  # DPF_ECORRUPT
+        e.ctx.release(prep)
+        assert_same(e.run(clean), expect(clean), "clean")
+    finally:
+        e.close()
+
+
 def test_batch_mixing_lean_and_string_matcher_queries(eng):
     """A batch with one CONTAINS-on-FSST query runs the kernel build with the
     general string matcher for every query in it; the same queries alone run
