@@ -348,9 +348,9 @@ typedef struct dpf_plan {
  * table in device memory (served by L1/L2). */
 enum dpf_ht_place { DPF_HT_AUTO = 0, DPF_HT_SMEM = 1, DPF_HT_GLOBAL = 2 };
 typedef struct dpf_tuning {
-  uint32_t chunk_rows;   /* rows per scheduling ticket (one warp's unit of work):
-                            multiple of 512, at most 2^24; 0 = chosen for the
-                            batch (equal tickets of at most 4096 rows)         */
+  uint32_t chunk_rows;   /* most rows of a scheduling ticket (one warp's unit of
+                            work; a launch is cut into equal ones of at most
+                            this): multiple of 512, at most 2^24; 0 = 4096     */
   uint32_t threads;      /* threads per CTA: 128 or 256; 512 or 1024 (2 / 1 CTAs
                             per SM) for device-resident, unstaged batches
                             without CONTAINS / FSST steps; 0 = 1024 for one

@@ -745,19 +745,25 @@ void value_bounds(uint32_t codec, const uint8_t* pages, const uint64_t* page_off
   cb.set(col, codec);
 }
 
-// Fraction of a column's rows in pages whose zone map meets [lo, hi]: the
-// rows a first step over that range decodes (the kernel skips the other
-// pages unread).
-double zone_fraction(const Column& col, int32_t lo, int32_t hi) {
-  if (col.nrows == 0 || col.zones.empty()) return 1.0;
-  if (lo > hi) return 0.0;
-  uint64_t kept = 0;
-  for (uint64_t p = 0; p < col.zones.size(); ++p) {
-    const int2 z = col.zones[p];
-    if (z.y < lo || z.x > hi) continue;
-    kept += std::min<uint64_t>(col.page_rows, col.nrows - p * uint64_t(col.page_rows));
+// The part of a column whose pages' zone map meets [lo, hi]: the rows a first
+// step over that range decodes (the kernel skips the other pages unread).
+struct ZonePart {
+  uint64_t row0 = 0, rows = 0;  // from the first such page to the last
+  uint64_t kept = 0;            // rows in such pages
+};
+ZonePart zone_part(const Column& col, int32_t lo, int32_t hi) {
+  ZonePart z;
+  for (uint64_t p = 0; p < col.zones.size() && lo <= hi; ++p) {
+    if (col.zones[p].y < lo || col.zones[p].x > hi) continue;
+    const uint64_t a = p * uint64_t(col.page_rows), n = std::min<uint64_t>(col.page_rows, col.nrows - a);
+    if (z.kept == 0) z.row0 = a;
+    z.rows = a + n - z.row0;
+    z.kept += n;
   }
-  return double(kept) / double(col.nrows);
+  return z;
+}
+double zone_fraction(const Column& col, int32_t lo, int32_t hi) {
+  return col.nrows ? double(zone_part(col, lo, hi).kept) / double(col.nrows) : 1.0;
 }
 
 // Estimated fraction of rows a step keeps, for ordering the steps: range
@@ -839,8 +845,9 @@ struct ColumnSet {
 };
 
 // alone: the plan is the launch's only one and may run in the 1,024-thread build.
+// share: what the launch will read of the table.
 dpf_status compile_plan(dpf_ctx* c, const dpf_plan& P, DevQuery& Q, bool* host,
-                        std::vector<const HashTable*>& probes, bool alone) {
+                        std::vector<const HashTable*>& probes, bool alone, ScanShare* share) {
   std::memset(&Q, 0, sizeof Q);
   ColumnSet cs{c, Q};
   if (P.n_preds < 0 || P.n_preds > DPF_MAX_PREDS || P.n_joins < 0 || P.n_joins > DPF_MAX_JOINS ||
@@ -1080,10 +1087,15 @@ dpf_status compile_plan(dpf_ctx* c, const dpf_plan& P, DevQuery& Q, bool* host,
     }
     for (uint32_t a = 0; a < Q.naggs; ++a) cost += Q.agg_op[a] == DPF_AGG_COUNT ? 0.0 : surv * kSparseCost;
     // 1 = the star join: 16 for its dense step, 11 for the survivors; a query that reads no page costs its tickets
-    Q.cost = float(std::max(0.25, cost / 27.0));
+    share->cost = std::max(0.25, cost / 27.0);
   }
-  Q.live = Q.nsteps == 0 ? 1.0f
-                         : float(zone_fraction(c->cols[cs.ids[Q.steps[0].col]], Q.steps[0].zlo, Q.steps[0].zhi));
+  *share = ScanShare{0, cs.nrows, 1.0, share->cost};
+  if (Q.nsteps != 0) {
+    const ZonePart z = zone_part(c->cols[cs.ids[Q.steps[0].col]], Q.steps[0].zlo, Q.steps[0].zhi);
+    share->row0 = z.row0;
+    share->rows = std::max<uint64_t>(z.rows, 1);
+    share->live = double(z.kept) / double(share->rows);
+  }
   // When the first step keeps enough rows (>= 3 % estimated), most 32-byte
   // sectors of step 1's column hold a survivor's field anyway: prefetch its
   // mini blocks into L2 while the dense tiles run, so that step's
@@ -1190,13 +1202,9 @@ uint64_t plans_signature(dpf_ctx* c, const dpf_plan* plans, int32_t n) {
 
 // Fields left 0 take the tuning dpf_autotune stored for these plans, else the
 // defaults.
-// Which fields nothing named: the library chooses them for the batch (chunk:
-// kDefaultChunkRows is the largest ticket and layout_tickets chooses; threads:
-// 256 unless the wide build suits the query better).
-struct OpenFields {
-  bool chunk, threads;
-};
-OpenFields fill_tuning_defaults(dpf_ctx* c, dpf_tuning& t, const dpf_plan* plans, int32_t n) {
+// Returns whether nothing named the threads: then the library chooses (256
+// unless the wide build suits the query better).
+bool fill_tuning_defaults(dpf_ctx* c, dpf_tuning& t, const dpf_plan* plans, int32_t n) {
   if (t.chunk_rows == 0 || t.threads == 0 || t.ht_placement == 0 || t.ctas_per_sm == 0 || t.staging == 0 ||
       t.group_agg == 0) {
     auto it = c->tune_cache.find(plans_signature(c, plans, n));
@@ -1216,13 +1224,13 @@ OpenFields fill_tuning_defaults(dpf_ctx* c, dpf_tuning& t, const dpf_plan* plans
   if (t.ctas_per_sm == 0) t.ctas_per_sm = d.ctas_per_sm;
   if (t.staging == 0) t.staging = d.staging;
   if (t.group_agg == 0) t.group_agg = d.group_agg;
-  const OpenFields open{t.chunk_rows == 0, t.threads == 0 && t.ctas_per_sm == 0};
+  const bool open_threads = t.threads == 0 && t.ctas_per_sm == 0;
   if (t.chunk_rows == 0) t.chunk_rows = kDefaultChunkRows;
   if (t.threads == 0) t.threads = 256;
   if (t.ht_placement == 0) t.ht_placement = DPF_HT_AUTO;
   if (t.staging == 0) t.staging = kDefaultStaging;
   if (t.group_agg == 0) t.group_agg = kDefaultGroupAgg;
-  return open;
+  return open_threads;
 }
 
 // A flat JSON object of launch-configuration fields (dpf_set_tuning): the
@@ -1362,7 +1370,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   p->hq.resize(size_t(n));
   dpf_tuning t{};
   if (tuning) t = *tuning;
-  const OpenFields open = fill_tuning_defaults(c, t, plans, n);
+  const bool open_threads = fill_tuning_defaults(c, t, plans, n);
   if (t.chunk_rows % (kMbPerWarpTile * kMB) != 0 || t.chunk_rows > (1u << 24))
     return fail(DPF_EINVAL, "chunk_rows %u must be a multiple of %u and at most 2^24", t.chunk_rows, kMbPerWarpTile * kMB);
   if (t.threads != 128 && t.threads != 256 && t.threads != 512 && t.threads != 1024)
@@ -1373,6 +1381,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   bool any_warp_agg = false;
   bool host = false;
   std::vector<uint64_t> qbegin(2 * size_t(n) + 2);
+  std::vector<ScanShare> shares(static_cast<size_t>(n));
   // scratch per query: acc | done; results per query: record count | records
   std::vector<uint64_t> off_acc(n), off_done(n);
   uint64_t scratch = 0, results = 64;
@@ -1391,7 +1400,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     DevQuery& Q = p->hq[i];
     bool h = false;
     std::vector<const HashTable*> probes;
-    dpf_status st = compile_plan(c, plans[i], Q, &h, probes, n == 1);
+    dpf_status st = compile_plan(c, plans[i], Q, &h, probes, n == 1, &shares[size_t(i)]);
     if (st) return fail(st, "plan %d: %s", i, t_last_error.c_str());
     host |= h;
     const size_t used = place_tables(Q, table_budget, t.ht_placement == DPF_HT_AUTO);
@@ -1437,7 +1446,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   // 3 x 256 build (80 registers) wins, 32 against 35 us for a star of 5 M
   // rows, as it does for a raw prefix at any size (207 against 211 us), and in
   // a batch, whose CTAs change queries (223 against 345 us).
-  if (open.threads && n == 1 && !host && !text && !stage_bw && t.ht_placement == DPF_HT_AUTO &&
+  if (open_threads && n == 1 && !host && !text && !stage_bw && t.ht_placement == DPF_HT_AUTO &&
       p->hq[0].nrows >= kWideRows && (p->hq[0].nsteps == 0 || p->hq[0].steps[0].kind != ST_PREFIX) &&
       fused_blocks_per_sm(1024, acc_slots, max_tables, host, kFusedMinBlocksLo, stage_bw, text) >= 1)
     t.threads = 1024;
@@ -1456,14 +1465,15 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     return fail(DPF_EINVAL, "fused kernel does not fit on an SM with %u threads and %zu table bytes", t.threads, max_tables);
   }
   if (t.ctas_per_sm == 0 || int(t.ctas_per_sm) > per_sm || min_blocks == kFusedMinBlocksHi) t.ctas_per_sm = uint32_t(per_sm);
-  p->L.strided =
-      layout_tickets(p->hq.data(), n, uint64_t(c->num_sms) * t.ctas_per_sm * (t.threads / 32), t.chunk_rows, !open.chunk,
-                 qbegin.data());
-  // one device block, uploaded by one copy: plans | ticket table | scheduler state (zero)
+  const uint64_t ctas = uint64_t(c->num_sms) * t.ctas_per_sm;
+  layout_tickets(p->hq.data(), shares.data(), n, ctas * (t.threads / 32), t.chunk_rows, qbegin.data());
+  // one device block, uploaded by one copy: plans | ticket table | scheduler
+  // state | a batch's ticket counters, one per CTA (zero)
   const uint64_t at_begin = sizeof(DevQuery) * uint64_t(n), at_sched = align16(at_begin + 8 * qbegin.size());
+  const uint64_t at_drawn = align16(at_sched + sizeof(Sched)), up_bytes = at_drawn + (n > 1 ? 4 * ctas : 0);
   dpf_status st;
   if ((st = dev_alloc(c, scratch, reinterpret_cast<void**>(&p->scratch))) ||
-      (st = dev_alloc(c, at_sched + sizeof(Sched), reinterpret_cast<void**>(&p->dq))) ||
+      (st = dev_alloc(c, up_bytes, reinterpret_cast<void**>(&p->dq))) ||
       (st = pin_alloc(c, results, reinterpret_cast<void**>(&p->results)))) {
     const std::string msg = t_last_error;
     release_prep(c, p.get());
@@ -1480,7 +1490,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     Q.out = p->results + p->off_rec[size_t(i)];
     *reinterpret_cast<uint32_t*>(p->results + p->off_n[size_t(i)]) = 0;
   }
-  std::vector<uint8_t> up(at_sched + sizeof(Sched), 0);
+  std::vector<uint8_t> up(up_bytes, 0);
   std::memcpy(up.data(), p->hq.data(), at_begin);
   std::memcpy(up.data() + at_begin, qbegin.data(), 8 * qbegin.size());
   const cudaStream_t us = on ? *on : c->io;
@@ -1505,7 +1515,8 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   p->L.sched = p->sched;
   p->L.status_out = reinterpret_cast<unsigned int*>(p->results);
   p->L.threads = int(t.threads);
-  p->L.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(uint64_t(c->num_sms) * t.ctas_per_sm, p->L.owned + p->L.pool)));
+  p->L.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(ctas, p->L.owned + p->L.pool)));
+  if (n > 1 && p->L.owned) p->L.drawn = reinterpret_cast<unsigned int*>(reinterpret_cast<uint8_t*>(p->dq) + at_drawn);
   p->L.smem_tables = max_tables;
   p->L.acc_slots = acc_slots;
   p->L.host_data = host;
@@ -1570,10 +1581,10 @@ namespace dpf {
 // Compiles one plan for dpf_execute_noalloc (no device allocation): the
 // device plan with hash tables placed in shared memory as dpf_prepare's
 // automatic placement would, the table bytes and the launch geometry.
-dpf_status noalloc_compile(dpf_ctx* c, const dpf_plan* plan, DevQuery* Q, size_t* smem_tables, bool* host,
-                           int* device, int* num_sms) {
+dpf_status noalloc_compile(dpf_ctx* c, const dpf_plan* plan, DevQuery* Q, ScanShare* share, size_t* smem_tables,
+                           bool* host, int* device, int* num_sms) {
   std::vector<const HashTable*> probes;
-  dpf_status st = compile_plan(c, *plan, *Q, host, probes, false);
+  dpf_status st = compile_plan(c, *plan, *Q, host, probes, false, share);
   if (st) return st;
   const size_t used = place_tables(*Q, size_t(48 * 1024), true);
   *smem_tables = used;
@@ -2558,7 +2569,8 @@ dpf_status dpf_plan_footprint(dpf_ctx* c, const dpf_plan* plan, uint64_t* bytes)
   DevQuery Q;
   bool host = false;
   std::vector<const HashTable*> probes;
-  dpf_status st = compile_plan(c, *plan, Q, &host, probes, true);
+  ScanShare share;
+  dpf_status st = compile_plan(c, *plan, Q, &host, probes, true, &share);
   if (st) return st;
   const uint64_t S1 = 1 + Q.naggs;
   *bytes = align16(uint64_t(Q.domain) * S1 * 8) + 32 + align16(uint64_t(std::max<uint32_t>(Q.domain, 1)) * sizeof(dpf_record)) +

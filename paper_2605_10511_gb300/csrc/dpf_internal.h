@@ -142,16 +142,15 @@ struct alignas(16) DevQuery {
   uint64_t nrows;
   uint32_t page_rows;
   uint32_t chunk_rows;
-  // Tickets of the query (layout_tickets): the first tail_first are owned by
-  // CTAs and cover chunk_rows rows each, one after the other through the table,
-  // or page_tickets of them per page (the page's last one fewer rows), so that
-  // none crosses a page.  The others are in the pool and cover tail_rows rows
-  // each, from row tail_row on.
+  // Tickets of the query (layout_tickets, ticket_rows), from row row0 on, the
+  // start of a page: the first tail_first are owned by CTAs and cover chunk_rows
+  // rows each, one after the other through the table, or page_tickets of them
+  // per page (the page's last one fewer rows), so that none crosses a page.
+  // The others are in the pool and cover tail_rows rows each, from row
+  // row0 + tail_row on.
   uint64_t nchunks;
-  uint64_t tail_first, tail_row;
+  uint64_t tail_first, tail_row, row0;
   uint32_t page_tickets, tail_rows;
-  float cost;                  // host: estimated cost of a row, 1 = a star join's
-  float live;                  // host: fraction of the rows in pages that the first step's range meets
   uint32_t stage;              // > 0: the first step's mini blocks are staged in the warp's
                                // shared-memory ring, whose slots hold up to `stage` bits a value
   // aggregation: slot 0 = count, slot 1 + a = aggregate a
@@ -183,6 +182,24 @@ inline bool needs_string_matcher(const DevQuery& Q) {
       return true;
   }
   return false;
+}
+
+// Rows [*r0, *r1) of the query's ticket t.
+__host__ __device__ inline void ticket_rows(const DevQuery& Q, uint64_t t, uint64_t* r0, uint64_t* r1) {
+  uint64_t a, b;
+  if (t >= Q.tail_first) {  // one of the pool's
+    a = Q.tail_row + (t - Q.tail_first) * Q.tail_rows;
+    b = a + Q.tail_rows;
+  } else if (Q.page_tickets) {
+    const uint64_t p = t / Q.page_tickets, end = (p + 1) * Q.page_rows;
+    a = p * Q.page_rows + (t - p * Q.page_tickets) * Q.chunk_rows;
+    b = a + Q.chunk_rows < end ? a + Q.chunk_rows : end;
+  } else {
+    a = t * Q.chunk_rows;
+    b = a + Q.chunk_rows;
+  }
+  *r0 = Q.row0 + a;
+  *r1 = Q.row0 + b < Q.nrows ? Q.row0 + b : Q.nrows;
 }
 
 struct Sched {

@@ -31,7 +31,8 @@ __device__ __forceinline__ uint32_t* shared_acc() { return reinterpret_cast<uint
 struct alignas(16) CtaState {
   DevQuery q;
   int wq[32];          // query of the ticket each warp holds (INT_MAX: none left)
-  unsigned int drawn;  // tickets drawn from the CTA's own range
+  unsigned int drawn;  // tickets drawn from the CTA's own range (one query)
+  unsigned int victim; // batches: the CTA whose run this one's warps draw from, at first its own
   unsigned int mine;   // tickets of the current query this CTA processed
   int last;
   unsigned int warp_sum[32];
@@ -403,18 +404,7 @@ __device__ void process_ticket(const DevQuery& Q, uint64_t chunk, const uint8_t*
                                uint8_t* ring) {
   const uint64_t PR = Q.page_rows;
   uint64_t r0, r1;
-  if (chunk >= Q.tail_first) {  // one of the pool's
-    r0 = Q.tail_row + (chunk - Q.tail_first) * Q.tail_rows;
-    r1 = r0 + Q.tail_rows;
-  } else if (Q.page_tickets) {
-    const uint64_t p = chunk / Q.page_tickets;
-    r0 = p * PR + (chunk - p * Q.page_tickets) * Q.chunk_rows;
-    r1 = tmin<uint64_t>(r0 + Q.chunk_rows, (p + 1) * PR);
-  } else {
-    r0 = chunk * Q.chunk_rows;
-    r1 = r0 + Q.chunk_rows;
-  }
-  r1 = tmin<uint64_t>(Q.nrows, r1);
+  ticket_rows(Q, chunk, &r0, &r1);
   const bool gid0 = Q.nsteps != 0 && step_adds_gid(Q.steps[0]);
   for (uint64_t p = r0 / PR; p <= (r1 - 1) / PR; ++p) {
     const uint64_t pr0 = tmax<uint64_t>(r0, p * PR), pr1 = tmin<uint64_t>(r1, (p + 1) * PR);
@@ -534,6 +524,34 @@ __device__ void load_smem_tables(const DevQuery& Q, uint8_t* stab) {
   }
 }
 
+// Batches: a ticket of another CTA's run, when this CTA's is used up.  A run's
+// cost is an estimate, so the CTAs that finish early take over from those that
+// hold most.  The lanes look at 32 CTAs spread over the grid; the one with the
+// most tickets left is drawn from, unless it has no more than its own warps are
+// about to draw.  Returns the ticket, or ~0 when nothing is worth it.  The CTA's
+// warps follow one another (CtaState::victim), so that they stay on one query.
+__device__ __noinline__ unsigned long long steal_ticket(unsigned int* drawn, uint64_t owned, CtaState& cs, int lane) {
+  for (uint32_t k = 1; k <= 4; ++k) {
+    const uint32_t v = uint32_t((uint64_t(blockIdx.x) + k + uint64_t(lane) * gridDim.x / 32) % gridDim.x);
+    const uint64_t v0 = owned * v / gridDim.x, v1 = owned * (v + 1) / gridDim.x;
+    const uint32_t size = uint32_t(v1 - v0), x = __ldcg(drawn + v), left = size - tmin(size, x);
+    const uint32_t best = __reduce_max_sync(kFull, left);
+    if (best <= (blockDim.x >> 5)) return ~0ull;
+    const int w = __ffs(__ballot_sync(kFull, left == best)) - 1;
+    unsigned long long t = ~0ull;
+    if (lane == w) {
+      const uint32_t i = atomicAdd(drawn + v, 1u);
+      if (i < size) {
+        t = v0 + i;
+        cs.victim = v;
+      }
+    }
+    t = __shfl_sync(kFull, t, w);
+    if (t != ~0ull) return t;
+  }
+  return ~0ull;
+}
+
 // kText = false: the build without the general string matcher (CONTAINS,
 // FSST), launched for batches that have no such step.  kStage: the build
 // with the staging ring (device-resident batches without such steps,
@@ -543,7 +561,7 @@ __device__ void load_smem_tables(const DevQuery& Q, uint8_t* stab) {
 template <bool kHost, int kMinBlocks, bool kText, bool kStage = false, int kThreads = 256>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQuery* __restrict__ queries,
                                                        const uint64_t* __restrict__ qbegin, int nq,
-                                                       uint64_t owned, uint64_t pool, bool strided, Sched* sched,
+                                                       uint64_t owned, uint64_t pool, unsigned int* drawn, Sched* sched,
                                                        unsigned int* status_out, uint32_t acc_slots,
                                                        uint32_t tables_bytes, uint32_t stage_bw) {
   __shared__ CtaState cs;
@@ -552,32 +570,45 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
   uint32_t* lists = reinterpret_cast<uint32_t*>(stab + tables_bytes);
   // Warps draw tickets on their own (one ticket = a range of rows of one
   // query, processed by one warp), so no CTA barrier separates tickets.  Each
-  // CTA owns an equal share of the launch's `owned` tickets, which its warps
-  // draw with a shared-memory counter, so a small launch's warps need no
-  // global atomic: every gridDim-th one (strided: a clustered table's skipped
-  // pages fall to every CTA alike), or a run of a batch's (it stays on one
-  // query, or few).  Then its warps
-  // draw from the `pool` of small tickets all CTAs share (sched->next), so
-  // that they finish together.  The CTA meets only when its warps' tickets
+  // CTA owns an equal share of the launch's `owned` tickets.  Of one query's it
+  // is every gridDim-th one (a clustered table's skipped pages fall to every
+  // CTA alike), drawn with a shared-memory counter, so a small launch's warps
+  // need no global atomic.  Of a batch's it is a run, so that the CTA stays on
+  // one query, or few, drawn with the CTA's counter in `drawn`, so that others
+  // can take over (steal_ticket).  Then the warps draw from the `pool` of small
+  // tickets that all CTAs share (sched->next).  The CTA meets only when its warps' tickets
   // leave the current query: it flushes that query's accumulators and moves to
   // the smallest query any warp holds.
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   uint32_t* list = lists + uint32_t(warp) * kListCap;
   uint8_t* ring = reinterpret_cast<uint8_t*>(lists + nw * kListCap) +
                   size_t(warp) * (kText ? kSearchWords * sizeof(uint32_t) : stage_warp_bytes(stage_bw));
-  const uint64_t own0 = owned * blockIdx.x / gridDim.x, own1 = owned * (blockIdx.x + 1) / gridDim.x;
-  if (threadIdx.x == 0) cs.drawn = 0;
+  if (threadIdx.x == 0) {
+    cs.drawn = 0;
+    cs.victim = blockIdx.x;
+  }
   __syncthreads();
   // Draws the warp's next ticket: its query (INT_MAX: none left), and in t its
   // index among the query's tickets (owned ones first).  qbegin[0..nq] = each
   // query's first owned ticket, qbegin[nq + 1 ..] = its first pool ticket.
   auto draw = [&](unsigned long long& t) -> int {
-    unsigned int x = 0;
-    if (lane == 0) x = atomicAdd(&cs.drawn, 1u);
-    x = __shfl_sync(kFull, x, 0);
-    t = strided ? uint64_t(x) * gridDim.x + blockIdx.x : own0 + x;
+    if (drawn != nullptr) {
+      if (lane == 0) {
+        const uint32_t v = *const_cast<volatile unsigned int*>(&cs.victim);
+        const uint64_t i = owned * v / gridDim.x + atomicAdd(drawn + v, 1u);
+        t = i < owned * (v + 1) / gridDim.x ? i : ~0ull;
+      }
+      t = __shfl_sync(kFull, t, 0);
+      if (t == ~0ull) t = steal_ticket(drawn, owned, cs, lane);
+      if (t == ~0ull) return INT_MAX;
+    } else {
+      unsigned int x = 0;
+      if (lane == 0) x = atomicAdd(&cs.drawn, 1u);
+      x = __shfl_sync(kFull, x, 0);
+      t = uint64_t(x) * gridDim.x + blockIdx.x;
+    }
     const uint64_t* begin = qbegin;
-    const bool mine = t < (strided ? owned : own1);
+    const bool mine = t < owned;
     if (!mine) {
       if (pool == 0) return INT_MAX;
       if (lane == 0) t = atomicAdd(&sched->next, 1ull);
@@ -634,6 +665,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
     if (old == gridDim.x - 1) {
       sched->next = 0ull;
       sched->exited = 0u;
+      if (drawn != nullptr)
+        for (uint32_t i = 0; i < gridDim.x; ++i) drawn[i] = 0u;
       // every other CTA has left: the launch's status word, and a clean one for the next
       if (status_out) *status_out = atomicExch(&sched->status, 0u);
       __threadfence();
@@ -657,7 +690,7 @@ cudaError_t launch_as(const FusedLaunch& L, size_t smem, uint32_t tb, cudaStream
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   k<<<L.grid, L.threads, smem, s>>>(
-      L.queries, L.qbegin, L.nq, L.owned, L.pool, L.strided, L.sched, L.status_out, L.acc_slots, tb, L.stage_bw);
+      L.queries, L.qbegin, L.nq, L.owned, L.pool, L.drawn, L.sched, L.status_out, L.acc_slots, tb, L.stage_bw);
   return cudaGetLastError();
 }
 

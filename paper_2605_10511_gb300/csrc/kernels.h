@@ -49,12 +49,18 @@ constexpr uint64_t kRankMaxRange = uint64_t(1) << 28;
 // after one literal byte (256 entries), and behind the former a flag per code.
 inline uint32_t fsst_match_bytes(uint32_t plen) { return (plen + 1) * 512u; }
 
-// Cuts the n queries of a launch into tickets for `warps` resident warps: sets
-// each query's chunk_rows, tail_first, tail_rows and nchunks and fills begin
-// (2 n + 2 entries, FusedLaunch::qbegin).  chunk_rows = the largest ticket;
-// fixed: every owned ticket has that size (a tuning that names it).
-// Returns whether CTAs own every gridDim-th ticket (FusedLaunch::strided).
-bool layout_tickets(DevQuery* Q, int n, uint64_t warps, uint32_t chunk_rows, bool fixed, uint64_t* begin);
+// What a launch reads of a query's table, and how long a row of it takes.
+struct ScanShare {
+  uint64_t row0, rows;  // from the first to the last page that the first step's range meets (at least one row)
+  double live;          // fraction of those rows in such pages
+  double cost;          // time of a row, 1 = a star join's
+};
+
+// Cuts the n queries of a launch into tickets of at most chunk_rows rows for
+// `warps` resident warps: sets each query's chunk_rows, page_tickets, tail_first,
+// tail_row, tail_rows, row0 and nchunks and fills begin (2 n + 2 entries,
+// FusedLaunch::qbegin).
+void layout_tickets(DevQuery* Q, const ScanShare* S, int n, uint64_t warps, uint32_t chunk_rows, uint64_t* begin);
 
 // Fused persistent kernel over a batch of compiled queries (Sec. 3.2).
 // qbegin[0..nq] = first owned ticket of each query (qbegin[nq] = owned),
@@ -64,7 +70,7 @@ struct FusedLaunch {
   const uint64_t* qbegin;
   int nq;
   uint64_t owned, pool;
-  bool strided;         // a CTA owns every gridDim-th ticket, else a run of them
+  unsigned int* drawn;  // batches with owned tickets: a counter per CTA, zero between launches (else nullptr)
   Sched* sched;
   unsigned int* status_out;   // where the launch leaves its status word (mapped host memory); nullptr: in sched
   int grid, threads;

@@ -21,8 +21,8 @@
 
 namespace dpf {
 
-dpf_status noalloc_compile(dpf_ctx* c, const dpf_plan* plan, DevQuery* Q, size_t* smem_tables, bool* host,
-                           int* device, int* num_sms);
+dpf_status noalloc_compile(dpf_ctx* c, const dpf_plan* plan, DevQuery* Q, ScanShare* share, size_t* smem_tables,
+                           bool* host, int* device, int* num_sms);
 std::recursive_mutex& ctx_mutex(dpf_ctx* c);
 
 // Capacity of the shared scratch region (1 MiB): scheduler state, the
@@ -84,10 +84,11 @@ extern "C" dpf_status dpf_execute_noalloc(dpf_ctx* ctx, const dpf_plan* plan, vo
       return fail(DPF_EINVAL, "dpf_execute_noalloc cannot be captured into a CUDA graph (the stream is capturing)");
   }
   DevQuery Q;
+  ScanShare share;
   size_t smem_tables = 0;
   bool host = false;
   int device = 0, num_sms = 0;
-  dpf_status st = noalloc_compile(ctx, plan, &Q, &smem_tables, &host, &device, &num_sms);
+  dpf_status st = noalloc_compile(ctx, plan, &Q, &share, &smem_tables, &host, &device, &num_sms);
   if (st) return st;
   int prev = -1;
   cudaGetDevice(&prev);
@@ -132,7 +133,7 @@ extern "C" dpf_status dpf_execute_noalloc(dpf_ctx* ctx, const dpf_plan* plan, vo
   const int per_sm = fused_blocks_per_sm(L.threads, L.acc_slots, smem_tables, host, L.min_blocks, 0, L.text);
   if (per_sm < 1) return fail(DPF_EINVAL, "dpf_execute_noalloc: fused kernel does not fit on an SM");
   uint64_t qbegin[4];
-  L.strided = layout_tickets(&Q, 1, uint64_t(num_sms) * per_sm * (L.threads / 32), kDefaultChunkRows, false, qbegin);
+  layout_tickets(&Q, &share, 1, uint64_t(num_sms) * per_sm * (L.threads / 32), kDefaultChunkRows, qbegin);
   L.owned = qbegin[1];
   L.pool = qbegin[3];
   L.grid = int(std::max<uint64_t>(1, std::min<uint64_t>(uint64_t(num_sms) * per_sm, Q.nchunks)));
