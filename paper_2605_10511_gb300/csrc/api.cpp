@@ -796,6 +796,35 @@ double step_selectivity(const DevStep& S, const Column* col, const HashTable* ht
   return S.kind == ST_NOTRANGE ? 1.0 - in : in;
 }
 
+// Estimated time of a step, in us per million rows of the table, for sharing a
+// batch's rows out: dense as the first step, else over the surviving fraction
+// of the rows.  Fitted to single queries' times (256-thread builds, slope over
+// the rows): star join 3.4; scan with 2 %, 30 % and all rows left by its first
+// step 1.6, 2.6 and 2.8, with all of them aggregated over two columns 11.2;
+// group-by of all rows 8.6; chain (delta keys, a rank table) 6.1; on strings of
+// 28 bytes prefix 5.1, CONTAINS 17 to 21, LIKE 20 to 25; FSST (14 bytes a
+// string) prefix 16, CONTAINS 20 to 33.
+constexpr double kStarTime = 3.4;
+double step_time(const DevStep& S, const Column& col, bool first, double surv) {
+  const double bytes = col.nrows ? double(col.bytes) / double(col.nrows) : 0.0;
+  const bool text = S.kind == ST_PREFIX || S.kind == ST_CONTAINS || S.kind == ST_LIKE, fsst = col.codec == C_FSST;
+  if (!first) {
+    // survivors share sectors and rounds: no dearer from one row in sixteen on;
+    // a string step decodes the lengths of each of their mini blocks
+    const double shared = std::min(1.0, surv / 0.06);
+    if (text) return 3.0 * std::min(1.0, 128.0 * surv) + 2.5 * bytes * surv;
+    return (S.kind == ST_PROBE || is_step64(S.kind) ? 2.4 : 1.2) * shared;
+  }
+  switch (S.kind) {
+    case ST_ALL: return 0.0;
+    case ST_PREFIX: return fsst ? 1.15 * bytes : 1.5 + 0.13 * bytes;
+    case ST_CONTAINS: return (fsst ? 1.6 : 0.65) * bytes;
+    case ST_LIKE: return 0.8 * bytes;
+    case ST_PROBE: return S.ht_kind == HT_DIRECT ? 1.0 : 3.0;
+    default: return 0.7;
+  }
+}
+
 struct ColumnSet {
   dpf_ctx* c;
   DevQuery& Q;
@@ -1079,17 +1108,18 @@ dpf_status compile_plan(dpf_ctx* c, const dpf_plan& P, DevQuery& Q, bool* host,
   }
   Q.nsteps = uint32_t(steps.size());
   for (size_t i = 0; i < steps.size(); ++i) Q.steps[i] = steps[order[i]];
+  *share = ScanShare{0, cs.nrows, 1.0, 0.5};
   {
-    double cost = steps.empty() ? 12.0 : bits[order[0]], surv = 1.0;
+    double surv = 1.0;
     for (size_t i = 0; i < order.size(); ++i) {
-      if (i > 0) cost += surv * kSparseCost;
+      const Column& col = c->cols[cs.ids[Q.steps[i].col]];
+      share->cost += step_time(Q.steps[i], col, i == 0, surv);
       surv *= std::min(1.0, sel[order[i]]);
     }
-    for (uint32_t a = 0; a < Q.naggs; ++a) cost += Q.agg_op[a] == DPF_AGG_COUNT ? 0.0 : surv * kSparseCost;
-    // 1 = the star join: 16 for its dense step, 11 for the survivors; a query that reads no page costs its tickets
-    share->cost = std::max(0.25, cost / 27.0);
+    for (uint32_t a = 0; a < Q.naggs; ++a)
+      share->cost += Q.agg_op[a] == DPF_AGG_COUNT ? 0.0 : (Q.agg_op[a] == DPF_AGG_SUM ? 5.0 : 10.0) * surv;
+    share->cost = std::max(0.25, share->cost / kStarTime);
   }
-  *share = ScanShare{0, cs.nrows, 1.0, share->cost};
   if (Q.nsteps != 0) {
     const ZonePart z = zone_part(c->cols[cs.ids[Q.steps[0].col]], Q.steps[0].zlo, Q.steps[0].zhi);
     share->row0 = z.row0;

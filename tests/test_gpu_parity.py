@@ -330,6 +330,32 @@ def test_a_launch_that_met_corrupt_data_fails_every_read(unfused):
         e.close()
 
 
+@pytest.mark.parametrize("tuning", [None, (1024, 256), (16384, 128)])
+def test_batch_of_string_searches_and_integer_queries(eng, tuning):
+    """LIKE, CONTAINS (raw and FSST), PREFIX, star joins and scans of uneven
+    sizes in one launch: rows that cost 0.5 to 10 times a star join's, whose
+    shares are estimates, so that CTAs take over from one another."""
+    ws = []
+    for i, rows in enumerate((300_007, 20_001, 64_000)):
+        like = synth.strings(rows=rows, page_rows=8192, seed=70 + i, text=True)
+        like["query"]["preds"] = [{"col": "s", "op": "like", "args": [b"%a_%e%"]}]
+        ws += [like, synth.star_join(rows=2 * rows + 3, seed=80 + i, page_rows=8192),
+               synth.strings(rows=rows + 77, page_rows=4096, seed=90 + i, text=True, contains=b"ab", codec="fsst"),
+               synth.scan_filter_aggregate(rows=3 * rows, page_rows=8192, seed=60 + i),
+               synth.strings(rows=rows // 2, page_rows=8192, seed=95 + i)]
+    for i, w in enumerate(ws):
+        w["name"] = f"mixed_{i}_{w['name']}"
+        eng.load_workload(w)
+    prep = eng.ctx.prepare([eng.plan(w) for w in ws], dpf.Tuning(*tuning, 0, 0, 0, 0) if tuning else None)
+    try:
+        for _ in range(2):
+            eng.ctx.launch(prep)
+            for i, w in enumerate(ws):
+                assert_same(eng.ctx.read_result(prep, i), expect(w), (i, w["name"]))
+    finally:
+        eng.ctx.release(prep)
+
+
 def test_batch_mixing_lean_and_string_matcher_queries(eng):
     """A batch with one CONTAINS-on-FSST query runs the kernel build with the
     general string matcher for every query in it; the same queries alone run
