@@ -1392,12 +1392,13 @@ __device__ __forceinline__ bool step_adds_gid(const DevStep& S) {
 // aggregation visit every entry once, whatever its position.
 //  - Few rows: a warp scan of the lanes' counts gives each lane its first
 //    slot, and it writes its rows there one after the other.
-//  - From kOrderedRows rows on (and always when the pages come over the host
-//    link, where a sector read twice costs most): in row order, one ballot per
-//    32 rows.  A later round's 32 entries are then neighbours, whose packed
-//    fields share sectors, and the writes fall into distinct banks.
-//  - A tile that lost no row is copied without ballots.
-constexpr uint32_t kOrderedRows = kMB * TB / 4;
+//  - When the pages come over the host link, where a sector read twice costs
+//    most: in row order, one ballot per 32 rows.  A later round's 32 entries are
+//    then neighbours, whose packed fields share sectors, and the writes fall
+//    into distinct banks (star of 17 M rows 411 -> 371 us).  For resident pages
+//    that only lengthened the code (star of 67 M rows 198 us with the ballots
+//    for tiles that keep a quarter of their rows, 194 without; chain 330, 323).
+//  - A tile that lost no row is copied without either.
 template <bool kHost, bool kGid = true>
 __device__ __forceinline__ uint32_t tile_compact(const TileState& T, uint32_t* list, uint32_t n0, uint32_t row_base,
                                                  int lane) {
@@ -1416,7 +1417,7 @@ __device__ __forceinline__ uint32_t tile_compact(const TileState& T, uint32_t* l
       for (int k = 0; k < 4; ++k)
         list[n0 + uint32_t(t * kMB + k * 32 + lane)] =
             (row_base + uint32_t(t * kMB + k * 32 + lane)) | (kGid ? T.gid[t][k] << kRowBits : 0u);
-  } else if (kHost || total >= kOrderedRows) {
+  } else if (kHost) {
     const uint32_t lt = (1u << lane) - 1u;
     uint32_t n = n0;
 #pragma unroll
