@@ -1419,13 +1419,6 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   p->off_rec.resize(size_t(n));
   size_t max_tables = 0;
   uint32_t acc_slots = 0;
-  // SMEM placement: what the opt-in shared memory leaves after the largest
-  // accumulator region, the warps' lists and group buffers, and the plan
-  const int per_cta_fixed = int(kSmemAccSlots * 8) + int(t.threads / 32) * int(kListBytesPerWarp) + 4096;
-  const size_t table_budget =
-      t.ht_placement == DPF_HT_GLOBAL ? 0
-      : t.ht_placement == DPF_HT_SMEM ? size_t(std::max(0, c->smem_optin - per_cta_fixed))
-                                      : size_t(48 * 1024);
   for (int i = 0; i < n; ++i) {
     DevQuery& Q = p->hq[i];
     bool h = false;
@@ -1433,8 +1426,6 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     dpf_status st = compile_plan(c, plans[i], Q, &h, probes, n == 1, &shares[size_t(i)]);
     if (st) return fail(st, "plan %d: %s", i, t_last_error.c_str());
     host |= h;
-    const size_t used = place_tables(Q, table_budget, t.ht_placement == DPF_HT_AUTO);
-    max_tables = std::max(max_tables, used);
     const uint32_t S1 = 1 + Q.naggs;
     Q.use_smem_acc = uint64_t(Q.domain) * S1 <= kSmemAccSlots ? 1u : 0u;
     Q.warp_agg = t.group_agg == DPF_GROUP_AGG_WARP && Q.domain > 1 ? 1u : 0u;
@@ -1445,13 +1436,24 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     p->off_n[size_t(i)] = results; results += 16;
     p->off_rec[size_t(i)] = results; results += align16(uint64_t(std::max<uint32_t>(Q.domain, 1)) * sizeof(dpf_record));
   }
+  bool text = false;
+  for (const DevQuery& q : p->hq) text = text || needs_string_matcher(q);
+  // SMEM placement: what the opt-in shared memory leaves after the largest
+  // accumulator region (with the string search's scratch: after the batch's own
+  // and that, where it is more), the warps' lists, and the plan
+  const int warps = int(t.threads / 32);
+  const int fixed = std::max(int(kSmemAccSlots * 8), int(acc_slots * 8) + (text ? warps * int(kSearchWords * 4) : 0)) +
+                    warps * int(kListBytesPerWarp) + 4096;
+  const size_t table_budget = t.ht_placement == DPF_HT_GLOBAL ? 0
+                              : t.ht_placement == DPF_HT_SMEM ? size_t(std::max(0, c->smem_optin - fixed))
+                                                              : size_t(48 * 1024);
+  for (DevQuery& Q : p->hq)
+    max_tables = std::max(max_tables, place_tables(Q, table_budget, t.ht_placement == DPF_HT_AUTO));
   // Staging ring: a launch stages all of its queries or none; a query can be
   // staged when its first step is an integer step over device-resident
   // pages.  The ring's slots are as wide as the widest mini block of those
   // steps' columns.
   uint32_t stage_bw = 0;
-  bool text = false;
-  for (const DevQuery& q : p->hq) text = text || needs_string_matcher(q);
   if (t.staging == DPF_STAGE_ON && !host && !text) {
     bool all = true;
     for (const DevQuery& Q : p->hq) {

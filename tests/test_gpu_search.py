@@ -38,6 +38,48 @@ def _workload(kind, rows, page_rows, codec, seed):
             "query": {"preds": [], "joins": [], "group": [], "aggs": [{"op": "count"}, {"op": "sum", "cols": ["m"]}]}}, s
 
 
+@pytest.mark.parametrize("keys", [20_000, 75_000, 81_000])
+@pytest.mark.parametrize("codec,op,pat", [("str", "contains", b"abcd"), ("fsst", "contains", b"cdab"), ("str", "like", b"%ab%c_%")])
+def test_search_beside_shared_memory_tables(codec, op, pat, keys):
+    """Join tables placed in shared memory until it is full (81,000 keys of two
+    bytes are within the accumulators' and lists' budget and not within what the
+    search's scratch leaves: that table is probed in device memory)."""
+    w, s = _workload("short", 6007, 4096, codec, keys)
+    rng = np.random.default_rng(keys)
+    dim = {"k": {"codec": "for", "values": rng.permutation(keys).astype(np.int32) + 1},
+           "p": {"codec": "dict", "values": (np.arange(keys) % 1024).astype(np.int32)}}
+    w["tables"]["d"] = {"rows": keys, "page_rows": 4096, "cols": dim}
+    w["tables"]["f"]["cols"]["fk"] = {"codec": "for", "values": rng.integers(1, keys + 1, len(s)).astype(np.int32)}
+    w["name"] += f"_smem_{op}"
+    w["query"] = {"preds": [{"col": "s", "op": op, "args": [pat]}], "group": [{"join": 0, "field": 0}],
+                  "joins": [{"fk": "fk", "dim": "d", "key": "k", "preds": [], "payload": ["p"]}],
+                  "aggs": [{"op": "count"}, {"op": "sum", "cols": ["m"]}, {"op": "sum_mul", "cols": ["m", "m"]}]}
+    want = oracle.run_query(w, from_encoded=False)
+    e = dpf.Engine(device=0)
+    try:
+        for threads in (128, 256):
+            got = e.run(w, tuning=dpf.Tuning(0, threads, dpf.HT_PLACE["smem"], 0, 0, 0))
+            assert got.shape == want.shape and all(np.array_equal(got[f], want[f]) for f in ("key", "count", "val"))
+    finally:
+        e.close()
+
+
+@pytest.mark.parametrize("codec,op,pat", [("str", "contains", b"abcda"), ("fsst", "contains", b"cd"), ("str", "like", b"%cd_b%"),
+                                          ("fsst", "contains", b"\xff")])
+@pytest.mark.parametrize("kind,rows,page_rows", [("escapes", 2500, 128), ("long", 389, 256), ("short", 70_003, 65536)])
+def test_search_over_host_resident_pages(kind, rows, page_rows, codec, op, pat):
+    w, _ = _workload(kind, rows, page_rows, codec, rows + 2)
+    w["query"]["preds"] = [{"col": "s", "op": op, "args": [pat]}]
+    want = oracle.run_query(w, from_encoded=False)
+    e = dpf.Engine(device=0)
+    try:
+        e.load_workload(w, fact_placement="host")
+        got = e.run(w)
+        assert np.array_equal(got["count"], want["count"]) and np.array_equal(got["val"], want["val"])
+    finally:
+        e.close()
+
+
 @pytest.mark.parametrize("codec", ["str", "fsst"])
 @pytest.mark.parametrize("kind,rows,page_rows", [("runs", 3001, 1024), ("escapes", 2500, 128), ("long", 389, 256),
                                                  ("short", 5003, 4096), ("short", 1, 128)])
