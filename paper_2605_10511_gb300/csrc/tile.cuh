@@ -756,12 +756,15 @@ __device__ __forceinline__ uint32_t like_push(const DevStep& S, const uint8_t* b
 
 // Starts of a mini block's 128 strings from the bw-bit fields f of their
 // lengths (length = base + field): st[k] = bytes before row 32k + lane;
-// returns the fields' sum.  Fields of at most 11 bits are summed two to a
-// register (128 of them stay below 2^16 a half).
+// returns the fields' sum.  Fields of at most kPackedBits bits are summed two to
+// a register: a half holds the sum of one group of 32, below 2^16; the groups'
+// totals are added in whole registers.
+constexpr uint32_t kPackedBits = 11;
+static_assert(32u * ((1u << kPackedBits) - 1) < (1u << 16), "a half must not carry into the other");
 __device__ __forceinline__ uint32_t string_starts(const uint32_t (&f)[4], uint32_t base, uint32_t bw, int lane,
                                                   uint32_t (&st)[4]) {
   uint32_t sum;
-  if (bw <= 11) {
+  if (bw <= kPackedBits) {
     uint32_t a = f[0] | (f[1] << 16), b = f[2] | (f[3] << 16);
     const uint32_t a0 = a, b0 = b;
 #pragma unroll

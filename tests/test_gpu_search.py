@@ -80,6 +80,42 @@ def test_search_over_host_resident_pages(kind, rows, page_rows, codec, op, pat):
         e.close()
 
 
+def _lengths(bits, rows, rng):
+    """Lengths whose fields take `bits` bits, most of them at the largest."""
+    top = 2**bits - 1
+    n = np.where(rng.random(rows) < 0.9, top, rng.integers(0, top, rows))
+    n[::128] = 0
+    n[1::128] = top
+    return n
+
+
+@pytest.mark.parametrize("bits", [10, 11, 12])
+@pytest.mark.parametrize("codec", ["str", "fsst"])
+def test_starts_of_strings_with_wide_length_fields(bits, codec):
+    """Mini blocks whose length fields have 11 bits (summed two to a register)
+    and 12 (one), at their largest in every row."""
+    rng = np.random.default_rng(bits)
+    rows = 700
+    n = _lengths(bits, rows, rng)
+    s = [bytes(rng.integers(97, 123, int(k), dtype=np.uint8)) for k in n]
+    s = [x[:-4] + b"%03dz" % (i % 1000) if len(x) > 8 else x for i, x in enumerate(s)]
+    off = np.zeros(rows + 1, np.uint64)
+    off[1:] = np.cumsum([len(x) for x in s])
+    w = {"name": f"wide_{bits}_{codec}", "fact": "f",
+         "tables": {"f": {"rows": rows, "page_rows": 256, "cols": {
+             "s": {"codec": codec, "bytes": np.frombuffer(b"".join(s), np.uint8), "offsets": off},
+             "m": {"codec": "for", "values": np.arange(rows, dtype=np.int32)}}}},
+         "query": {"preds": [], "joins": [], "group": [], "aggs": [{"op": "sum", "cols": ["m"]}]}}
+    e = dpf.Engine(device=0)
+    try:
+        for pat in [b"%03dz" % i for i in (0, 5, 126, 127, 128, 255, 511, 699)] + [b"00z"]:
+            got = e.run(dict(w, query=dict(w["query"], preds=[{"col": "s", "op": "contains", "args": [pat]}])))
+            hit = [i for i, x in enumerate(s) if pat in x]
+            assert int(got["count"][0]) == len(hit) and int(got["val"][0, 0]) == sum(hit), pat
+    finally:
+        e.close()
+
+
 @pytest.mark.parametrize("codec", ["str", "fsst"])
 @pytest.mark.parametrize("kind,rows,page_rows", [("runs", 3001, 1024), ("escapes", 2500, 128), ("long", 389, 256),
                                                  ("short", 5003, 4096), ("short", 1, 128)])
