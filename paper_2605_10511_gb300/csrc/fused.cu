@@ -1,5 +1,5 @@
 // Launch and occupancy of the fused kernel (fused_kernel.cuh): picks one of
-// its six builds for a batch and sizes its dynamic shared memory.
+// its builds for a batch and sizes its dynamic shared memory.
 #include "tile.cuh"
 
 namespace dpf {

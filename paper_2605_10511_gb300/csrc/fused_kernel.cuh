@@ -1,16 +1,18 @@
 // The fused persistent kernel (Sec. 3.2, Sec. 4.1 "fused kernel composition"),
-// as a header: each of fused_lean.cu, fused_text.cu and fused_host.cu
-// compiles two of its six builds (device-resident pages without / with the
-// general string matcher, host-resident pages; 3 and 4 resident CTAs per
-// SM each), so the builds compile in parallel.
+// as a header: fused_lean.cu, fused_text.cu, fused_host.cu and fused_stage.cu
+// each compile two of its builds (device-resident pages without / with the
+// general string matcher, host-resident pages, device-resident pages staged
+// in shared memory; 3 and 4 resident CTAs per SM) and fused_wide.cu those for
+// CTAs of 512 and 1,024 threads, so the builds compile in parallel.
 //
 // One launch executes every query of a batch.  Each warp repeatedly takes a
-// ticket (one chunk of one query's fact table: the outer loop of Sec. 3.2
-// without host intervention), splits the chunk into tiles of TB mini blocks and runs decode -> predicates -> probes -> aggregation on
-// them with all row state in registers.  Per-CTA int64 accumulators live in
+// ticket (a range of rows of one query's fact table: the outer loop of Sec. 3.2
+// without host intervention), splits it into tiles of TB mini blocks and runs
+// decode -> predicates -> probes -> aggregation on them with all row state in
+// registers.  Per-CTA int64 accumulators live in
 // shared memory while the CTA stays on one query; they are added to the
 // query's global accumulators when the CTA moves to another query or exits.
-// The CTA that flushes a query's last chunk turns its accumulators into
+// The CTA that flushes a query's last ticket turns its accumulators into
 // records ordered by key tuple (the record format of Kernel #3, Sec. 3.1) and
 // zeroes the scratch state, so the kernel can be replayed from a CUDA graph.
 #pragma once

@@ -1354,7 +1354,6 @@ constexpr uint32_t kTileRows = kMB * TB;
 constexpr uint32_t kRowBits = 12;
 constexpr uint32_t kSegMbs = (1u << kRowBits) / kMB;  // mini blocks per segment (16)
 constexpr uint32_t kListCap = 1024;                    // entries per warp list
-constexpr int kListUnroll = 1;  // survivor rounds whose loads are issued together (measured best at 1)
 static_assert(kTileRows <= (1u << kRowBits), "row index field too narrow");
 static_assert(kListCap >= kTileRows, "a list must hold one tile");
 static_assert(kListBytesPerWarp == kListCap * 4, "the host's per-warp shared-memory figure");
@@ -1652,42 +1651,32 @@ template <bool kHost, int kOp>
 __device__ __forceinline__ uint32_t list_step_t(const DevQuery& Q, const DevStep& S, const PageState& P,
                                                 uint32_t seg_mb, uint32_t* list, uint32_t n, const uint8_t* stab,
                                                 int lane, unsigned int* status) {
-  // Rounds of 32 survivors are taken kListUnroll at a time: their entries
-  // and packed values are all loaded before any is used, so the warp keeps
-  // that many independent loads in flight.  Compacted entries are written
-  // only after the group's entries were read, never ahead of them.
+  // A round takes 32 survivors (two or four rounds with their loads issued
+  // together measured slower: star of 67 M rows 243 us, 254 and 286).  Kept
+  // entries are written after the round's were read, never ahead of them.
   const uint32_t lt = (1u << lane) - 1u;
   uint32_t out = 0;
-  for (uint32_t i0 = 0; i0 < n; i0 += 32 * kListUnroll) {
-    uint32_t r[kListUnroll], gid[kListUnroll], v[kListUnroll];
-    bool valid[kListUnroll];
-#pragma unroll
-    for (int u = 0; u < kListUnroll; ++u) {
-      valid[u] = i0 + 32u * u + lane < n;
-      const uint32_t e = valid[u] ? list[i0 + 32u * u + lane] : 0u;
-      r[u] = e & ((1u << kRowBits) - 1u);
-      gid[u] = e >> kRowBits;
-    }
-#pragma unroll
-    for (int u = 0; u < kListUnroll; ++u) v[u] = point_value<kHost>(Q, S.col, P, seg_mb, r[u], valid[u]);
+  for (uint32_t i0 = 0; i0 < n; i0 += 32) {
+    const bool valid = i0 + lane < n;
+    const uint32_t e = valid ? list[i0 + lane] : 0u;
+    const uint32_t r = e & ((1u << kRowBits) - 1u);
+    uint32_t gid = e >> kRowBits;
+    const uint32_t v = point_value<kHost>(Q, S.col, P, seg_mb, r, valid);
     __syncwarp();
-#pragma unroll
-    for (int u = 0; u < kListUnroll; ++u) {
-      bool keep;
-      if (kOp <= PM_OPEN) {
-        keep = row_probe<kOp>(S, stab, v[u], valid[u], gid[u], status);
-      } else if (kOp == 5) {
-        gid[u] += v[u] * S.key_mul;
-        keep = valid[u];
-      } else if (kOp == 6 || kOp == 7) {
-        keep = valid[u] && (((v[u] - uint32_t(S.lo)) <= uint32_t(S.hi) - uint32_t(S.lo)) != (kOp == 7));
-      } else {
-        keep = valid[u] && step_pred(S, int32_t(v[u]));
-      }
-      const uint32_t m = __ballot_sync(kFull, keep);
-      if (keep) list[out + __popc(m & lt)] = r[u] | (gid[u] << kRowBits);
-      out += __popc(m);
+    bool keep;
+    if (kOp <= PM_OPEN) {
+      keep = row_probe<kOp>(S, stab, v, valid, gid, status);
+    } else if (kOp == 5) {
+      gid += v * S.key_mul;
+      keep = valid;
+    } else if (kOp == 6 || kOp == 7) {
+      keep = valid && (((v - uint32_t(S.lo)) <= uint32_t(S.hi) - uint32_t(S.lo)) != (kOp == 7));
+    } else {
+      keep = valid && step_pred(S, int32_t(v));
     }
+    const uint32_t m = __ballot_sync(kFull, keep);
+    if (keep) list[out + __popc(m & lt)] = r | (gid << kRowBits);
+    out += __popc(m);
   }
   __syncwarp();
   return out;
