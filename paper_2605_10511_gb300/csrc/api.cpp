@@ -111,6 +111,7 @@ struct Prep {
   // the launch's status word, then each query's record count and records.
   uint8_t* results = nullptr;
   std::vector<uint64_t> off_n, off_rec;  // byte offsets of the queries' counts and records
+  uint8_t* up = nullptr;          // pinned copy of what dq holds, while its upload may still read it
   FusedLaunch L{};
   dpf_tuning tuning{};
   cudaEvent_t ev = nullptr;
@@ -1367,6 +1368,7 @@ dpf_status release_prep(dpf_ctx* c, Prep* p) {
   dev_free(c, p->dq);  // with the ticket table and the scheduler state behind it
   dev_free(c, p->scratch);
   pin_free(c, p->results);
+  pin_free(c, p->up);
   dev_free(c, p->unf_scratch);
   return DPF_OK;
 }
@@ -1506,7 +1508,8 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   dpf_status st;
   if ((st = dev_alloc(c, scratch, reinterpret_cast<void**>(&p->scratch))) ||
       (st = dev_alloc(c, up_bytes, reinterpret_cast<void**>(&p->dq))) ||
-      (st = pin_alloc(c, results, reinterpret_cast<void**>(&p->results)))) {
+      (st = pin_alloc(c, results, reinterpret_cast<void**>(&p->results))) ||
+      (st = pin_alloc(c, up_bytes, reinterpret_cast<void**>(&p->up)))) {
     const std::string msg = t_last_error;
     release_prep(c, p.get());
     return fail(st, "%s", msg.c_str());
@@ -1522,16 +1525,21 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     Q.out = p->results + p->off_rec[size_t(i)];
     *reinterpret_cast<uint32_t*>(p->results + p->off_n[size_t(i)]) = 0;
   }
-  std::vector<uint8_t> up(up_bytes, 0);
-  std::memcpy(up.data(), p->hq.data(), at_begin);
-  std::memcpy(up.data() + at_begin, qbegin.data(), 8 * qbegin.size());
+  // uploaded from pinned memory: a pageable source of more than 64 KB (26 plans)
+  // may make the call wait for the stream's earlier work
+  std::memcpy(p->up, p->hq.data(), at_begin);
+  std::memcpy(p->up + at_begin, qbegin.data(), 8 * qbegin.size());
+  const uint64_t filled = at_begin + 8 * qbegin.size();
+  std::memset(p->up + filled, 0, up_bytes - filled);
   const cudaStream_t us = on ? *on : c->io;
   cudaError_t e = cudaMemsetAsync(p->scratch, 0, scratch, us);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(p->dq, up.data(), up.size(), cudaMemcpyHostToDevice, us);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(p->dq, p->up, up_bytes, cudaMemcpyHostToDevice, us);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev, cudaEventDisableTiming);
   if (e != cudaSuccess || !on) {
     const cudaError_t e2 = cudaStreamSynchronize(us);  // nothing may still write blocks that are freed
     if (e == cudaSuccess) e = e2;
+    pin_free(c, p->up);  // uploaded
+    p->up = nullptr;
   }
   if (e != cudaSuccess) {
     release_prep(c, p.get());

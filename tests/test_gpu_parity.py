@@ -296,6 +296,26 @@ def test_fsst_codes_outside_the_table_are_rejected(eng):
     assert ex.value.status == -9  # DPF_ECORRUPT
 
 
+def test_a_large_one_shot_batch_does_not_wait_for_its_stream(eng):
+    """dpf_execute_plan of 60 plans (150 KB of them) on a stream that is busy for
+    100 ms or so returns long before the stream gets there."""
+    import torch
+    w = synth.scan_filter_aggregate(rows=5000, page_rows=1024)
+    eng.load_workload(w)
+    plans = [eng.plan(w) for _ in range(60)]
+    want = expect(w)
+    s = torch.cuda.Stream()
+    for busy in (False, True, True):     # the first call allocates
+        if busy:
+            with torch.cuda.stream(s):
+                torch.cuda._sleep(200_000_000)
+        ids = eng.ctx.execute(plans, s)
+        idle = s.query()
+        for q in ids:
+            assert_same(eng.ctx.fetch(q), want, "one of 60")
+        assert not (busy and idle), "the call waited for the stream"
+
+
 @pytest.mark.parametrize("unfused", [False, True])
 def test_a_launch_that_met_corrupt_data_fails_every_read(unfused):
     """A dictionary code beyond the dictionary drops its row: no query of that
