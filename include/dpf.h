@@ -73,7 +73,8 @@ dpf_status dpf_create(dpf_ctx** out, int32_t device, uint64_t hbm_budget,
 /* Waits for the context's work, frees every object it owns. */
 dpf_status dpf_destroy(dpf_ctx* ctx);
 /* Device bytes held by the context's live objects (columns, hash tables,
- * prepared batches; their results lie in pinned host memory).  Without
+ * prepared batches; a batch's results of up to 16 MiB lie in pinned host
+ * memory, larger ones in device memory).  Without
  * allocation hooks, freed blocks of up to 1 GiB (8 GiB in all) are kept for
  * reuse and not counted here; with a budget, live plus kept bytes stay within
  * it.  Of the pinned result blocks at most 64 MiB are kept when freed.
@@ -459,9 +460,9 @@ dpf_status dpf_release(dpf_ctx* ctx, dpf_prep_id prep);
  * the device status word. */
 dpf_status dpf_autotune(dpf_ctx* ctx, const dpf_plan* plans, int32_t n, void* stream, uint32_t reps,
                         dpf_tuning* best, float* best_ms);
-/* Device bytes one plan occupies while it runs (int64 accumulators of its
- * group domain, result records, device plan), for admission by memory
- * footprint.  Errors: as dpf_prepare. */
+/* Bytes one plan occupies while it runs (int64 accumulators of its group
+ * domain, device plan, and its result records, wherever the batch's lie), for
+ * admission by memory footprint.  Errors: as dpf_prepare. */
 dpf_status dpf_plan_footprint(dpf_ctx* ctx, const dpf_plan* plan, uint64_t* bytes);
 
 /* The unfused baseline: the same single plan prepared as a chain of one

@@ -109,7 +109,10 @@ struct Prep {
   // Results, in mapped pinned host memory that the kernels write directly, so
   // a read waits for the launch's event and copies nothing from the device:
   // the launch's status word, then each query's record count and records.
+  // Beyond kPinResults the counts and records are in device memory (outputs),
+  // where the context's budget and block cache hold.
   uint8_t* results = nullptr;
+  uint8_t* outputs = nullptr;            // counts and records: results, or a device block
   std::vector<uint64_t> off_n, off_rec;  // byte offsets of the queries' counts and records
   uint8_t* up = nullptr;          // pinned copy of what dq holds, while its upload may still read it
   FusedLaunch L{};
@@ -252,6 +255,9 @@ void dev_free(dpf_ctx* c, void* p) {
 }
 
 constexpr uint64_t kPinCacheMaxBytes = uint64_t(64) << 20;  // freed pinned bytes kept for reuse
+// Largest results of a batch in pinned memory: four such blocks are kept when
+// freed, where a larger one would be allocated anew by every prepare.
+constexpr uint64_t kPinResults = uint64_t(16) << 20;
 
 // Mapped pinned host memory, the same address on the host and the device.
 dpf_status pin_alloc(dpf_ctx* c, uint64_t bytes, void** out) {
@@ -1367,6 +1373,7 @@ dpf_status release_prep(dpf_ctx* c, Prep* p) {
   if (p->ev) cudaEventDestroy(p->ev);
   dev_free(c, p->dq);  // with the ticket table and the scheduler state behind it
   dev_free(c, p->scratch);
+  if (p->outputs != p->results) dev_free(c, p->outputs);
   pin_free(c, p->results);
   pin_free(c, p->up);
   dev_free(c, p->unf_scratch);
@@ -1508,7 +1515,8 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   dpf_status st;
   if ((st = dev_alloc(c, scratch, reinterpret_cast<void**>(&p->scratch))) ||
       (st = dev_alloc(c, up_bytes, reinterpret_cast<void**>(&p->dq))) ||
-      (st = pin_alloc(c, results, reinterpret_cast<void**>(&p->results))) ||
+      (st = pin_alloc(c, results <= kPinResults ? results : 64, reinterpret_cast<void**>(&p->results))) ||
+      (results > kPinResults && (st = dev_alloc(c, results, reinterpret_cast<void**>(&p->outputs)))) ||
       (st = pin_alloc(c, up_bytes, reinterpret_cast<void**>(&p->up)))) {
     const std::string msg = t_last_error;
     release_prep(c, p.get());
@@ -1516,14 +1524,14 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
   }
   p->dqbegin = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(p->dq) + at_begin);
   p->sched = reinterpret_cast<Sched*>(reinterpret_cast<uint8_t*>(p->dq) + at_sched);
+  if (!p->outputs) p->outputs = p->results;
   std::memset(p->results, 0, 64);
   for (int i = 0; i < n; ++i) {
     DevQuery& Q = p->hq[i];
     Q.acc = reinterpret_cast<unsigned long long*>(p->scratch + off_acc[i]);
     Q.done = reinterpret_cast<unsigned int*>(p->scratch + off_done[i]);
-    Q.out_n = reinterpret_cast<unsigned int*>(p->results + p->off_n[size_t(i)]);
-    Q.out = p->results + p->off_rec[size_t(i)];
-    *reinterpret_cast<uint32_t*>(p->results + p->off_n[size_t(i)]) = 0;
+    Q.out_n = reinterpret_cast<unsigned int*>(p->outputs + p->off_n[size_t(i)]);
+    Q.out = p->outputs + p->off_rec[size_t(i)];
   }
   // uploaded from pinned memory: a pageable source of more than 64 KB (26 plans)
   // may make the call wait for the stream's earlier work
@@ -1591,7 +1599,7 @@ dpf_status wait_event(cudaEvent_t ev, int32_t timeout_ms) {
   }
 }
 
-dpf_status read_result(Prep* p, int32_t i, dpf_record* buf, uint64_t cap, uint64_t* n_out,
+dpf_status read_result(dpf_ctx* c, Prep* p, int32_t i, dpf_record* buf, uint64_t cap, uint64_t* n_out,
                        int32_t timeout_ms) {
   if (i < 0 || i >= p->nq) return fail(DPF_EINVAL, "query index %d out of range", i);
   if (!p->launched) return fail(DPF_EINVAL, "batch %d was never launched", p->id);
@@ -1599,8 +1607,14 @@ dpf_status read_result(Prep* p, int32_t i, dpf_record* buf, uint64_t cap, uint64
   if (st) return st;
   // the launch's kernels wrote its status, counts and records here
   uint32_t status, n;
+  const bool pinned = p->outputs == p->results;
   std::memcpy(&status, p->results, 4);
-  std::memcpy(&n, p->results + p->off_n[size_t(i)], 4);
+  if (pinned) {
+    std::memcpy(&n, p->outputs + p->off_n[size_t(i)], 4);
+  } else {
+    CUDA_TRY(cudaMemcpyAsync(&n, p->outputs + p->off_n[size_t(i)], 4, cudaMemcpyDeviceToHost, c->io));
+    CUDA_TRY(cudaStreamSynchronize(c->io));
+  }
   if (status) {  // of the whole launch: every query of it reports the error
     if (status & S_CORRUPT) return fail(DPF_ECORRUPT, "device reported corrupt data (status %u)", status);
     return fail(DPF_EINTERNAL, "device reported an internal error (status %u)", status);
@@ -1609,7 +1623,13 @@ dpf_status read_result(Prep* p, int32_t i, dpf_record* buf, uint64_t cap, uint64
   if (cap < n) return fail(DPF_ETRUNC, "need %u records", n);
   if (n) {
     if (!buf) return fail(DPF_EINVAL, "buf is NULL");
-    std::memcpy(buf, p->results + p->off_rec[size_t(i)], uint64_t(n) * sizeof(dpf_record));
+    const uint8_t* from = p->outputs + p->off_rec[size_t(i)];
+    if (pinned) {
+      std::memcpy(buf, from, uint64_t(n) * sizeof(dpf_record));
+    } else {
+      CUDA_TRY(cudaMemcpyAsync(buf, from, uint64_t(n) * sizeof(dpf_record), cudaMemcpyDeviceToHost, c->io));
+      CUDA_TRY(cudaStreamSynchronize(c->io));
+    }
   }
   return DPF_OK;
 }
@@ -2678,7 +2698,7 @@ dpf_status dpf_read_result(dpf_ctx* c, dpf_prep_id id, int32_t i, dpf_record* bu
   DeviceGuard g(c->device);
   Prep* p = find_prep(c, id);
   if (!p) return fail(DPF_EINVAL, "unknown batch %d", id);
-  return read_result(p, i, buf, cap, n_out, timeout_ms);
+  return read_result(c, p, i, buf, cap, n_out, timeout_ms);
 }
 
 dpf_status dpf_prepare_unfused(dpf_ctx* c, const dpf_plan* plan, dpf_prep_id* out) {
@@ -2852,7 +2872,7 @@ dpf_status dpf_fetch_result(dpf_ctx* c, dpf_query_id id, dpf_record* buf, uint64
   Prep* p = find_prep(c, dpf_prep_id(id >> 20));
   const int32_t i = int32_t(id & 0xfffff);
   if (!p || !p->oneshot || i >= p->nq || p->fetched[i]) return fail(DPF_ENOTFOUND, "unknown or fetched query id %lld", (long long)id);
-  dpf_status st = read_result(p, i, buf, cap, n_out, timeout_ms);
+  dpf_status st = read_result(c, p, i, buf, cap, n_out, timeout_ms);
   if (st) return st;
   p->fetched[i] = 1;
   if (std::all_of(p->fetched.begin(), p->fetched.end(), [](char f) { return f != 0; })) {

@@ -296,6 +296,44 @@ def test_fsst_codes_outside_the_table_are_rejected(eng):
     assert ex.value.status == -9  # DPF_ECORRUPT
 
 
+def test_results_beyond_the_pinned_limit():
+    """24 queries of 65,536 groups each (75 MB of records): counted as device
+    memory, given back and used again; a small batch's are not counted."""
+    rng = np.random.default_rng(12)
+    n = 150_001
+    a, b = (np.concatenate([np.arange(256), rng.integers(0, 256, n - 256)]).astype(np.int32) for _ in range(2))
+    v = rng.integers(-1000, 1000, n).astype(np.int32)
+    w = {"name": "wide_groups", "fact": "f", "tables": {"f": {"rows": n, "page_rows": 8192, "cols": {
+        "a": {"codec": "dict", "values": a}, "b": {"codec": "dict", "values": b}, "v": {"codec": "for", "values": v}}}},
+        "query": {"preds": [], "joins": [], "group": [{"col": "a"}, {"col": "b"}], "aggs": [{"op": "sum", "cols": ["v"]}]}}
+    gid = a.astype(np.int64) * 256 + b
+    count = np.bincount(gid, minlength=65536)
+    total = np.bincount(gid, weights=v, minlength=65536).astype(np.int64)
+    have = np.nonzero(count)[0]
+    e = dpf.Engine(device=0)
+    try:
+        e.load_workload(w)
+        plan = e.plan(w)
+        base = e.ctx.memory_used()
+        prep = e.ctx.prepare([plan])
+        small = e.ctx.memory_used() - base
+        assert small < 65536 * 48                      # accumulators and plan
+        e.ctx.release(prep)
+        for _ in range(3):
+            prep = e.ctx.prepare([plan] * 24)
+            assert e.ctx.memory_used() - base >= 24 * 65536 * 48
+            for _ in range(2):
+                e.ctx.launch(prep)
+                for i in (0, 11, 23):
+                    got = e.ctx.read_result(prep, i)
+                    assert np.array_equal(got["key"][:, 0] * 256 + got["key"][:, 1], have)
+                    assert np.array_equal(got["count"], count[have]) and np.array_equal(got["val"][:, 0], total[have])
+            e.ctx.release(prep)
+            assert e.ctx.memory_used() == base
+    finally:
+        e.close()
+
+
 def test_a_large_one_shot_batch_does_not_wait_for_its_stream(eng):
     """dpf_execute_plan of 60 plans (150 KB of them) on a stream that is busy for
     100 ms or so returns long before the stream gets there."""
