@@ -236,7 +236,8 @@ dpf_status dev_alloc(dpf_ctx* c, uint64_t bytes, void** out) {
   return DPF_OK;
 }
 
-void dev_free(dpf_ctx* c, void* p) {
+// keep: the block is kept for reuse while the kept blocks stay within that.
+void dev_free(dpf_ctx* c, void* p, uint64_t keep = kCacheMaxBytes) {
   if (!p) return;
   auto it = c->dev_sizes.find(p);
   if (it == c->dev_sizes.end()) return;
@@ -245,7 +246,7 @@ void dev_free(dpf_ctx* c, void* p) {
   c->dev_sizes.erase(it);
   if (c->has_hooks) {
     c->hooks.free(p, c->hooks.user);
-  } else if (bytes <= kCacheMaxBlock && c->cached + bytes <= kCacheMaxBytes &&
+  } else if (bytes <= kCacheMaxBlock && c->cached + bytes <= keep &&
              (!c->budget || c->used + c->cached + bytes <= c->budget)) {
     c->cache.emplace(bytes, p);
     c->cached += bytes;
@@ -356,13 +357,15 @@ dpf_status upload(dpf_ctx* c, void* dst, const void* src, uint64_t bytes) {
   return DPF_OK;
 }
 
-// Device blocks of one call, freed when it ends.
+// Device blocks of one call, freed when it ends.  They are as large as the
+// column loaded, so only kStagingKeep bytes of them stay for the next load.
+constexpr uint64_t kStagingKeep = uint64_t(64) << 20;
 struct Staging {
   dpf_ctx* c;
   std::vector<void*> blocks;
   ~Staging() {
     cudaStreamSynchronize(c->io);  // nothing of the call may still use them
-    for (void* p : blocks) dev_free(c, p);
+    for (void* p : blocks) dev_free(c, p, kStagingKeep);
   }
   template <class T>
   bool get(uint64_t count, T** out) {
