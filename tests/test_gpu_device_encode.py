@@ -63,6 +63,53 @@ def test_a_load_gives_its_raw_values_back():
         assert free - torch.cuda.mem_get_info(0)[0] <= 100 << 20
 
 
+def _workload(enc_cols, page_rows, n, preds, group, name):
+    return {"name": name, "fact": "f", "tables": {"f": {"rows": n, "page_rows": page_rows, "cols": enc_cols}},
+            "query": {"preds": preds, "joins": [], "group": group, "aggs": [{"op": "count"}, {"op": "sum", "cols": ["m"]}]}}
+
+
+@pytest.mark.parametrize("codec,page_rows", [("for", 1024), ("delta", 4096), ("dict", 1024)])
+def test_zones_and_dictionaries_made_on_the_device(codec, page_rows):
+    """Ranges that skip most pages, and a group-by over the dictionary, give the
+    same records on the column encoded on the device and on the one loaded from
+    the host encoder's pages, and those of the values themselves."""
+    rng = np.random.default_rng(page_rows)
+    n = 50_021
+    top = {"for": 2**31 - 1, "delta": 2_000_000_000, "dict": 40_000}[codec]
+    v = np.sort(rng.integers(-top, top, n)).astype(np.int32)
+    if codec == "dict":
+        v = (v // 97 * 97).astype(np.int32)
+    if codec == "for":                          # unsorted inside a page, sorted over pages
+        for p in range(0, n, page_rows):
+            v[p:p + page_rows] = rng.permutation(v[p:p + page_rows])
+    m = rng.integers(1, 1000, n).astype(np.int32)
+    cols = {"v": {"codec": codec, "values": v}, "m": {"codec": "for", "values": m}}
+    lo, hi = int(np.sort(v)[n // 3]), int(np.sort(v)[n // 3 + 700])
+    ranges = [(lo, hi), (int(v.min()), int(v.min())), (int(v.max()), int(v.max())), (hi, lo - 1), (-2**31, lo), (int(v[n // 2]),) * 2]
+    e = dpf.Engine(device=0)
+    try:
+        dev = _workload(cols, page_rows, n, [], [], f"dev_{codec}")
+        e.load_workload(dev)
+        host = _workload(cols, page_rows, n, [], [], f"host_{codec}")
+        e.tables[(host["name"], "f")] = 991
+        for k, c in cols.items():
+            e.cols[(host["name"], "f", k)] = e.ctx.load_encoded(dpf.encode_column(c, page_rows), table=991)
+        group = [{"col": "v"}] if codec == "dict" and np.unique(v).size <= 65536 else []
+        for a, b in ranges:
+            keep = (v >= a) & (v <= b)
+            got = []
+            for w in (dev, host):
+                q = dict(w, query=dict(w["query"], preds=[{"col": "v", "op": "between", "args": [a, b]}], group=group))
+                got.append(e.run(q))
+            assert got[0].tobytes() == got[1].tobytes(), (codec, a, b)
+            assert int(got[0]["count"].sum()) == int(keep.sum()) and int(got[0]["val"][:, 1].sum()) == int(m[keep].sum())
+            if group:
+                u, c = np.unique(v[keep], return_counts=True)
+                assert np.array_equal(got[0]["key"][:, 0], u) and np.array_equal(got[0]["count"], c)
+    finally:
+        e.close()
+
+
 def test_refusals_stay():
     off = np.arange(40001, dtype=np.uint64)
     off[100] = 0
