@@ -154,7 +154,7 @@ dpf_status dpf_load_encoded(dpf_ctx* ctx, const dpf_column_desc* desc, const uin
  * least 16,384 rows and DICT columns of at least 1,024 (values spanning at
  * most 2^20) that are placed in device memory are encoded on the device; the
  * call then holds their raw values there while it runs (of which blocks of at
- * most 64 MiB in all are kept for reuse), and encodes on the host when they
+ * most 256 MiB in all are kept for reuse), and encodes on the host when they
  * do not fit.  Everything else is encoded on the host and
  * uploaded (dpf_load_encoded).  The caller keeps ownership of `values` /
  * `str_offsets`. */

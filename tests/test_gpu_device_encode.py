@@ -47,20 +47,20 @@ def test_pages_equal_the_host_encoders(n, page_rows):
 
 
 def test_a_load_gives_its_raw_values_back():
-    """256 MB of values that encode to 4 MB: what a load leaves allocated is the
-    pages and at most 64 MiB of blocks for the next one."""
+    """Half a GB of values that encode to 8 MB: what a load leaves allocated is the
+    pages and at most 256 MiB of blocks for the next one."""
     import torch
-    n = 1 << 26
+    n = 1 << 27
     with dpf.Context(0) as ctx:
         ctx.load_column({"codec": "for", "values": np.arange(20_000, dtype=np.int32)}, table=1)
         free = torch.cuda.mem_get_info(0)[0]
         for _ in range(2):
             cid = ctx.load_column({"codec": "for", "values": np.zeros(n, np.int32)}, table=2)
-            assert ctx.column_info(cid)["encoded_bytes"] < 8 << 20
-            assert free - torch.cuda.mem_get_info(0)[0] <= 100 << 20
+            assert ctx.column_info(cid)["encoded_bytes"] < 16 << 20
+            assert free - torch.cuda.mem_get_info(0)[0] <= 300 << 20
         for _ in range(2):   # small ones are kept
             ctx.load_column({"codec": "for64", "values": np.arange(1 << 20, dtype=np.int64)}, table=3)
-        assert free - torch.cuda.mem_get_info(0)[0] <= 100 << 20
+        assert free - torch.cuda.mem_get_info(0)[0] <= 300 << 20
 
 
 def _workload(enc_cols, page_rows, n, preds, group, name):
