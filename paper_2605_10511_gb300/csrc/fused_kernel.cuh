@@ -526,13 +526,23 @@ __device__ void load_smem_tables(const DevQuery& Q, uint8_t* stab) {
   }
 }
 
-// Batches: a ticket of another CTA's run, when this CTA's is used up.  A run's
-// cost is an estimate, so the CTAs that finish early take over from those that
-// hold most.  The lanes look at 32 CTAs spread over the grid; the one with the
-// most tickets left is drawn from, unless it has no more than its own warps are
-// about to draw.  Returns the ticket, or ~0 when nothing is worth it.  The CTA's
-// warps follow one another (CtaState::victim), so that they stay on one query.
-__device__ __noinline__ unsigned long long steal_ticket(unsigned int* drawn, uint64_t owned, CtaState& cs, int lane) {
+// Batches: the warp's next ticket, from its CTA's run, or from another CTA's
+// when that is used up.  A run's cost is an estimate, so the CTAs that finish
+// early take over from those that hold most: the lanes look at 32 CTAs spread
+// over the grid, and the one with the most tickets left is drawn from, unless it
+// has no more than its own warps are about to draw.  Returns the ticket, or ~0
+// when nothing is worth it.  The CTA's warps follow one another
+// (CtaState::victim), so that they stay on one query.  Out of line: inside the
+// loop over tickets it cost launches of one small query up to 1.5 us.
+__device__ __noinline__ unsigned long long draw_batch(unsigned int* drawn, uint64_t owned, CtaState& cs, int lane) {
+  unsigned long long t = ~0ull;
+  if (lane == 0) {
+    const uint32_t v = *const_cast<volatile unsigned int*>(&cs.victim);
+    const uint64_t i = owned * v / gridDim.x + atomicAdd(drawn + v, 1u);
+    if (i < owned * (v + 1) / gridDim.x) t = i;
+  }
+  t = __shfl_sync(kFull, t, 0);
+  if (t != ~0ull) return t;
   for (uint32_t k = 1; k <= 4; ++k) {
     const uint32_t v = uint32_t((uint64_t(blockIdx.x) + k + uint64_t(lane) * gridDim.x / 32) % gridDim.x);
     const uint64_t v0 = owned * v / gridDim.x, v1 = owned * (v + 1) / gridDim.x;
@@ -540,7 +550,6 @@ __device__ __noinline__ unsigned long long steal_ticket(unsigned int* drawn, uin
     const uint32_t best = __reduce_max_sync(kFull, left);
     if (best <= (blockDim.x >> 5)) return ~0ull;
     const int w = __ffs(__ballot_sync(kFull, left == best)) - 1;
-    unsigned long long t = ~0ull;
     if (lane == w) {
       const uint32_t i = atomicAdd(drawn + v, 1u);
       if (i < size) {
@@ -577,7 +586,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
   // CTA alike), drawn with a shared-memory counter, so a small launch's warps
   // need no global atomic.  Of a batch's it is a run, so that the CTA stays on
   // one query, or few, drawn with the CTA's counter in `drawn`, so that others
-  // can take over (steal_ticket).  Then the warps draw from the `pool` of small
+  // can take over (draw_batch).  Then the warps draw from the `pool` of small
   // tickets that all CTAs share (sched->next).  The CTA meets only when its warps' tickets
   // leave the current query: it flushes that query's accumulators and moves to
   // the smallest query any warp holds.
@@ -595,13 +604,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) fused_kernel(const DevQu
   // query's first owned ticket, qbegin[nq + 1 ..] = its first pool ticket.
   auto draw = [&](unsigned long long& t) -> int {
     if (drawn != nullptr) {
-      if (lane == 0) {
-        const uint32_t v = *const_cast<volatile unsigned int*>(&cs.victim);
-        const uint64_t i = owned * v / gridDim.x + atomicAdd(drawn + v, 1u);
-        t = i < owned * (v + 1) / gridDim.x ? i : ~0ull;
-      }
-      t = __shfl_sync(kFull, t, 0);
-      if (t == ~0ull) t = steal_ticket(drawn, owned, cs, lane);
+      t = draw_batch(drawn, owned, cs, lane);
       if (t == ~0ull) return INT_MAX;
     } else {
       unsigned int x = 0;

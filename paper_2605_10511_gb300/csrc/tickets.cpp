@@ -32,15 +32,17 @@ void cut(DevQuery& Q, uint64_t rows, uint64_t big, uint64_t small, uint64_t tail
 
 // One ticket per warp, of about per_warp rows.  A ticket that crosses a page
 // is two runs of tiles, one after the other, which costs about as long as 256
-// more cheap rows (a scan of 1 M rows: 17 against 14 us); so when a page's
-// equal tickets are not much larger than that, none crosses a page.
+// more rows of a star join or scan (a scan of 1 M rows: 17 against 14 us; a star
+// of 4.1 M rows in pages of 4,096: 35 against 30), fewer of a dearer query; so
+// when a page's equal tickets are not much larger than that, none crosses a
+// page.
 void cut_once(DevQuery& Q, const ScanShare& S, uint64_t per_warp, uint64_t warps) {
   const uint64_t P = Q.page_rows, big = round_up(per_warp, kMB);
   cut(Q, S.rows, big, 0, 0);
   if (big >= P) return;
   for (uint64_t per = (P + big - 1) / big; per > 0; --per) {
     const uint64_t rows = round_up((P + per - 1) / per, kMB), n = (P + rows - 1) / rows;  // n <= per tickets a page
-    if (double(rows) > double(big) + 256.0 / S.cost) return;
+    if (double(rows) > double(big) + std::min(256.0, 320.0 / S.cost)) return;
     const uint64_t count = S.rows / P * n + (S.rows % P + rows - 1) / rows;
     if (count > std::max(warps, Q.nchunks)) continue;
     Q.chunk_rows = uint32_t(rows);
@@ -75,7 +77,7 @@ void cut_once(DevQuery& Q, const ScanShare& S, uint64_t per_warp, uint64_t warps
 //    and loads the next one's tables, which a pool drawn in query order makes
 //    every CTA do (24 queries of up to 4 M rows: 138 us, with a fifth of the
 //    rows in a pool 220).  What the estimates miss is taken over from CTAs that
-//    have most left (steal_ticket).  Tickets of at most kBatchRows rows.
+//    have most left (draw_batch).  Tickets of at most kBatchRows rows.
 //  - A batch of large queries (kInOrderRows each on average) is drawn whole
 //    from the pool, query by query, each query's last rows in small tickets:
 //    the CTAs' meetings at its few switches cost little and no estimate of a
