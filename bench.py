@@ -52,7 +52,7 @@ def _peaks():
         return 6800.0, "fallback"
 
 
-KERNEL_SOURCES = ("fused.cu", "fused_kernel.cuh", "fused_lean.cu", "fused_text.cu", "fused_host.cu", "fused_stage.cu",
+KERNEL_SOURCES = ("fused.cu", "tickets.cpp", "fused_kernel.cuh", "fused_lean.cu", "fused_text.cu", "fused_host.cu", "fused_stage.cu",
                   "fused_wide.cu", "tile.cuh",
                   "dpf_device.cuh", "dpf_internal.h", "kernels.h")
 

@@ -371,8 +371,8 @@ typedef struct dpf_tuning {
                             resident pages only                              */
   int32_t group_agg;     /* enum dpf_group_agg: how grouped aggregates are added
                             into the accumulators: one int64 atomic per row,
-                            or warp-aggregated (lanes of a round holding the
-                            same group, found by __match_any_sync, add once) */
+                            or warp-aggregated (the lanes of a round holding
+                            its first row's group add once)                  */
 } dpf_tuning;
 enum dpf_staging { DPF_STAGE_DEFAULT = 0, DPF_STAGE_ON = 1, DPF_STAGE_OFF = 2 };
 enum dpf_group_agg { DPF_GROUP_AGG_DEFAULT = 0, DPF_GROUP_AGG_WARP = 1, DPF_GROUP_AGG_ATOMIC = 2 };

@@ -17,7 +17,7 @@ constexpr uint32_t kMbPerWarpTile = 4;
 // shared memory fits; the launch configuration (ctas_per_sm) picks one.
 constexpr int kFusedMinBlocksLo = 3;
 constexpr int kFusedMinBlocksHi = 4;
-// Rows of one scheduling ticket (one warp's unit of work) unless tuned.
+// Most rows of one scheduling ticket (one warp's unit of work) unless tuned.
 constexpr uint32_t kDefaultChunkRows = 4096;
 // Rows from which one query takes the 1,024-thread build unless tuned.
 constexpr uint64_t kWideRows = uint64_t(1) << 23;

@@ -75,9 +75,14 @@ void cut_once(DevQuery& Q, const ScanShare& S, uint64_t per_warp, uint64_t warps
 //  - A batch is cut into tickets of about equal cost, the same number for every
 //    warp, all owned, in runs: a CTA that changes its query flushes it, meets
 //    and loads the next one's tables, which a pool drawn in query order makes
-//    every CTA do (24 queries of up to 4 M rows: 138 us, with a fifth of the
+//    every CTA do (24 queries of up to 4 M rows: 148 us, with a fifth of the
 //    rows in a pool 220).  What the estimates miss is taken over from CTAs that
-//    have most left (draw_batch).  Tickets of at most kBatchRows rows.
+//    have most left (draw_batch; without it 32 queries over a year of 8 M rows
+//    1,380 us, with it 690).  A ticket costs at most what 4,096 rows of a star
+//    join do, and has at most kBatchRows rows, as little as a meeting waits for:
+//    of 1,024, 2,048 and 4,096 rows 64 queries of up to 24 M rows take 1,150,
+//    1,060 and 1,080 us, the 24 queries 147, 148 and 195, the 32 676, 695 and
+//    785, 12 star joins of 6 to 11 M rows 500, 410 and 397.
 //  - A batch of large queries (kInOrderRows each on average) is drawn whole
 //    from the pool, query by query, each query's last rows in small tickets:
 //    the CTAs' meetings at its few switches cost little and no estimate of a
