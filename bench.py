@@ -121,8 +121,8 @@ def stored_traffic(workload, fact_rows, alg_bytes=None):
 
 def stored_link_bytes(workload, fact_rows):
     """Bytes the host-resident variant's fused kernel received over the host
-    link per launch (ncu ctc__rx_bytes_data_user.sum from the committed
-    summary of that capture, scaled by rows), or None when absent or taken
+    link per launch (ncu syslts__d_sectors_fill_sysmem.sum x 32 bytes, from the
+    committed summary of that capture, scaled by rows), or None when absent or taken
     on other kernel sources."""
     path = os.path.join(ROOT, "profiles", f"fused_kernel_{workload}_host.txt")
     try:
@@ -714,11 +714,6 @@ def main():
             e["page_bytes_gbs"] = rate
             e["page_bytes_frac_of_host_link"] = rate / links["host_read_gbs"]
             link, src = stored_link_bytes(args.workload, fact_rows)
-            if link is None:
-                t, tsrc = stored_traffic(args.workload, fact_rows)
-                if t is not None:
-                    link, src = t, ("estimate: the DRAM bytes of the HBM-resident kernel's capture of this query "
-                                    f"({tsrc}); the host-resident kernel reads the same sectors over the link")
             if link is not None:
                 # the kernel reads only the sectors holding a survivor's field of
                 # the later steps' columns: the bytes that crossed the link
