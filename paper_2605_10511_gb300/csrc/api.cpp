@@ -114,7 +114,7 @@ struct Prep {
   uint8_t* results = nullptr;
   uint8_t* outputs = nullptr;            // counts and records: results, or a device block
   std::vector<uint64_t> off_n, off_rec;  // byte offsets of the queries' counts and records
-  uint8_t* up = nullptr;          // pinned copy of what dq holds, while its upload may still read it
+  uint8_t* up = nullptr;          // one-shot: pinned copy of what dq holds, which its upload reads
   FusedLaunch L{};
   dpf_tuning tuning{};
   cudaEvent_t ev = nullptr;
@@ -1522,7 +1522,7 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
       (st = dev_alloc(c, up_bytes, reinterpret_cast<void**>(&p->dq))) ||
       (st = pin_alloc(c, results <= kPinResults ? results : 64, reinterpret_cast<void**>(&p->results))) ||
       (results > kPinResults && (st = dev_alloc(c, results, reinterpret_cast<void**>(&p->outputs)))) ||
-      (st = pin_alloc(c, up_bytes, reinterpret_cast<void**>(&p->up)))) {
+      (on && (st = pin_alloc(c, up_bytes, reinterpret_cast<void**>(&p->up))))) {
     const std::string msg = t_last_error;
     release_prep(c, p.get());
     return fail(st, "%s", msg.c_str());
@@ -1538,21 +1538,21 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
     Q.out_n = reinterpret_cast<unsigned int*>(p->outputs + p->off_n[size_t(i)]);
     Q.out = p->outputs + p->off_rec[size_t(i)];
   }
-  // uploaded from pinned memory: a pageable source of more than 64 KB (26 plans)
-  // may make the call wait for the stream's earlier work
-  std::memcpy(p->up, p->hq.data(), at_begin);
-  std::memcpy(p->up + at_begin, qbegin.data(), 8 * qbegin.size());
+  // on a caller's stream uploaded from pinned memory: a pageable source of more
+  // than 64 KB (26 plans) may make the call wait for the stream's earlier work
+  std::vector<uint8_t> pageable(on ? 0 : up_bytes);
+  uint8_t* up = on ? p->up : pageable.data();
+  std::memcpy(up, p->hq.data(), at_begin);
+  std::memcpy(up + at_begin, qbegin.data(), 8 * qbegin.size());
   const uint64_t filled = at_begin + 8 * qbegin.size();
-  std::memset(p->up + filled, 0, up_bytes - filled);
+  std::memset(up + filled, 0, up_bytes - filled);
   const cudaStream_t us = on ? *on : c->io;
   cudaError_t e = cudaMemsetAsync(p->scratch, 0, scratch, us);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(p->dq, p->up, up_bytes, cudaMemcpyHostToDevice, us);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(p->dq, up, up_bytes, cudaMemcpyHostToDevice, us);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev, cudaEventDisableTiming);
   if (e != cudaSuccess || !on) {
     const cudaError_t e2 = cudaStreamSynchronize(us);  // nothing may still write blocks that are freed
     if (e == cudaSuccess) e = e2;
-    pin_free(c, p->up);  // uploaded
-    p->up = nullptr;
   }
   if (e != cudaSuccess) {
     release_prep(c, p.get());
