@@ -545,8 +545,7 @@ dpf_status dpf_fetch_result(dpf_ctx* ctx, dpf_query_id id, dpf_record* buf, uint
  * stay resident in the context; queries are submitted as plans over them.
  * A dispatcher thread owned by the server keeps up to max_inflight batches
  * on the device, each on its own stream, and launches the queued queries
- * (FIFO, up to max_batch per launch) as soon as a slot is free (beside a
- * running batch, fewer than max_batch wait up to 40 us for more) and their
+ * (FIFO, up to max_batch per launch) as soon as a slot is free and their
  * device footprint (dpf_plan_footprint) fits mem_budget next to the
  * queries already running: continuous batching.  A query's records do not
  * depend on the batch it ran in. */

@@ -140,13 +140,6 @@ void dpf_server::finish_slot(Slot& s) {
   done_cv.notify_all();
 }
 
-// Longest wait of a short queue beside a running batch: arrivals a few tens of
-// microseconds apart then share a launch, where launches of one query each take
-// the SMs from one another.  16 variants of a star join of 268 M rows, two batches
-// in flight: p99 at 500 queries a second 4.2 ms, without the wait 5.4 to 5.7; at
-// 1,000 p50 / p90 / p99 1.75 / 6.3 / 18.9 to 20.1 ms, without 1.64 / 6.0 / 18.9.
-static constexpr double kGatherUs = 40.0;
-
 void dpf_server::run() {
   std::unique_lock<std::mutex> lk(mu);
   for (;;) {
@@ -163,11 +156,9 @@ void dpf_server::run() {
       finish_slot(s);  // also reports a failed launch through dpf_read_result
       lk.lock();
     }
-    // launches: FIFO, while a slot is free and the head of the queue fits;
-    // beside a running batch, a short queue waits up to kGatherUs for company
+    // launches: FIFO, while a slot is free and the head of the queue fits
     for (Slot& s : slots) {
       if (s.busy || pending.empty()) continue;
-      if (any_busy && pending.size() < cfg.max_batch && !stop && now_us() - pending.front()->submit_us < kGatherUs) break;
       std::vector<std::shared_ptr<Request>> batch;
       uint64_t bytes = 0;
       while (!pending.empty() && batch.size() < cfg.max_batch) {
