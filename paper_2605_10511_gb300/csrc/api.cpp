@@ -1487,11 +1487,11 @@ dpf_status prepare(dpf_ctx* c, const dpf_plan* plans, int32_t n, const dpf_tunin
                 t.threads);
   // One large query over device-resident integers runs best as one CTA of
   // 1,024 threads per SM (64 registers, 32 warps; one copy of its tables and
-  // accumulators to fill and flush): star join of 67 M rows 229 -> 205 us,
-  // chain of 17 M 102 -> 90, group-by of 10 M 88 -> 85.  Below kWideRows the
-  // 3 x 256 build (80 registers) wins, 32 against 35 us for a star of 5 M
-  // rows, as it does for a raw prefix at any size (207 against 211 us), and in
-  // a batch, whose CTAs change queries (223 against 345 us).
+  // accumulators to fill and flush): star join of 67 M rows 226 -> 178 us,
+  // chain of 17 M 97 -> 80.  Below kWideRows the 3 x 256 build (80 registers)
+  // wins, 32 against 35 us for a star of 5 M rows, as it does in a batch of
+  // small queries (24 of up to 4 M rows 149 against 174 us; of 64 up to 24 M the
+  // wide one takes 853 against 1,058); a raw prefix takes the same in both.
   if (open_threads && n == 1 && !host && !text && !stage_bw && t.ht_placement == DPF_HT_AUTO &&
       p->hq[0].nrows >= kWideRows && (p->hq[0].nsteps == 0 || p->hq[0].steps[0].kind != ST_PREFIX) &&
       fused_blocks_per_sm(1024, acc_slots, max_tables, host, kFusedMinBlocksLo, stage_bw, text) >= 1)
